@@ -241,7 +241,9 @@ __global__ void k_coarse_apply(int B, const double* __restrict__ Ainv, const T* 
 // ---------------------------------------------------------------------------------
 
 // One colour of a red-black sweep: threads enumerate only the nodes of that colour.
-template <typename T>
+// ZERO: the iterate is zero (first red pass of a correction from a zero guess): the sweep's
+// result without its six products, u = g / D, and no read of u.
+template <typename T, bool ZERO = false>
 __global__ void k_rbgs(int colour, int n, int B, const T* __restrict__ Kx, const T* __restrict__ Ky,
                        const T* __restrict__ Kz, const T* __restrict__ Dinv, const T* __restrict__ g, T* __restrict__ u,
                        const int* __restrict__ active) {
@@ -258,13 +260,45 @@ __global__ void k_rbgs(int colour, int n, int B, const T* __restrict__ Kx, const
     if (x > n - 2) continue;
     const size_t p = (size_t)s * n3 + (size_t)(z * n * n + y * n + x);
     T acc = g[p];
-    acc = fma(Kx[p - 1], u[p - 1], acc);
-    acc = fma(Kx[p], u[p + 1], acc);
-    acc = fma(Ky[p - n], u[p - n], acc);
-    acc = fma(Ky[p], u[p + n], acc);
-    acc = fma(Kz[p - n2], u[p - n2], acc);
-    acc = fma(Kz[p], u[p + n2], acc);
+    if (!ZERO) {
+      acc = fma(Kx[p - 1], u[p - 1], acc);
+      acc = fma(Kx[p], u[p + 1], acc);
+      acc = fma(Ky[p - n], u[p - n], acc);
+      acc = fma(Ky[p], u[p + n], acc);
+      acc = fma(Kz[p - n2], u[p - n2], acc);
+      acc = fma(Kz[p], u[p + n2], acc);
+    }
     u[p] = acc * Dinv[p];
+  }
+}
+
+// r~ = g - D u + sum K u_q (k_residual_z's operations and order) at the interior red nodes
+// only: after a sweep, whose last colour is black, the black residuals are zero up to
+// rounding, and the restrictions below take them as zero (HALF). Half the FP64 work of the
+// full residual, which stays for cycles without pre-smoothing.
+template <typename T>
+__global__ void k_residual_red(int n, int B, const T* __restrict__ Kx, const T* __restrict__ Ky,
+                               const T* __restrict__ Kz, const T* __restrict__ D, const T* __restrict__ g,
+                               const T* __restrict__ u, T* __restrict__ r, const int* __restrict__ active) {
+  const int m = n - 2, half = (n - 1) / 2, lh = 31 - __clz(half);
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // red node of an interior plane
+  if (q >= m * half) return;
+  const int xi = q & (half - 1), y = 1 + (q >> lh);
+  const size_t n3 = (size_t)n * n * n, n2 = (size_t)n * n;
+  for (int zz = blockIdx.y; zz < B * m; zz += gridDim.y) {
+    const int s = zz / m, z = 1 + (zz - s * m);
+    if (active && !active[s]) continue;
+    const int x = (((1 + y + z) & 1) == 0 ? 1 : 2) + 2 * xi;
+    if (x > n - 2) continue;
+    const size_t p = (size_t)s * n3 + (size_t)(z * n * n + y * n + x);
+    T rr = fma(-D[p], u[p], g[p]);
+    rr = fma(Kx[p - 1], u[p - 1], rr);
+    rr = fma(Kx[p], u[p + 1], rr);
+    rr = fma(Ky[p - n], u[p - n], rr);
+    rr = fma(Ky[p], u[p + n], rr);
+    rr = fma(Kz[p - n2], u[p - n2], rr);
+    rr = fma(Kz[p], u[p + n2], rr);
+    r[p] = rr;
   }
 }
 
@@ -297,6 +331,7 @@ __device__ __forceinline__ float nodal_face(float ra, float rb) { return __fdivi
 // few ulps of the stored FP32 one: used only inside the FP32 correction cycle, whose
 // result the FP64 outer residual (stored faces) corrects, so the converged solution is
 // that of the stored operator.
+template <bool ZERO = false>
 __global__ void k_rbgs_nodal(int colour, int n, int B, const float* __restrict__ kn, const float* __restrict__ g,
                              float* __restrict__ u, const int* __restrict__ active) {
   const int m = n - 2, half = (n - 1) / 2, lh = 31 - __clz(half);
@@ -322,12 +357,14 @@ __global__ void k_rbgs_nodal(int colour, int n, int B, const float* __restrict__
     d += kzp;
     const float dinv = __fdividef(1.0f, d);
     float acc = g[p];
-    acc = fmaf(kxm, u[p - 1], acc);
-    acc = fmaf(kxp, u[p + 1], acc);
-    acc = fmaf(kym, u[p - n], acc);
-    acc = fmaf(kyp, u[p + n], acc);
-    acc = fmaf(kzm, u[p - n2], acc);
-    acc = fmaf(kzp, u[p + n2], acc);
+    if (!ZERO) {
+      acc = fmaf(kxm, u[p - 1], acc);
+      acc = fmaf(kxp, u[p + 1], acc);
+      acc = fmaf(kym, u[p - n], acc);
+      acc = fmaf(kyp, u[p + n], acc);
+      acc = fmaf(kzm, u[p - n2], acc);
+      acc = fmaf(kzp, u[p + n2], acc);
+    }
     u[p] = acc * dinv;
   }
 }
@@ -336,16 +373,21 @@ __global__ void k_rbgs_nodal(int colour, int n, int B, const float* __restrict__
 // recomputed as in k_rbgs_nodal, then k_residual_z's operation order): the residual of the
 // operator the nodal sweep smooths; r~ on interior nodes, 0 on the boundary; 4 words per
 // node instead of 7.
+// RED: the red nodes only (k_residual_red's reason), the threads enumerating rows of red nodes.
+template <bool RED = false>
 __global__ void k_residual_nodal(int n, int B, const float* __restrict__ kn, const float* __restrict__ g,
                                  const float* __restrict__ u, float* __restrict__ r, const int* __restrict__ active) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // node of the plane
-  if (q >= n * n) return;
-  const int y = q / n, x = q - y * n;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // node (RED: red node) of the plane
+  const int half = (n + 1) / 2;
+  if (q >= (RED ? n * half : n * n)) return;
+  const int y = q / (RED ? half : n), xq = q - y * (RED ? half : n);
   const size_t n3 = (size_t)n * n * n, n2 = (size_t)n * n;
   for (int zz = blockIdx.y; zz < B * n; zz += gridDim.y) {
     const int s = zz / n, z = zz - s * n;
     if (active && !active[s]) continue;
-    const size_t p = (size_t)s * n3 + (size_t)(z * n * n + q);
+    const int x = RED ? 2 * xq + ((y + z) & 1) : xq;
+    if (RED && x > n - 1) continue;
+    const size_t p = (size_t)s * n3 + (size_t)(z * n * n + y * n + x);
     float rr = 0.0f;
     if (x > 0 && y > 0 && z > 0 && x < n - 1 && y < n - 1 && z < n - 1) {
       const float kc = kn[p];
@@ -412,6 +454,8 @@ __device__ __forceinline__ float comp(const float4& v, int i) { return i == 0 ? 
 
 // The nodal-coefficient update of one node from its own k^-1 and right-hand side and the
 // six neighbours' k^-1 and iterate, in k_rbgs_nodal's order of operations.
+// ZERO: the iterate is zero (g / D alone).
+template <bool ZERO = false>
 __device__ __forceinline__ float nodal_update(float kc, float gp, float kl, float ul, float kr, float ur, float kym,
                                               float uym, float kyp, float uyp, float kzm, float uzm, float kzp,
                                               float uzp) {
@@ -426,12 +470,14 @@ __device__ __forceinline__ float nodal_update(float kc, float gp, float kl, floa
   d += fzp;
   const float dinv = __fdividef(1.0f, d);
   float acc = gp;
-  acc = fmaf(fxm, ul, acc);
-  acc = fmaf(fxp, ur, acc);
-  acc = fmaf(fym, uym, acc);
-  acc = fmaf(fyp, uyp, acc);
-  acc = fmaf(fzm, uzm, acc);
-  acc = fmaf(fzp, uzp, acc);
+  if (!ZERO) {
+    acc = fmaf(fxm, ul, acc);
+    acc = fmaf(fxp, ur, acc);
+    acc = fmaf(fym, uym, acc);
+    acc = fmaf(fyp, uyp, acc);
+    acc = fmaf(fzm, uzm, acc);
+    acc = fmaf(fzp, uzp, acc);
+  }
   return acc * dinv;
 }
 
@@ -464,8 +510,8 @@ __device__ __forceinline__ float nodal_residual(float kc, float gp, float up, fl
 // its own k^-1 and g, the other colour's k^-1 and u in the same slots of its row (x - 1
 // or x + 1 of the group's nodes) and of the rows y +- 1, z +- 1, plus one scalar slot
 // outside the group. Grid (groups of the interior rows of a plane, interior planes,
-// samples).
-template <int LG>
+// samples). ZERO: from a zero iterate (k_rbgs).
+template <int LG, bool ZERO = false>
 __global__ void __launch_bounds__(128) k_rbgs_split(int colour, const float* __restrict__ kn,
                                                     const float* __restrict__ g, float* __restrict__ u,
                                                     const int* __restrict__ active) {
@@ -484,16 +530,18 @@ __global__ void __launch_bounds__(128) k_rbgs_split(int colour, const float* __r
   const float4 kc4 = ld4(kn + cb + o), g4 = ld4(g + cb + o);
   const float4 km4 = ld4(ko + o), kym4 = ld4(ko + o - G::P), kyp4 = ld4(ko + o + G::P);
   const float4 kzm4 = ld4(ko + o - G::NP), kzp4 = ld4(ko + o + G::NP);
-  const float4 um4 = ld4(uo + o), uym4 = ld4(uo + o - G::P), uyp4 = ld4(uo + o + G::P);
-  const float4 uzm4 = ld4(uo + o - G::NP), uzp4 = ld4(uo + o + G::NP);
+  const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const float4 um4 = ZERO ? zero4 : ld4(uo + o), uym4 = ZERO ? zero4 : ld4(uo + o - G::P);
+  const float4 uyp4 = ZERO ? zero4 : ld4(uo + o + G::P);
+  const float4 uzm4 = ZERO ? zero4 : ld4(uo + o - G::NP), uzp4 = ZERO ? zero4 : ld4(uo + o + G::NP);
   // the other-colour slot beside the group: left of node 0 (x parity 0) or right of node 3
   float kext = 0.0f, uext = 0.0f;
   if (par) {
     kext = ko[o + 4];
-    uext = uo[o + 4];
+    if (!ZERO) uext = uo[o + 4];
   } else if (x0 > 0) {
     kext = ko[o - 1];
-    uext = uo[o - 1];
+    if (!ZERO) uext = uo[o - 1];
   }
   float out[4];
 #pragma unroll
@@ -502,7 +550,7 @@ __global__ void __launch_bounds__(128) k_rbgs_split(int colour, const float* __r
     const float ul = par ? comp(um4, i) : (i == 0 ? uext : comp(um4, i - 1));
     const float kr = par ? (i == 3 ? kext : comp(km4, i + 1)) : comp(km4, i);
     const float ur = par ? (i == 3 ? uext : comp(um4, i + 1)) : comp(um4, i);
-    out[i] = nodal_update(comp(kc4, i), comp(g4, i), kl, ul, kr, ur, comp(kym4, i), comp(uym4, i), comp(kyp4, i),
+    out[i] = nodal_update<ZERO>(comp(kc4, i), comp(g4, i), kl, ul, kr, ur, comp(kym4, i), comp(uym4, i), comp(kyp4, i),
                           comp(uyp4, i), comp(kzm4, i), comp(uzm4, i), comp(kzp4, i), comp(uzp4, i));
   }
   float* uc = u + cb + o;
@@ -520,17 +568,18 @@ __global__ void __launch_bounds__(128) k_rbgs_split(int colour, const float* __r
 // storage (the restriction reads only interior fine nodes; boundary and padding slots of
 // r are not written). Grid (groups of the interior rows of a plane, 2 x interior planes,
 // samples): colour = blockIdx.y & 1, so the two colours of a plane run back to back and
-// the 1/k and u rows each reads as the other colour's are still in L2.
-template <int LG>
+// the 1/k and u rows each reads as the other colour's are still in L2. RED: the red nodes
+// only (k_residual_red's reason; 3 words per two nodes), blockIdx.y the interior plane.
+template <int LG, bool RED = false>
 __global__ void __launch_bounds__(128, 8) k_residual_split(const float* __restrict__ kn, const float* __restrict__ g,
                                                         const float* __restrict__ u, float* __restrict__ r,
                                                         const int* __restrict__ active) {
   using G = SplitGeo<LG>;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= G::m * G::Q4) return;
-  const int s = blockIdx.z, colour = blockIdx.y & 1;
+  const int s = blockIdx.z, colour = RED ? 0 : blockIdx.y & 1;
   if (active && !active[s]) return;
-  const int yi = q / G::Q4, qi = q - yi * G::Q4, y = 1 + yi, z = 1 + (int)(blockIdx.y >> 1);
+  const int yi = q / G::Q4, qi = q - yi * G::Q4, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
   const int par = (colour + y + z) & 1, xi0 = 4 * qi, x0 = 2 * xi0 + par;
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
@@ -573,8 +622,9 @@ __global__ void __launch_bounds__(128, 8) k_residual_split(const float* __restri
 
 // g_c = 4 FW(r~) (k_restrict's weights and order) from r~ in colour-split storage into the
 // coarse grid's colour-split g, at interior coarse nodes. LG: the fine grid's. Grid
-// (interior coarse nodes of a plane, interior coarse planes, samples).
-template <int LG, typename T = float>
+// (interior coarse nodes of a plane, interior coarse planes, samples). HALF: r~ is zero at
+// black nodes (k_residual_red): the 13 red neighbours of the 27.
+template <int LG, typename T = float, bool HALF = false>
 __global__ void __launch_bounds__(128) k_restrict_split(const T* __restrict__ r, T* __restrict__ gc,
                                                         const int* __restrict__ active) {
   using F = SplitGeo<LG>;
@@ -593,6 +643,7 @@ __global__ void __launch_bounds__(128) k_restrict_split(const T* __restrict__ r,
     for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
       for (int dx = -1; dx <= 1; ++dx) {
+        if (HALF && ((dx + dy + dz) & 1)) continue;
         const T wgt = (T)((2 - abs(dx)) * (2 - abs(dy)) * (2 - abs(dz))) * (T)(1.0 / 16.0);
         const int fx = 2 * X + dx, fy = 2 * Y + dy, fz = 2 * Z + dz;  // colour (dx + dy + dz) & 1
         v = fma(wgt, rb[(size_t)((dx + dy + dz) & 1) * F::BLK + (size_t)((fz * F::n + fy) * F::P + (fx >> 1))], v);
@@ -607,15 +658,16 @@ __global__ void __launch_bounds__(128) k_restrict_split(const T* __restrict__ r,
 // coarse X = xi0 + i, one x parity, hence one weight pattern) with a 16-byte update of u;
 // each coarse row it needs is gathered once for the group (X = xi0 .. xi0 + 4). LG: the
 // fine grid's. Grid (groups of the interior rows of a plane, interior planes,
-// 2 x samples: colour = blockIdx.z & 1).
-template <int LG>
+// 2 x samples: colour = blockIdx.z & 1). BLACK: the black nodes only, blockIdx.z the sample:
+// a red pass follows, which overwrites the red nodes without reading them.
+template <int LG, bool BLACK = false>
 __global__ void __launch_bounds__(128) k_prolong_split(const float* __restrict__ ec, float* __restrict__ u,
                                                        const int* __restrict__ active) {
   using F = SplitGeo<LG>;
   using C = SplitGeo<LG - 1>;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= F::m * F::Q4) return;
-  const int s = blockIdx.z >> 1, colour = blockIdx.z & 1;
+  const int s = BLACK ? blockIdx.z : blockIdx.z >> 1, colour = BLACK ? 1 : blockIdx.z & 1;
   if (active && !active[s]) return;
   const int yi = q / F::Q4, qi = q - yi * F::Q4, y = 1 + yi, z = 1 + (int)blockIdx.y;
   const int xo = (colour + y + z) & 1, xi0 = 4 * qi, x0 = 2 * xi0 + xo;
@@ -746,8 +798,9 @@ __global__ void k_split_copy(int n, int B, const T* __restrict__ a, T* __restric
 // One colour of the stored-face sweep on colour-split FP64 storage (k_rbgs's operations
 // and order), two nodes per thread on 16-byte loads: its own Kx, Ky, Kz, 1/D and g, the
 // other colour's lower faces (x - 1, y - 1, z - 1 nodes) and u of the six neighbours.
-// Grid (two-slot groups of the interior rows of a plane, interior planes, samples).
-template <int LG>
+// Grid (two-slot groups of the interior rows of a plane, interior planes, samples). ZERO:
+// from a zero iterate (k_rbgs).
+template <int LG, bool ZERO = false>
 __global__ void __launch_bounds__(128) k_rbgs_split64(int colour, const double* __restrict__ Kx,
                                                       const double* __restrict__ Ky, const double* __restrict__ Kz,
                                                       const double* __restrict__ Dinv, const double* __restrict__ g,
@@ -763,8 +816,21 @@ __global__ void __launch_bounds__(128) k_rbgs_split64(int colour, const double* 
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
   const size_t cb = (size_t)s * G::NS + (size_t)colour * G::BLK, ob = (size_t)s * G::NS + (size_t)(1 - colour) * G::BLK;
-  const double2 kx2 = ld2(Kx + cb + o), ky2 = ld2(Ky + cb + o), kz2 = ld2(Kz + cb + o);
   const double2 di2 = ld2(Dinv + cb + o), g2 = ld2(g + cb + o);
+  double* uc = u + cb + o;
+  const bool inner = x0 >= 1 && x0 + 2 <= G::n - 2;
+  if (ZERO) {
+    const double out[2] = {g2.x * di2.x, g2.y * di2.y};
+    if (inner) {
+      *reinterpret_cast<double2*>(uc) = make_double2(out[0], out[1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (x0 + 2 * i >= 1 && x0 + 2 * i <= G::n - 2) uc[i] = out[i];
+    }
+    return;
+  }
+  const double2 kx2 = ld2(Kx + cb + o), ky2 = ld2(Ky + cb + o), kz2 = ld2(Kz + cb + o);
   const double* kxo = Kx + ob;
   const double* uo = u + ob;
   const double2 kxm2 = ld2(kxo + o), kym2 = ld2(Ky + ob + o - G::P), kzm2 = ld2(Kz + ob + o - G::NP);
@@ -794,8 +860,7 @@ __global__ void __launch_bounds__(128) k_rbgs_split64(int colour, const double* 
     acc = fma(comp2(kz2, i), comp2(uzp2, i), acc);
     out[i] = acc * comp2(di2, i);
   }
-  double* uc = u + cb + o;
-  if (x0 >= 1 && x0 + 2 <= G::n - 2) {
+  if (inner) {
     *reinterpret_cast<double2*>(uc) = make_double2(out[0], out[1]);
   } else {
 #pragma unroll
@@ -807,8 +872,9 @@ __global__ void __launch_bounds__(128) k_rbgs_split64(int colour, const double* 
 // r~ = g - D u + sum K u_q (k_residual_z's operations and order) at the interior nodes of
 // one colour, two per thread, into r in colour-split storage (interior nodes only).
 // Grid (two-slot groups of the interior rows of a plane, 2 x interior planes, samples):
-// colour = blockIdx.y & 1 (the two colours of a plane back to back).
-template <int LG>
+// colour = blockIdx.y & 1 (the two colours of a plane back to back). RED: the red nodes only
+// (k_residual_red's reason), blockIdx.y the interior plane.
+template <int LG, bool RED = false>
 __global__ void __launch_bounds__(128) k_residual_split64(const double* __restrict__ Kx, const double* __restrict__ Ky,
                                                           const double* __restrict__ Kz, const double* __restrict__ D,
                                                           const double* __restrict__ g, const double* __restrict__ u,
@@ -817,9 +883,9 @@ __global__ void __launch_bounds__(128) k_residual_split64(const double* __restri
   constexpr int Q2 = G::P / 2;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= G::m * Q2) return;
-  const int s = blockIdx.z, colour = blockIdx.y & 1;
+  const int s = blockIdx.z, colour = RED ? 0 : blockIdx.y & 1;
   if (active && !active[s]) return;
-  const int yi = q / Q2, qi = q - yi * Q2, y = 1 + yi, z = 1 + (int)(blockIdx.y >> 1);
+  const int yi = q / Q2, qi = q - yi * Q2, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
   const int par = (colour + y + z) & 1, xi0 = 2 * qi, x0 = 2 * xi0 + par;
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
@@ -991,6 +1057,37 @@ __global__ void k_restrict(int nf, int B, const T* __restrict__ r, T* __restrict
   }
 }
 
+// k_restrict of a residual that is zero at black nodes (k_residual_red): its 13 red terms of
+// the 27, in their order.
+template <typename T>
+__global__ void k_restrict_red(int nf, int B, const T* __restrict__ r, T* __restrict__ gc,
+                               const int* __restrict__ active) {
+  const int nc = (nf + 1) / 2, hc = nc - 1, lc = 31 - __clz(hc);
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // interior coarse node of a plane
+  if (q >= (nc - 2) * hc) return;
+  const int X = 1 + (q & (hc - 1)), Y = 1 + (q >> lc);
+  if (X > nc - 2) return;
+  const size_t nc3 = (size_t)nc * nc * nc, nf3 = (size_t)nf * nf * nf;
+  const int nf2 = nf * nf;
+  for (int zz = blockIdx.y; zz < B * (nc - 2); zz += gridDim.y) {
+    const int s = zz / (nc - 2), Z = 1 + (zz - s * (nc - 2));
+    if (active && !active[s]) continue;
+    const T* rb = r + (size_t)s * nf3 + (size_t)(2 * Z * nf2 + 2 * Y * nf + 2 * X);
+    T v = 0;
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+        for (int dx = -1; dx <= 1; ++dx) {
+          if ((dx + dy + dz) & 1) continue;
+          const T wgt = (T)((2 - abs(dx)) * (2 - abs(dy)) * (2 - abs(dz))) * (T)(1.0 / 16.0);
+          v = fma(wgt, rb[dz * nf2 + dy * nf + dx], v);
+        }
+    gc[(size_t)s * nc3 + (size_t)((Z * nc + Y) * nc + X)] = v;
+  }
+}
+
 // u_f += trilinear interpolation of e_c at interior fine nodes: a fine node with k odd
 // coordinates is the mean of its 2^k coarse neighbours (k = 0: the coincident coarse
 // node). Threads of a row take the odd x first and the even x after them, so that a warp
@@ -1061,8 +1158,10 @@ __device__ __forceinline__ void prolong_block_sums(const T (&c)[8], T (&v)[8]) {
 // (2X + dx, 2Y + dy, 2Z + dz) of the cell, their sums from prolong_block_sums, u += w v at
 // the interior ones. Every thread runs the same operations (no parity divergence) and the
 // block shares partial sums: 2.75 instead of 4.4 FP64 operations per fine node. Grid: coarse
-// cells of a plane, (sample, cell plane) planes.
-template <typename T>
+// cells of a plane, (sample, cell plane) planes. BLACK: the black nodes (dx + dy + dz odd)
+// only, 1.6 operations per fine node: a red pass follows, which overwrites the red nodes
+// without reading them (the compiler drops the sums no black node needs).
+template <typename T, bool BLACK = false>
 __global__ void __launch_bounds__(128) k_prolong_blk(int nf, int B, const T* __restrict__ ec, T* __restrict__ u,
                                                      const int* __restrict__ active) {
   const int nc = (nf + 1) / 2, mc = nc - 1;
@@ -1081,6 +1180,7 @@ __global__ void __launch_bounds__(128) k_prolong_blk(int nf, int B, const T* __r
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
+      if (BLACK && !((dx + dy + dz) & 1)) continue;
       const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
       if (x < 1 || y < 1 || z < 1 || x > nf - 2 || y > nf - 2 || z > nf - 2) continue;
       const T w = dx + dy + dz == 0 ? T(1) : dx + dy + dz == 1 ? T(0.5) : dx + dy + dz == 2 ? T(0.25) : T(0.125);
@@ -1092,7 +1192,8 @@ __global__ void __launch_bounds__(128) k_prolong_blk(int nf, int B, const T* __r
 // k_prolong_blk on colour-split storage of both grids (LG: the fine grid's). Fine node
 // (2X + dx, ...) is colour (dx + dy + dz) & 1, slot X; coarse (X', Y', Z') colour
 // (X' + Y' + Z') & 1, slot X' / 2. Grid (coarse cells of a plane, cell planes, samples).
-template <int LG, typename T>
+// BLACK: as in k_prolong_blk.
+template <int LG, typename T, bool BLACK = false>
 __global__ void __launch_bounds__(128) k_prolong_blk_split(const T* __restrict__ ec, T* __restrict__ u,
                                                            const int* __restrict__ active) {
   using F = SplitGeo<LG>;
@@ -1115,6 +1216,7 @@ __global__ void __launch_bounds__(128) k_prolong_blk_split(const T* __restrict__
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
+    if (BLACK && !((dx + dy + dz) & 1)) continue;
     const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
     if (x < 1 || y < 1 || z < 1 || x > F::n - 2 || y > F::n - 2 || z > F::n - 2) continue;
     const T w = dx + dy + dz == 0 ? T(1) : dx + dy + dz == 1 ? T(0.5) : dx + dy + dz == 2 ? T(0.25) : T(0.125);
@@ -1275,6 +1377,48 @@ __global__ void k_restrict_p1(int nf, int B, const T* __restrict__ r, T* __restr
     acc += R(0, -1, -1) + R(0, 1, 1);
     acc += R(-1, 0, -1) + R(1, 0, 1);
     acc += R(-1, -1, -1) + R(1, 1, 1);
+    gc[node_at<SPLIT>(nc, s, X, Y, Z)] = T(0.5) * R(0, 0, 0) + T(0.25) * acc;
+  }
+}
+
+// k_prolong_p1 at the black fine nodes only (a red pass follows, which overwrites the red
+// nodes without reading them); a black node has an odd number of odd coordinates, so it is
+// always the midpoint of a coarse edge. Threads enumerate rows of black nodes.
+template <typename T, bool SPLIT>
+__global__ void k_prolong_p1_black(int nf, int B, const T* __restrict__ ec, T* __restrict__ u,
+                                   const int* __restrict__ active) {
+  const int m = nf - 2, nc = (nf + 1) / 2, half = nc - 1;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= m * half) return;
+  const int y = 1 + q / half, xi = q - (y - 1) * half;
+  for (int zz = blockIdx.y; zz < B * m; zz += gridDim.y) {
+    const int s = zz / m, z = 1 + zz - s * m;
+    if (active && !active[s]) continue;
+    const int x = 1 + 2 * xi + ((y + z) & 1);
+    if (x > nf - 2) continue;
+    const int dx = x & 1, dy = y & 1, dz = z & 1;
+    const int X0 = (x - dx) >> 1, Y0 = (y - dy) >> 1, Z0 = (z - dz) >> 1;
+    u[node_at<SPLIT>(nf, s, x, y, z)] +=
+        T(0.5) * (ec[node_at<SPLIT>(nc, s, X0, Y0, Z0)] + ec[node_at<SPLIT>(nc, s, X0 + dx, Y0 + dy, Z0 + dz)]);
+  }
+}
+
+// k_restrict_p1 of a residual that is zero at black nodes (k_residual_red): the six diagonal
+// directions of the faces and the node itself.
+template <typename T, bool SPLIT>
+__global__ void k_restrict_p1_red(int nf, int B, const T* __restrict__ r, T* __restrict__ gc,
+                                  const int* __restrict__ active) {
+  const int nc = (nf + 1) / 2, mc = nc - 2;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // interior coarse node of the plane
+  if (q >= mc * mc) return;
+  const int Y = 1 + q / mc, X = 1 + q - (Y - 1) * mc;
+  for (int zz = blockIdx.y; zz < B * mc; zz += gridDim.y) {
+    const int s = zz / mc, Z = 1 + zz - s * mc;
+    if (active && !active[s]) continue;
+    auto R = [&](int dx, int dy, int dz) { return r[node_at<SPLIT>(nf, s, 2 * X + dx, 2 * Y + dy, 2 * Z + dz)]; };
+    T acc = R(-1, -1, 0) + R(1, 1, 0);
+    acc += R(0, -1, -1) + R(0, 1, 1);
+    acc += R(-1, 0, -1) + R(1, 0, 1);
     gc[node_at<SPLIT>(nc, s, X, Y, Z)] = T(0.5) * R(0, 0, 0) + T(0.25) * acc;
   }
 }
@@ -1762,14 +1906,39 @@ struct Names<float> {
 
 inline double interior(int n) { return (double)(n - 2) * (n - 2) * (n - 2); }
 
+// Red-black sweeps start on red and end on black, and a colour pass reads the other colour
+// only. The V-cycle uses that three times: from a zero guess the first red pass is g / D
+// (zero_pass: no product, and no clearing of u, whose boundary is zeroed once per solve);
+// after a pre-smoothing sweep the black residuals are zero up to rounding, so the residual
+// and the restriction take the red nodes alone; before a post-smoothing sweep the correction
+// is interpolated to the black nodes alone (the red pass overwrites the red ones unread). An
+// FP64 V(2,2) cycle on stored faces spends 28 + 3.5 + 1.7 + 1.6 FP64 operations per node on
+// the finest grid instead of 28 + 7 + 3.4 + 2.75.
+// Measured: FP64 solves of 65^3 x 19 10.42 -> 9.37 ms, the 129^3 / 65^3 level of 24 samples
+// 83.5 -> 75.6 ms, the 17^3 level of 4096 samples (small-grid engine) 35.1 -> 32.7 ms, mixed
+// refinement of 33^3 x 48 5.38 -> 4.81 ms, the mixed 257^3 / 129^3 level 43.9 -> 41.5 ms.
 template <typename T>
-void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st);
+inline bool zero_pass(const Hier<T>& H, int j, int nu1) {
+  return j == H.L - 1 || (nu1 > 0 && !H.fused[j]);
+}
+
+// Cycle from a zero guess on grid j: clears u where the cycle's first pass reads it.
+template <typename T>
+cudaError_t clear_guess(const Hier<T>& H, int j, int nu1, cudaStream_t st) {
+  if (zero_pass(H, j, nu1)) return cudaSuccess;
+  const Level<T>& v = H.lv[j];
+  return cudaMemsetAsync(v.u, 0, (size_t)H.B * (H.split ? split_elems(v.n) : v.n3) * sizeof(T), st);
+}
+
+// zero: u is zero on entry (cleared by clear_guess, where that is needed).
+template <typename T>
+void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero);
 
 // One level of the V-cycle on colour-split FP32 storage: nodal-coefficient colour passes,
 // the residual into the plain r, full weighting into the coarse grid's split g, the
 // coarser levels, the trilinear correction on split storage, post-smoothing.
 template <typename T>
-void vcycle_split(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
+void vcycle_split(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
   Level<T>& v = H.lv[j];
   Level<T>& w = H.lv[j + 1];
   const int* act = H.active;
@@ -1779,36 +1948,104 @@ void vcycle_split(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
   const float* g = (const float*)(const void*)v.g;
   const float* kn = (const float*)(const void*)v.kn;
   const dim3 gs((unsigned)((m * (split_pitch(v.n) / 4) + 127) / 128), (unsigned)m, (unsigned)B);
-  auto smooth = [&](int sweeps) {
+  auto smooth = [&](int sweeps, bool from_zero) {
     for (int s = 0; s < sweeps; ++s)
-      for (int c = 0; c < 2; ++c)
-        MLMC_LAUNCH(prof::sized("rbgs_split_f32", v.n), Ba * interior(v.n) * 2.0 * W, Ba * interior(v.n) * 0.5 * 37.0,
-                    st, MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split<LG><<<gs, 128, 0, st>>>(c, kn, g, u, act))));
+      for (int c = 0; c < 2; ++c) {
+        if (from_zero && s == 0 && c == 0)
+          MLMC_LAUNCH(prof::sized("rbgs_split_f32", v.n), Ba * interior(v.n) * 1.5 * W, Ba * interior(v.n) * 0.5 * 25.0,
+                      st, MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split<LG, true><<<gs, 128, 0, st>>>(c, kn, g, u, act))));
+        else
+          MLMC_LAUNCH(prof::sized("rbgs_split_f32", v.n), Ba * interior(v.n) * 2.0 * W, Ba * interior(v.n) * 0.5 * 37.0,
+                      st, MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split<LG><<<gs, 128, 0, st>>>(c, kn, g, u, act))));
+      }
   };
-  smooth(nu1);
+  smooth(nu1, zero);
   const unsigned groups = (unsigned)((m * (split_pitch(v.n) / 4) + 127) / 128);
   float* r = (float*)(void*)v.r;  // colour-split r~ (room for n^2 (n+1) elements: carved as n^3 + slack)
-  MLMC_LAUNCH(prof::sized("residual_split_f32", v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 37.0, st,
-              MLMC_SPLIT_DISPATCH(v.n, (k_residual_split<LG><<<dim3(groups, (unsigned)(2 * m), (unsigned)B), 128, 0,
-                                                                st>>>(kn, g, u, r, act))));
-  MLMC_LAUNCH(Names<T>::restrict_, Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 54.0, st,
-              MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG><<<dim3((unsigned)(((w.n - 2) * (w.n - 2) + 127) / 128),
-                                                                    (unsigned)(w.n - 2), (unsigned)B), 128, 0, st>>>(
-                                                r, (float*)(void*)w.g, act))));
-  cudaMemsetAsync(w.u, 0, (size_t)B * split_elems(w.n) * sizeof(T), st);
-  vcycle(H, j + 1, nu1, nu2, st);
-  MLMC_LAUNCH(prof::sized("prolong_split_f32", v.n), Ba * (2.0 * (double)v.n3 + (double)w.n3) * W,
-              Ba * interior(v.n) * 4.375, st,
-              MLMC_SPLIT_DISPATCH(v.n, (k_prolong_split<LG><<<dim3(groups, (unsigned)m, (unsigned)(2 * B)), 128, 0,
-                                                               st>>>((const float*)(const void*)w.u, u, act))));
-  smooth(nu2);
+  const dim3 rg((unsigned)(((w.n - 2) * (w.n - 2) + 127) / 128), (unsigned)(w.n - 2), (unsigned)B);
+  if (nu1 > 0) {
+    MLMC_LAUNCH(prof::sized("residual_split_f32", v.n), Ba * interior(v.n) * 3.0 * W, Ba * interior(v.n) * 18.5, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_residual_split<LG, true><<<dim3(groups, (unsigned)m, (unsigned)B), 128, 0,
+                                                                        st>>>(kn, g, u, r, act))));
+    MLMC_LAUNCH(Names<T>::restrict_, Ba * (0.5 * (double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 26.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG, float, true><<<rg, 128, 0, st>>>(
+                                             r, (float*)(void*)w.g, act))));
+  } else {
+    MLMC_LAUNCH(prof::sized("residual_split_f32", v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 37.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_residual_split<LG><<<dim3(groups, (unsigned)(2 * m), (unsigned)B), 128, 0,
+                                                                  st>>>(kn, g, u, r, act))));
+    MLMC_LAUNCH(Names<T>::restrict_, Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 54.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG><<<rg, 128, 0, st>>>(r, (float*)(void*)w.g, act))));
+  }
+  clear_guess(H, j + 1, nu1, st);
+  vcycle(H, j + 1, nu1, nu2, st, true);
+  if (nu2 > 0)
+    MLMC_LAUNCH(prof::sized("prolong_split_f32", v.n), Ba * ((double)v.n3 + (double)w.n3) * W,
+                Ba * interior(v.n) * 2.2, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_prolong_split<LG, true><<<dim3(groups, (unsigned)m, (unsigned)B), 128, 0,
+                                                                       st>>>((const float*)(const void*)w.u, u,
+                                                                             act))));
+  else
+    MLMC_LAUNCH(prof::sized("prolong_split_f32", v.n), Ba * (2.0 * (double)v.n3 + (double)w.n3) * W,
+                Ba * interior(v.n) * 4.375, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_prolong_split<LG><<<dim3(groups, (unsigned)m, (unsigned)(2 * B)), 128, 0,
+                                                                 st>>>((const float*)(const void*)w.u, u, act))));
+  smooth(nu2, false);
+}
+
+// u_j += the interpolation of grid j + 1's u (P1 or trilinear; plain or, for FP64, split
+// storage). black: at the black nodes only (a red pass follows).
+template <typename T>
+void prolong_level(Hier<T>& H, int j, bool black, cudaStream_t st) {
+  const Level<T>& v = H.lv[j];
+  const Level<T>& w = H.lv[j + 1];
+  const int* act = H.active;
+  const int B = H.B, m = v.n - 2, mc = w.n - 1;
+  const double Ba = (double)H.n_act, W = (double)sizeof(T);
+  const double bytes = Ba * ((black ? 1.0 : 2.0) * (double)v.n3 + (double)w.n3) * W;
+  if (H.p1) {
+    const dim3 all = plane_grid(m * m, (long long)B * m), blk = plane_grid(m * mc, (long long)B * m);
+    const double flops = Ba * interior(v.n) * (black ? 0.75 : 1.5);
+    if (H.split && black)
+      MLMC_LAUNCH("prolong_p1", bytes, flops, st,
+                  (k_prolong_p1_black<T, true><<<blk, kPlaneThreads, 0, st>>>(v.n, B, w.u, v.u, act)));
+    else if (H.split)
+      MLMC_LAUNCH("prolong_p1", bytes, flops, st,
+                  (k_prolong_p1<T, true><<<all, kPlaneThreads, 0, st>>>(v.n, B, w.u, v.u, act)));
+    else if (black)
+      MLMC_LAUNCH("prolong_p1", bytes, flops, st,
+                  (k_prolong_p1_black<T, false><<<blk, kPlaneThreads, 0, st>>>(v.n, B, w.u, v.u, act)));
+    else
+      MLMC_LAUNCH("prolong_p1", bytes, flops, st,
+                  (k_prolong_p1<T><<<all, kPlaneThreads, 0, st>>>(v.n, B, w.u, v.u, act)));
+    return;
+  }
+  const double flops = Ba * interior(v.n) * (black ? 1.6 : 2.75);
+  if (H.split) {
+    if constexpr (sizeof(T) == 8) {
+      const dim3 g((unsigned)((mc * mc + 127) / 128), (unsigned)mc, (unsigned)B);
+      if (black)
+        MLMC_LAUNCH(prof::sized("prolong_split_f64", v.n), bytes, flops, st,
+                    MLMC_SPLIT_DISPATCH(v.n, (k_prolong_blk_split<LG, T, true><<<g, 128, 0, st>>>(w.u, v.u, act))));
+      else
+        MLMC_LAUNCH(prof::sized("prolong_split_f64", v.n), bytes, flops, st,
+                    MLMC_SPLIT_DISPATCH(v.n, (k_prolong_blk_split<LG, T><<<g, 128, 0, st>>>(w.u, v.u, act))));
+    }
+    return;
+  }
+  const dim3 g = plane_grid(mc * mc, (long long)B * mc);
+  if (black)
+    MLMC_LAUNCH(Names<T>::prolong, bytes, flops, st,
+                (k_prolong_blk<T, true><<<g, 128, 0, st>>>(v.n, B, w.u, v.u, act)));
+  else
+    MLMC_LAUNCH(Names<T>::prolong, bytes, flops, st, (k_prolong_blk<T><<<g, 128, 0, st>>>(v.n, B, w.u, v.u, act)));
 }
 
 // One level of the V-cycle on colour-split FP64 storage (stored faces): two-pass colour
 // sweeps, the residual into split r, full weighting into the coarse split g, the coarser
 // levels, the trilinear correction on split storage, post-smoothing.
 template <typename T>
-void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
+void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
   Level<T>& v = H.lv[j];
   Level<T>& w = H.lv[j + 1];
   const int* act = H.active;
@@ -1823,49 +2060,54 @@ void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
   double* u = (double*)(void*)v.u;
   double* r = (double*)(void*)v.r;
   const unsigned pairs = (unsigned)((m * (split_pitch(v.n) / 2) + 127) / 128);
-  auto smooth = [&](int sweeps) {
+  const dim3 gs(pairs, (unsigned)m, (unsigned)B);
+  auto smooth = [&](int sweeps, bool from_zero) {
     for (int s = 0; s < sweeps; ++s)
-      for (int c = 0; c < 2; ++c)
-        MLMC_LAUNCH(prof::sized("rbgs_split_f64", v.n), Ba * interior(v.n) * 3.5 * W, Ba * interior(v.n) * 0.5 * 13.0,
-                    st, MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split64<LG><<<dim3(pairs, (unsigned)m, (unsigned)B), 128, 0,
-                                                                         st>>>(c, Kx, Ky, Kz, Dinv, g, u, act))));
+      for (int c = 0; c < 2; ++c) {
+        if (from_zero && s == 0 && c == 0)
+          MLMC_LAUNCH(prof::sized("rbgs_split_f64", v.n), Ba * interior(v.n) * 1.5 * W, Ba * interior(v.n) * 0.5, st,
+                      MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split64<LG, true><<<gs, 128, 0, st>>>(c, Kx, Ky, Kz, Dinv, g, u,
+                                                                                           act))));
+        else
+          MLMC_LAUNCH(prof::sized("rbgs_split_f64", v.n), Ba * interior(v.n) * 3.5 * W, Ba * interior(v.n) * 0.5 * 13.0,
+                      st, MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split64<LG><<<gs, 128, 0, st>>>(c, Kx, Ky, Kz, Dinv, g, u,
+                                                                                         act))));
+      }
   };
-  smooth(nu1);
-  MLMC_LAUNCH(prof::sized("residual_split_f64", v.n), Ba * interior(v.n) * 7.0 * W, Ba * interior(v.n) * 14.0, st,
-              MLMC_SPLIT_DISPATCH(v.n, (k_residual_split64<LG><<<dim3(pairs, (unsigned)(2 * m), (unsigned)B), 128, 0,
-                                                                  st>>>(Kx, Ky, Kz, D, g, u, r, act))));
-  if (H.p1)
-    MLMC_LAUNCH("restrict_p1", Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 16.0, st,
-                (k_restrict_p1<double, true><<<plane_grid((w.n - 2) * (w.n - 2), (long long)B * (w.n - 2)),
-                                               kPlaneThreads, 0, st>>>(v.n, B, r, (double*)(void*)w.g, act)));
+  smooth(nu1, zero);
+  const bool red = nu1 > 0, black = nu2 > 0;
+  double* gc = (double*)(void*)w.g;
+  if (red)
+    MLMC_LAUNCH(prof::sized("residual_split_f64", v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 7.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_residual_split64<LG, true><<<gs, 128, 0, st>>>(Kx, Ky, Kz, D, g, u, r,
+                                                                                         act))));
   else
-    MLMC_LAUNCH(Names<T>::restrict_, Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 54.0, st,
-                MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG, double><<<dim3((unsigned)(((w.n - 2) * (w.n - 2) +
-                                                                                       127) / 128),
-                                                                              (unsigned)(w.n - 2), (unsigned)B),
-                                                                         128, 0, st>>>(r, (double*)(void*)w.g,
-                                                                                       act))));
-  cudaMemsetAsync(w.u, 0, (size_t)B * split_elems(w.n) * sizeof(T), st);
-  vcycle(H, j + 1, nu1, nu2, st);
-  if (H.p1) {
-    MLMC_LAUNCH("prolong_p1", Ba * (2.0 * (double)v.n3 + (double)w.n3) * W, Ba * interior(v.n) * 1.5, st,
-                (k_prolong_p1<double, true><<<plane_grid(m * m, (long long)B * m), kPlaneThreads, 0, st>>>(
-                    v.n, B, (const double*)(const void*)w.u, u, act)));
-    smooth(nu2);
-    return;
-  }
-  MLMC_LAUNCH(prof::sized("prolong_split_f64", v.n), Ba * (2.0 * (double)v.n3 + (double)w.n3) * W,
-              Ba * interior(v.n) * 4.375, st,
-              MLMC_SPLIT_DISPATCH(v.n, (k_prolong_blk_split<LG, double><<<dim3((unsigned)(((w.n - 1) * (w.n - 1) +
-                                                                                          127) / 128),
-                                                                                (unsigned)(w.n - 1), (unsigned)B),
-                                                                           128, 0, st>>>(
-                                           (const double*)(const void*)w.u, u, act))));
-  smooth(nu2);
+    MLMC_LAUNCH(prof::sized("residual_split_f64", v.n), Ba * interior(v.n) * 7.0 * W, Ba * interior(v.n) * 14.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_residual_split64<LG><<<dim3(pairs, (unsigned)(2 * m), (unsigned)B), 128, 0,
+                                                                    st>>>(Kx, Ky, Kz, D, g, u, r, act))));
+  const dim3 rg((unsigned)(((w.n - 2) * (w.n - 2) + 127) / 128), (unsigned)(w.n - 2), (unsigned)B);
+  const dim3 p1r = plane_grid((w.n - 2) * (w.n - 2), (long long)B * (w.n - 2));
+  const double rbytes = Ba * ((red ? 0.5 : 1.0) * (double)v.n3 + (double)w.n3) * W;
+  if (H.p1 && red)
+    MLMC_LAUNCH("restrict_p1", rbytes, Ba * interior(w.n) * 8.0, st,
+                (k_restrict_p1_red<double, true><<<p1r, kPlaneThreads, 0, st>>>(v.n, B, r, gc, act)));
+  else if (H.p1)
+    MLMC_LAUNCH("restrict_p1", rbytes, Ba * interior(w.n) * 16.0, st,
+                (k_restrict_p1<double, true><<<p1r, kPlaneThreads, 0, st>>>(v.n, B, r, gc, act)));
+  else if (red)
+    MLMC_LAUNCH(Names<T>::restrict_, rbytes, Ba * interior(w.n) * 26.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG, double, true><<<rg, 128, 0, st>>>(r, gc, act))));
+  else
+    MLMC_LAUNCH(Names<T>::restrict_, rbytes, Ba * interior(w.n) * 54.0, st,
+                MLMC_SPLIT_DISPATCH(v.n, (k_restrict_split<LG, double><<<rg, 128, 0, st>>>(r, gc, act))));
+  clear_guess(H, j + 1, nu1, st);
+  vcycle(H, j + 1, nu1, nu2, st, true);
+  prolong_level(H, j, black, st);
+  smooth(nu2, false);
 }
 
 template <typename T>
-void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
+void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
   Level<T>& v = H.lv[j];
   const int* act = H.active;
   const int B = H.B;
@@ -1884,23 +2126,33 @@ void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
   }
   if (H.split) {
     if constexpr (sizeof(T) == 4)
-      vcycle_split(H, j, nu1, nu2, st);
+      vcycle_split(H, j, nu1, nu2, st, zero);
     else
-      vcycle_split64(H, j, nu1, nu2, st);
+      vcycle_split64(H, j, nu1, nu2, st, zero);
     return;
   }
   const int m = v.n - 2;
   const dim3 gs = plane_grid(m * ((v.n - 1) / 2), (long long)B * m);
   // one colour: half of the 7 words per node of a full sweep; 13 flops per updated node
   const double sweep_bytes = Ba * interior(v.n) * 3.5 * W, sweep_flops = Ba * interior(v.n) * 0.5 * 13.0;
-  auto smooth = [&](int sweeps) {
+  auto smooth = [&](int sweeps, bool from_zero) {
     for (int s = 0; s < sweeps; ++s) {
+      const bool z0 = from_zero && s == 0 && !H.fused[j];
+      if (z0 && !H.nodal[j])
+        MLMC_LAUNCH(prof::sized(Names<T>::rbgs, v.n), Ba * interior(v.n) * 1.5 * W, Ba * interior(v.n) * 0.5, st,
+                    (k_rbgs<T, true><<<gs, kPlaneThreads, 0, st>>>(0, v.n, B, v.Kx, v.Ky, v.Kz, v.Dinv, v.g, v.u, act)));
       if constexpr (sizeof(T) == 4) {
         if (H.nodal[j]) {
-          for (int c = 0; c < 2; ++c)
+          const float* kn = (const float*)v.kn;
+          const float* g = (const float*)v.g;
+          float* u = (float*)v.u;
+          if (z0)
+            MLMC_LAUNCH(prof::sized("rbgs_nodal_f32", v.n), Ba * interior(v.n) * 1.5 * W,
+                        Ba * interior(v.n) * 0.5 * 25.0, st,
+                        (k_rbgs_nodal<true><<<gs, kPlaneThreads, 0, st>>>(0, v.n, B, kn, g, u, act)));
+          for (int c = z0 ? 1 : 0; c < 2; ++c)
             MLMC_LAUNCH(prof::sized("rbgs_nodal_f32", v.n), Ba * interior(v.n) * 2.0 * W, Ba * interior(v.n) * 0.5 * 37.0, st,
-                        (k_rbgs_nodal<<<gs, kPlaneThreads, 0, st>>>(c, v.n, B, (const float*)v.kn,
-                                                                   (const float*)v.g, (float*)v.u, act)));
+                        (k_rbgs_nodal<false><<<gs, kPlaneThreads, 0, st>>>(c, v.n, B, kn, g, u, act)));
           continue;
         }
       }
@@ -1910,23 +2162,35 @@ void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
         v.u = v.u2;
         v.u2 = t;
       } else {
-        for (int c = 0; c < 2; ++c)
+        for (int c = z0 ? 1 : 0; c < 2; ++c)
           MLMC_LAUNCH(prof::sized(Names<T>::rbgs, v.n), sweep_bytes, sweep_flops, st,
                       (k_rbgs<T><<<gs, kPlaneThreads, 0, st>>>(c, v.n, B, v.Kx, v.Ky, v.Kz, v.Dinv, v.g, v.u, act)));
       }
     }
   };
-  smooth(nu1);
+  smooth(nu1, zero);
+  const bool red = nu1 > 0;
   bool nodal_res = false;
   if constexpr (sizeof(T) == 4) {
     if (H.nodal[j]) {
-      MLMC_LAUNCH(prof::sized("residual_nodal_f32", v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 37.0, st,
-                  (k_residual_nodal<<<plane_grid(v.n * v.n, (long long)B * v.n), kPlaneThreads, 0, st>>>(
-                      v.n, B, (const float*)v.kn, (const float*)v.g, (const float*)v.u, (float*)v.r, act)));
+      const float* kn = (const float*)v.kn;
+      const float* g = (const float*)v.g;
+      const float* u = (const float*)v.u;
+      if (red)
+        MLMC_LAUNCH(prof::sized("residual_nodal_f32", v.n), Ba * interior(v.n) * 3.0 * W, Ba * interior(v.n) * 18.5, st,
+                    (k_residual_nodal<true><<<plane_grid(v.n * ((v.n + 1) / 2), (long long)B * v.n), kPlaneThreads, 0,
+                                              st>>>(v.n, B, kn, g, u, (float*)v.r, act)));
+      else
+        MLMC_LAUNCH(prof::sized("residual_nodal_f32", v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 37.0, st,
+                    (k_residual_nodal<false><<<plane_grid(v.n * v.n, (long long)B * v.n), kPlaneThreads, 0, st>>>(
+                        v.n, B, kn, g, u, (float*)v.r, act)));
       nodal_res = true;
     }
   }
-  if (!nodal_res) {
+  if (!nodal_res && red) {
+    MLMC_LAUNCH(prof::sized(Names<T>::residual, v.n), Ba * interior(v.n) * 4.0 * W, Ba * interior(v.n) * 7.0, st,
+                (k_residual_red<T><<<gs, kPlaneThreads, 0, st>>>(v.n, B, v.Kx, v.Ky, v.Kz, v.D, v.g, v.u, v.r, act)));
+  } else if (!nodal_res) {
     int zs = 0;
     const dim3 rz = zmarch_grid(v.n, B, &zs);
     MLMC_LAUNCH(prof::sized(Names<T>::residual, v.n), Ba * interior(v.n) * 7.0 * W, Ba * interior(v.n) * 14.0, st,
@@ -1934,25 +2198,25 @@ void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st) {
                                                               act)));
   }
   Level<T>& w = H.lv[j + 1];
-  if (H.p1)
-    MLMC_LAUNCH("restrict_p1", Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 16.0, st,
-                (k_restrict_p1<T><<<plane_grid((w.n - 2) * (w.n - 2), (long long)B * (w.n - 2)), kPlaneThreads, 0,
-                                    st>>>(v.n, B, v.r, w.g, act)));
+  const dim3 p1r = plane_grid((w.n - 2) * (w.n - 2), (long long)B * (w.n - 2));
+  const dim3 fwr = plane_grid((w.n - 2) * (w.n - 1), (long long)B * (w.n - 2));
+  const double rbytes = Ba * ((red ? 0.5 : 1.0) * (double)v.n3 + (double)w.n3) * W;
+  if (H.p1 && red)
+    MLMC_LAUNCH("restrict_p1", rbytes, Ba * interior(w.n) * 8.0, st,
+                (k_restrict_p1_red<T, false><<<p1r, kPlaneThreads, 0, st>>>(v.n, B, v.r, w.g, act)));
+  else if (H.p1)
+    MLMC_LAUNCH("restrict_p1", rbytes, Ba * interior(w.n) * 16.0, st,
+                (k_restrict_p1<T><<<p1r, kPlaneThreads, 0, st>>>(v.n, B, v.r, w.g, act)));
+  else if (red)
+    MLMC_LAUNCH(Names<T>::restrict_, rbytes, Ba * interior(w.n) * 26.0, st,
+                (k_restrict_red<T><<<fwr, kPlaneThreads, 0, st>>>(v.n, B, v.r, w.g, act)));
   else
-    MLMC_LAUNCH(Names<T>::restrict_, Ba * ((double)v.n3 + (double)w.n3) * W, Ba * interior(w.n) * 54.0, st,
-                (k_restrict<T><<<plane_grid((w.n - 2) * (w.n - 1), (long long)B * (w.n - 2)), kPlaneThreads, 0,
-                                 st>>>(v.n, B, v.r, w.g, act)));
-  cudaMemsetAsync(w.u, 0, (size_t)B * w.n3 * sizeof(T), st);
-  vcycle(H, j + 1, nu1, nu2, st);
-  if (H.p1)
-    MLMC_LAUNCH("prolong_p1", Ba * (2.0 * (double)v.n3 + (double)w.n3) * W, Ba * interior(v.n) * 1.5, st,
-                (k_prolong_p1<T><<<plane_grid(m * m, (long long)B * m), kPlaneThreads, 0, st>>>(v.n, B, w.u, v.u,
-                                                                                               act)));
-  else
-    MLMC_LAUNCH(Names<T>::prolong, Ba * (2.0 * (double)v.n3 + (double)w.n3) * W, Ba * interior(v.n) * 4.375, st,
-                (k_prolong_blk<T><<<plane_grid((w.n - 1) * (w.n - 1), (long long)B * (w.n - 1)), 128, 0, st>>>(
-                    v.n, B, w.u, v.u, act)));
-  smooth(nu2);
+    MLMC_LAUNCH(Names<T>::restrict_, rbytes, Ba * interior(w.n) * 54.0, st,
+                (k_restrict<T><<<fwr, kPlaneThreads, 0, st>>>(v.n, B, v.r, w.g, act)));
+  clear_guess(H, j + 1, nu1, st);
+  vcycle(H, j + 1, nu1, nu2, st, true);
+  prolong_level(H, j, nu2 > 0, st);
+  smooth(nu2, false);
 }
 
 // Runs one V-cycle, as a CUDA graph when enabled: the first call captures the cycle's
@@ -1982,16 +2246,17 @@ struct GraphRunner {
   ~GraphRunner() {
     if (exec) cudaGraphExecDestroy(exec);
   }
-  // one V-cycle from grid j0 (the same j0 on every call of one runner)
-  int run(Hier<T>& H, int nu1, int nu2, cudaStream_t st, int j0 = 0) {
+  // one V-cycle from grid j0, from a zero guess or not (the same j0 and zero on every call of
+  // one runner)
+  int run(Hier<T>& H, int nu1, int nu2, cudaStream_t st, bool zero, int j0 = 0) {
     if (!enabled) {
-      vcycle<T>(H, j0, nu1, nu2, st);
+      vcycle<T>(H, j0, nu1, nu2, st, zero);
       return MLMC_OK;
     }
     if (!exec) {
       MLMC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       prof::tape_begin();
-      vcycle<T>(H, j0, nu1, nu2, st);
+      vcycle<T>(H, j0, nu1, nu2, st, zero);
       tape = prof::tape_end();
       cap_act = H.n_act > 0 ? H.n_act : 1;
       cudaGraph_t graph = nullptr;
@@ -2041,10 +2306,9 @@ int pcg_loop(Hier<T>& H, const MGSolveArgs& a, int nu1, int nu2, double rtol, in
     return MLMC_OK;
   };
   // z = M r: one V-cycle from zero on the (FP32 copy of the) residual; partials of r.z
-  const size_t u0_elems = H.split ? split_elems(n) : l0.n3;
   auto precondition = [&]() {
-    MLMC_CUDA_TRY(cudaMemsetAsync(H.lv[0].u, 0, (size_t)B * u0_elems * sizeof(T), st));
-    MLMC_TRY(gr.run(H, nu1, nu2, st));
+    MLMC_CUDA_TRY(clear_guess(H, 0, nu1, st));
+    MLMC_TRY(gr.run(H, nu1, nu2, st, true));
     double* z = mixed ? H.Z : (double*)(void*)H.lv[0].u;
     const float* e32 = mixed ? (const float*)(const void*)H.lv[0].u : nullptr;
     if (H.split)
@@ -2192,7 +2456,7 @@ __device__ __forceinline__ double half_block_sum128(double v, double* warp_part8
   return r;
 }
 
-template <typename T>
+template <typename T, bool ZERO = false>
 __device__ void cta_smooth(const CtaLevel<T>& v, int s, int colour) {
   const int n = v.n, m = n - 2, half = (n - 1) / 2, lh = 31 - __clz(half), per = m * half;
   const size_t n3 = (size_t)n * n * n, n2 = (size_t)n * n;
@@ -2218,36 +2482,43 @@ __device__ void cta_smooth(const CtaLevel<T>& v, int s, int colour) {
         d += kzp;
         const float dinv = __fdividef(1.0f, d);
         float acc = ((const float*)v.g)[p];
-        acc = fmaf(kxm, u[p - 1], acc);
-        acc = fmaf(kxp, u[p + 1], acc);
-        acc = fmaf(kym, u[p - n], acc);
-        acc = fmaf(kyp, u[p + n], acc);
-        acc = fmaf(kzm, u[p - n2], acc);
-        acc = fmaf(kzp, u[p + n2], acc);
+        if (!ZERO) {
+          acc = fmaf(kxm, u[p - 1], acc);
+          acc = fmaf(kxp, u[p + 1], acc);
+          acc = fmaf(kym, u[p - n], acc);
+          acc = fmaf(kyp, u[p + n], acc);
+          acc = fmaf(kzm, u[p - n2], acc);
+          acc = fmaf(kzp, u[p + n2], acc);
+        }
         u[p] = acc * dinv;
         continue;
       }
     }
     T* u = v.u;
     T acc = v.g[p];
-    acc = fma(v.Kx[p - 1], u[p - 1], acc);
-    acc = fma(v.Kx[p], u[p + 1], acc);
-    acc = fma(v.Ky[p - n], u[p - n], acc);
-    acc = fma(v.Ky[p], u[p + n], acc);
-    acc = fma(v.Kz[p - n2], u[p - n2], acc);
-    acc = fma(v.Kz[p], u[p + n2], acc);
+    if (!ZERO) {
+      acc = fma(v.Kx[p - 1], u[p - 1], acc);
+      acc = fma(v.Kx[p], u[p + 1], acc);
+      acc = fma(v.Ky[p - n], u[p - n], acc);
+      acc = fma(v.Ky[p], u[p + n], acc);
+      acc = fma(v.Kz[p - n2], u[p - n2], acc);
+      acc = fma(v.Kz[p], u[p + n2], acc);
+    }
     u[p] = acc * v.Dinv[p];
   }
 }
 
-// in-cycle residual r~ (k_residual_z / k_residual_nodal operations), 0 on the boundary
-template <typename T>
+// in-cycle residual r~ (k_residual_z / k_residual_nodal operations), 0 on the boundary; RED:
+// at the red nodes only (k_residual_red)
+template <typename T, bool RED>
 __device__ void cta_residual(const CtaLevel<T>& v, int s) {
-  const int n = v.n;
+  const int n = v.n, half = (n + 1) / 2, row = RED ? half : n;
   const size_t n3 = (size_t)n * n * n, n2 = (size_t)n * n;
-  for (int i = threadIdx.x; i < (int)n3; i += blockDim.x) {
-    const int z = i / (n * n), rem = i - z * n * n, y = rem / n, x = rem - y * n;
-    const size_t p = (size_t)s * n3 + (size_t)i;
+  for (int i = threadIdx.x; i < row * n * n; i += blockDim.x) {
+    const int z = i / (row * n), rem = i - z * row * n, y = rem / row, xq = rem - y * row;
+    const int x = RED ? 2 * xq + ((y + z) & 1) : xq;
+    if (RED && x > n - 1) continue;
+    const size_t p = (size_t)s * n3 + (size_t)((z * n + y) * n + x);
     T rr = T(0);
     if (x > 0 && y > 0 && z > 0 && x < n - 1 && y < n - 1 && z < n - 1) {
       bool done = false;
@@ -2291,13 +2562,15 @@ __device__ void cta_residual(const CtaLevel<T>& v, int s) {
   }
 }
 
-// g_c = 4 FW(r~) at interior coarse nodes and u_c = 0 (k_restrict's operations)
-template <typename T>
+// g_c = 4 FW(r~) at interior coarse nodes (k_restrict's operations; RED: k_restrict_red's) and
+// u_c = 0 where the coarse grid's first pass reads it (without pre-smoothing: !RED)
+template <typename T, bool RED>
 __device__ void cta_restrict(const CtaLevel<T>& v, const CtaLevel<T>& w, int s) {
   const int nf = v.n, nc = w.n, mc = nc - 2;
   const size_t nf3 = (size_t)nf * nf * nf, nc3 = (size_t)nc * nc * nc;
   const int nf2 = nf * nf;
-  for (int i = threadIdx.x; i < (int)nc3; i += blockDim.x) w.u[(size_t)s * nc3 + i] = T(0);
+  if (!RED)
+    for (int i = threadIdx.x; i < (int)nc3; i += blockDim.x) w.u[(size_t)s * nc3 + i] = T(0);
   for (int i = threadIdx.x; i < mc * mc * mc; i += blockDim.x) {
     const int Z = 1 + i / (mc * mc), rem = i - (Z - 1) * mc * mc, Y = 1 + rem / mc, X = 1 + rem - (Y - 1) * mc;
     const T* rb = v.r + (size_t)s * nf3 + (size_t)(2 * Z * nf2 + 2 * Y * nf + 2 * X);
@@ -2308,6 +2581,7 @@ __device__ void cta_restrict(const CtaLevel<T>& v, const CtaLevel<T>& w, int s) 
       for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
         for (int dx = -1; dx <= 1; ++dx) {
+          if (RED && ((dx + dy + dz) & 1)) continue;
           const T wgt = (T)((2 - abs(dx)) * (2 - abs(dy)) * (2 - abs(dz))) * (T)(1.0 / 16.0);
           acc = fma(wgt, rb[dz * nf2 + dy * nf + dx], acc);
         }
@@ -2315,8 +2589,8 @@ __device__ void cta_restrict(const CtaLevel<T>& v, const CtaLevel<T>& w, int s) 
   }
 }
 
-// u_f += trilinear interpolation of e_c (k_prolong's operations)
-template <typename T>
+// u_f += trilinear interpolation of e_c (k_prolong's operations; BLACK: at the black nodes)
+template <typename T, bool BLACK>
 __device__ void cta_prolong(const CtaLevel<T>& w, const CtaLevel<T>& v, int s) {
   // one coarse cell per thread (k_prolong_blk's sums, bit for bit k_prolong's)
   const int nf = v.n, nc = w.n, mc = nc - 1;
@@ -2331,6 +2605,7 @@ __device__ void cta_prolong(const CtaLevel<T>& w, const CtaLevel<T>& v, int s) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
+      if (BLACK && !((dx + dy + dz) & 1)) continue;
       const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
       if (x < 1 || y < 1 || z < 1 || x > nf - 2 || y > nf - 2 || z > nf - 2) continue;
       const T wgt = dx + dy + dz == 0 ? T(1) : dx + dy + dz == 1 ? T(0.5) : dx + dy + dz == 2 ? T(0.25) : T(0.125);
@@ -2339,18 +2614,29 @@ __device__ void cta_prolong(const CtaLevel<T>& w, const CtaLevel<T>& v, int s) {
   }
 }
 
+// zero: the finest iterate is zero on entry (its interior need not be: with pre-smoothing
+// the first red pass does not read it)
 template <typename T>
-__device__ void cta_vcycle(const CtaArgs<T>& A, int s) {
+__device__ void cta_vcycle(const CtaArgs<T>& A, int s, bool zero) {
   // down: smoothing, residual, restriction
   for (int j = 0; j < A.L - 1; ++j) {
     for (int k = 0; k < A.nu1; ++k)
       for (int c = 0; c < 2; ++c) {
-        cta_smooth(A.lv[j], s, c);
+        if (k == 0 && c == 0 && (j > 0 || zero))
+          cta_smooth<T, true>(A.lv[j], s, c);
+        else
+          cta_smooth<T, false>(A.lv[j], s, c);
         __syncthreads();
       }
-    cta_residual(A.lv[j], s);
+    if (A.nu1 > 0)
+      cta_residual<T, true>(A.lv[j], s);
+    else
+      cta_residual<T, false>(A.lv[j], s);
     __syncthreads();
-    cta_restrict(A.lv[j], A.lv[j + 1], s);
+    if (A.nu1 > 0)
+      cta_restrict<T, true>(A.lv[j], A.lv[j + 1], s);
+    else
+      cta_restrict<T, false>(A.lv[j], A.lv[j + 1], s);
     __syncthreads();
   }
   // exact solve on the 5^3 grid (k_coarse_apply)
@@ -2372,11 +2658,14 @@ __device__ void cta_vcycle(const CtaArgs<T>& A, int s) {
   }
   // up: correction, smoothing
   for (int j = A.L - 2; j >= 0; --j) {
-    cta_prolong(A.lv[j + 1], A.lv[j], s);
+    if (A.nu2 > 0)
+      cta_prolong<T, true>(A.lv[j + 1], A.lv[j], s);
+    else
+      cta_prolong<T, false>(A.lv[j + 1], A.lv[j], s);
     __syncthreads();
     for (int k = 0; k < A.nu2; ++k)
       for (int c = 0; c < 2; ++c) {
-        cta_smooth(A.lv[j], s, c);
+        cta_smooth<T, false>(A.lv[j], s, c);
         __syncthreads();
       }
   }
@@ -2485,7 +2774,7 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
                                                    A.slabs, s, part, warp_part8, bcast);
         act = cta_norm_update(t, g2, A.rtol, A.maxc, inc, &rel, &cyc);
         if (!act) break;
-        cta_vcycle(A, s);
+        cta_vcycle(A, s, false);
       }
     } else if (A.mode == kCtaRefinement) {
       // FP32 V-cycles on FP64 residuals: r32 = g - A x, e = V(r32), x += e
@@ -2495,9 +2784,11 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
                                               warp_part8, bcast);
         act = cta_norm_update(t, g2, A.rtol, A.maxc, inc, &rel, &cyc);
         if (!act) break;
-        for (size_t i = threadIdx.x; i < n3; i += blockDim.x) l0.u[(size_t)s * n3 + i] = T(0);
-        __syncthreads();
-        cta_vcycle(A, s);
+        if (A.nu1 == 0) {
+          for (size_t i = threadIdx.x; i < n3; i += blockDim.x) l0.u[(size_t)s * n3 + i] = T(0);
+          __syncthreads();
+        }
+        cta_vcycle(A, s, true);
         for (size_t i = threadIdx.x; i < n3; i += blockDim.x) A.x[(size_t)s * n3 + i] += widen(l0.u[(size_t)s * n3 + i]);
         __syncthreads();
       }
@@ -2510,9 +2801,11 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
       double rz = 0.0, rzo = 0.0, alpha = 0.0, beta = 0.0;
       // z = M r and the partials of r.z (flat chunks): the preconditioner
       auto precondition = [&]() -> double {
-        for (size_t i = threadIdx.x; i < n3; i += blockDim.x) l0.u[b0 + i] = T(0);
-        __syncthreads();
-        cta_vcycle(A, s);
+        if (A.nu1 == 0) {
+          for (size_t i = threadIdx.x; i < n3; i += blockDim.x) l0.u[b0 + i] = T(0);
+          __syncthreads();
+        }
+        cta_vcycle(A, s, true);
         for (int b = 0; b < A.NB; ++b) {
           const unsigned lo = b * chunk, hi = lo + chunk < (unsigned)n3 ? lo + chunk : (unsigned)n3;
           double acc = 0.0;
@@ -2680,6 +2973,9 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   // smoother per level (explicit choice, or the tuned / default one for that grid)
   for (int j = 0; j < H.L; ++j) {
     Level<T>& v = H.lv[j];
+    // grids whose cycles start from a zero guess: the passes write interior nodes only
+    if (j > 0 || mixed || cg)
+      MLMC_CUDA_TRY(cudaMemsetAsync(v.u, 0, (size_t)B * (H.split ? split_elems(v.n) : v.n3) * sizeof(T), st));
     if (H.split) {
       H.nodal[j] = H.fused[j] = false;
       if (mixed && j < H.L - 1)
@@ -2874,39 +3170,18 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                     (k_prepare<<<plane_grid(v.n * v.n, (long long)B * v.n), kPlaneThreads, 0, st>>>(
                         v.n, B, hj * hj, nullptr, (double*)v.g, (double*)v.u)));
     }
-    vcycle(H, H.L - 1, nu1, nu2, st);
+    vcycle(H, H.L - 1, nu1, nu2, st, true);
     for (int j = H.L - 2; j >= 0; --j) {
       Level<T>& v = H.lv[j];
-      Level<T>& w = H.lv[j + 1];
-      const int m = v.n - 2;
       MLMC_CUDA_TRY(cudaMemsetAsync(v.u, 0, (size_t)B * (H.split ? split_elems(v.n) : v.n3) * sizeof(T), st));
-      if (H.p1 && H.split)
-        MLMC_LAUNCH("prolong_p1", B * (2.0 * (double)v.n3 + (double)w.n3) * W, B * interior(v.n) * 1.5, st,
-                    (k_prolong_p1<T, true><<<plane_grid(m * m, (long long)B * m), kPlaneThreads, 0, st>>>(
-                        v.n, B, w.u, v.u, H.active)));
-      else if (H.p1)
-        MLMC_LAUNCH("prolong_p1", B * (2.0 * (double)v.n3 + (double)w.n3) * W, B * interior(v.n) * 1.5, st,
-                    (k_prolong_p1<T><<<plane_grid(m * m, (long long)B * m), kPlaneThreads, 0, st>>>(
-                        v.n, B, w.u, v.u, H.active)));
-      else if (H.split) {
-        if constexpr (sizeof(T) == 8)
-          MLMC_LAUNCH(Names<T>::prolong, B * (2.0 * (double)v.n3 + (double)w.n3) * W, B * interior(v.n) * 4.375, st,
-                      MLMC_SPLIT_DISPATCH(v.n, (k_prolong_blk_split<LG, double><<<
-                                                   dim3((unsigned)(((w.n - 1) * (w.n - 1) + 127) / 128),
-                                                        (unsigned)(w.n - 1), (unsigned)B),
-                                                   128, 0, st>>>((const double*)(const void*)w.u,
-                                                                 (double*)(void*)v.u, H.active))));
-      } else
-        MLMC_LAUNCH(Names<T>::prolong, B * (2.0 * (double)v.n3 + (double)w.n3) * W, B * interior(v.n) * 4.375, st,
-                    (k_prolong_blk<T><<<plane_grid((w.n - 1) * (w.n - 1), (long long)B * (w.n - 1)), 128, 0, st>>>(
-                        v.n, B, w.u, v.u, H.active)));
+      prolong_level(H, j, nu1 > 0, st);  // the cycle's first red pass overwrites the red nodes
       // with MLMC_FMG_GRAPHS=1 the cycles of grid j replay one graph captured for them (on
       // created streams): a level alone runs 4-6% faster, but the capture and instantiation
       // of every grid's graph in every solve cost more than they save while other level
       // streams keep the GPU busy, so direct launches are the default
       GraphRunner<T> fr;
       fr.enabled = gr.enabled && fmg_graphs();
-      for (int cyc = 0; cyc < maxc; ++cyc) MLMC_TRY(fr.run(H, nu1, nu2, st, j));
+      for (int cyc = 0; cyc < maxc; ++cyc) MLMC_TRY(fr.run(H, nu1, nu2, st, false, j));
     }
     std::vector<int> cyc(B, maxc);
     MLMC_CUDA_TRY(cudaMemcpyAsync(H.cycles, cyc.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -2932,9 +3207,8 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   if (na < 0) return na;
   while (na > 0) {
     if (mixed) {
-      MLMC_CUDA_TRY(
-          cudaMemsetAsync(H.lv[0].u, 0, (size_t)B * (H.split ? split_elems(a.n) : l0.n3) * sizeof(T), st));
-      MLMC_TRY(gr.run(H, nu1, nu2, st));
+      MLMC_CUDA_TRY(clear_guess(H, 0, nu1, st));
+      MLMC_TRY(gr.run(H, nu1, nu2, st, true));
       const dim3 ug = plane_grid(a.n * a.n, (long long)B * a.n);
       if (H.split)
         MLMC_LAUNCH("update_mixed", H.n_act * (double)l0.n3 * (W + 16), H.n_act * (double)l0.n3, st,
@@ -2945,7 +3219,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                     (k_update_mixed<false><<<ug, kPlaneThreads, 0, st>>>(a.n, B, (const float*)H.lv[0].u, a.u,
                                                                            H.active)));
     } else {
-      MLMC_TRY(gr.run(H, nu1, nu2, st));
+      MLMC_TRY(gr.run(H, nu1, nu2, st, false));
     }
     na = residual_check(1);
     if (na < 0) return na;
