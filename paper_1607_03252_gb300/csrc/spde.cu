@@ -112,7 +112,9 @@ __global__ void k_spde_noise(const uint64_t* __restrict__ ids, int B, int lc, in
   }
 }
 
-// One colour of red-black Gauss-Seidel (red: x + y + z even):
+// One colour of red-black Gauss-Seidel (red: x + y + z even), one cell per thread: the plain form
+// of k_cc_rbgs4's pass, as are k_cc_restrict and k_cc_prolong of the restriction and interpolation
+// below (the cycle runs the row forms; these state the cycle in full and are what host runs use):
 // Z_p = (g_p + sum of the neighbours inside the box) / (c h^2 + n_p), with the four
 // possible reciprocals of the diagonal precomputed.
 // Grid (colour cells / blockDim, samples), C = 2^lc >= 4.
@@ -427,7 +429,7 @@ struct SpdeLevels {
   int nl = 0;
   int C[16];
   double *Z64, *g64;                // the FP64 iterate and right-hand side (finest grid)
-  float *e[16], *g[16], *r[16];     // the FP32 correction cycle's grids
+  float *e[16], *g[16];             // the FP32 correction cycle's grids
   double* partial;
   double* g2;
   int *active, *cycles, *flag;
@@ -449,12 +451,10 @@ size_t carve_levels(int B, int n, char* base, SpdeLevels* L) {
     const size_t cells = (size_t)B * c * c * c;
     float* e = (float*)take(cells * 4);
     float* g = (float*)take(cells * 4);
-    float* r = (float*)take(cells * 4);
     if (L) {
       L->C[nl] = c;
       L->e[nl] = e;
       L->g[nl] = g;
-      L->r[nl] = r;
     }
     ++nl;
   }
@@ -478,6 +478,258 @@ size_t carve_levels(int B, int n, char* base, SpdeLevels* L) {
   return (size_t)(p - base);
 }
 
+// The correction cycle's kernels on rows of four cells (16-byte loads, C = 2^lc >= 4), which use
+// the red-black structure: from a zero guess the first red pass is g times the reciprocal
+// diagonal; after a sweep, which ends on black, the black residuals are zero up to rounding, so
+// the coarse right-hand side takes the four red children of the eight; before a sweep, which
+// starts on red, only the black cells need the interpolated correction. They are bound by
+// launch latency up to 32^3 cells and by L2 above (the 128^3 x 4 grid's arrays stay in it).
+// With the small grids' single launch below, a 65^3 x 4 field takes 6.42 instead of 8.99 ms
+// (781 -> 381 launches).
+__device__ __forceinline__ float4 cc_ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float cc_at(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+// reciprocal diagonal of a cell with np neighbours inside the box
+__device__ __forceinline__ float cc_inv(int np, float i3, float i4, float i5, float i6) {
+  return np == 6 ? i6 : (np == 5 ? i5 : (np == 4 ? i4 : i3));
+}
+
+// The two cells of one colour in a row of four: k_cc_rbgs's operations (absent neighbours add
+// zero). ZERO: from a zero iterate. Grid (row quads / blockDim, samples).
+template <bool ZERO>
+__global__ void __launch_bounds__(kT) k_cc_rbgs4(int colour, int lc, int B, float i3, float i4, float i5, float i6,
+                                                 const float* __restrict__ g, float* __restrict__ Z,
+                                                 const int* __restrict__ active) {
+  const int C = 1 << lc;
+  const size_t C3 = (size_t)1 << (3 * lc), C2 = (size_t)1 << (2 * lc);
+  const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (C3 >> 2)) return;
+  const int x0 = (int)(q << 2) & (C - 1), y = (int)(q >> (lc - 2)) & (C - 1), z = (int)(q >> (2 * lc - 2));
+  const int par = (y + z + colour) & 1;  // cells x0 + par and x0 + par + 2
+  const int nyz = (y > 0) + (y < C - 1) + (z > 0) + (z < C - 1);
+  const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (int s = blockIdx.y; s < B; s += gridDim.y) {
+    if (!active[s]) continue;
+    const size_t p = (size_t)s * C3 + (q << 2);
+    const float4 g4 = cc_ld4(g + p);
+    const float ga = par ? g4.y : g4.x, gb = par ? g4.w : g4.z;
+    const int npa = nyz + (x0 + par > 0) + 1, npb = nyz + 1 + (x0 + par + 2 < C - 1);
+    float a = ga, b = gb;
+    if (!ZERO) {
+      const float4 c4 = cc_ld4(Z + p);
+      const float4 ym = y > 0 ? cc_ld4(Z + p - C) : none, yp = y < C - 1 ? cc_ld4(Z + p + C) : none;
+      const float4 zm = z > 0 ? cc_ld4(Z + p - C2) : none, zp = z < C - 1 ? cc_ld4(Z + p + C2) : none;
+      if (par) {
+        a += c4.x, a += c4.z, b += c4.z;
+        if (x0 + 4 < C) b += Z[p + 4];
+        a += ym.y, a += yp.y, a += zm.y, a += zp.y;
+        b += ym.w, b += yp.w, b += zm.w, b += zp.w;
+      } else {
+        if (x0 > 0) a += Z[p - 1];
+        a += c4.y, b += c4.y, b += c4.w;
+        a += ym.x, a += yp.x, a += zm.x, a += zp.x;
+        b += ym.z, b += yp.z, b += zm.z, b += zp.z;
+      }
+    }
+    Z[p + par] = a * cc_inv(npa, i3, i4, i5, i6);
+    Z[p + par + 2] = b * cc_inv(npb, i3, i4, i5, i6);
+  }
+}
+
+// Coarse right-hand side from the red residuals alone, for two coarse cells along x (a row of
+// four fine cells): g_c = (1/2) sum over the red children of g - ((c h^2 + n_p) Z_p - sum Z_q).
+// Nothing is stored on the fine grid. Grid (coarse cell pairs / blockDim, samples), Cf = 2^lcf.
+__global__ void __launch_bounds__(kT) k_cc_restrict_red(int lcf, int B, float ch2, const float* __restrict__ g,
+                                                        const float* __restrict__ Z, float* __restrict__ gc,
+                                                        const int* __restrict__ active) {
+  const int Cf = 1 << lcf, lcc = lcf - 1, Cc = 1 << lcc;
+  const size_t Cf3 = (size_t)1 << (3 * lcf), Cf2 = (size_t)1 << (2 * lcf), Cc3 = Cf3 >> 3;
+  const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (Cc3 >> 1)) return;
+  const int X = (int)(q << 1) & (Cc - 1), Y = (int)(q >> (lcc - 1)) & (Cc - 1), Zc = (int)(q >> (2 * lcc - 1));
+  const int x0 = 2 * X;
+  const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (int s = blockIdx.y; s < B; s += gridDim.y) {
+    if (!active[s]) continue;
+    float sum[2] = {0.0f, 0.0f};
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int y = 2 * Y + b, z = 2 * Zc + c, par = (b + c) & 1;
+        const size_t p = (size_t)s * Cf3 + ((size_t)z << (2 * lcf)) + ((size_t)y << lcf) + x0;
+        const float4 c4 = cc_ld4(Z + p), g4 = cc_ld4(g + p);
+        const float4 ym = y > 0 ? cc_ld4(Z + p - Cf) : none, yp = y < Cf - 1 ? cc_ld4(Z + p + Cf) : none;
+        const float4 zm = z > 0 ? cc_ld4(Z + p - Cf2) : none, zp = z < Cf - 1 ? cc_ld4(Z + p + Cf2) : none;
+        const int nyz = (y > 0) + (y < Cf - 1) + (z > 0) + (z < Cf - 1);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int i = par + 2 * k, x = x0 + i;  // the red child of coarse cell X + k in this row
+          const float l = i > 0 ? cc_at(c4, i - 1) : (x > 0 ? Z[p - 1] : 0.0f);
+          const float r = i < 3 ? cc_at(c4, i + 1) : (x < Cf - 1 ? Z[p + 4] : 0.0f);
+          float nb = cc_at(zm, i) + cc_at(zp, i);
+          nb += l;
+          nb += r;
+          nb += cc_at(ym, i);
+          nb += cc_at(yp, i);
+          const int np = nyz + (x > 0) + (x < Cf - 1);
+          sum[k] += cc_at(g4, i) - ((ch2 + (float)np) * cc_at(c4, i) - nb);
+        }
+      }
+    float* o = gc + (size_t)s * Cc3 + (q << 1);
+    *reinterpret_cast<float2*>(o) = make_float2(0.5f * sum[0], 0.5f * sum[1]);
+  }
+}
+
+// k_cc_prolong at the two black cells of a row of four (its weights and order). Grid (fine row
+// quads / blockDim, samples), Cf = 2^lcf.
+__global__ void __launch_bounds__(kT) k_cc_prolong_black(int lcf, int B, const float* __restrict__ ec,
+                                                         float* __restrict__ Z, const int* __restrict__ active) {
+  const int Cf = 1 << lcf, lcc = lcf - 1, Cc = Cf / 2;
+  const size_t Cf3 = (size_t)1 << (3 * lcf), Cc3 = Cf3 >> 3;
+  const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (Cf3 >> 2)) return;
+  const int x0 = (int)(q << 2) & (Cf - 1), y = (int)(q >> (lcf - 2)) & (Cf - 1), z = (int)(q >> (2 * lcf - 2));
+  const int par = (y + z + 1) & 1;  // black cells x0 + par and x0 + par + 2
+  const int X = x0 >> 1;            // parents X (cells x0, x0 + 1) and X + 1
+  int iy[2] = {y >> 1, (y & 1) ? (y >> 1) + 1 : (y >> 1) - 1};
+  int iz[2] = {z >> 1, (z & 1) ? (z >> 1) + 1 : (z >> 1) - 1};
+  if (iy[1] < 0 || iy[1] >= Cc) iy[1] = iy[0];
+  if (iz[1] < 0 || iz[1] >= Cc) iz[1] = iz[0];
+  // x neighbours of the two parents: an odd cell leans right, an even one left
+  const int na = par ? X + 1 : (X > 0 ? X - 1 : X), nb = par ? (X + 2 < Cc ? X + 2 : X + 1) : X;
+  for (int s = blockIdx.y; s < B; s += gridDim.y) {
+    if (!active[s]) continue;
+    const float* eb = ec + (size_t)s * Cc3;
+    float va[2], vb[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float wa[2], wb[2];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const float* row = eb + ((((size_t)iz[c] << lcc) + iy[b]) << lcc);
+        wa[b] = 0.75f * row[X] + 0.25f * row[na];
+        wb[b] = 0.75f * row[X + 1] + 0.25f * row[nb];
+      }
+      va[c] = 0.75f * wa[0] + 0.25f * wa[1];
+      vb[c] = 0.75f * wb[0] + 0.25f * wb[1];
+    }
+    float* o = Z + (size_t)s * Cf3 + (q << 2) + par;
+    o[0] += 0.75f * va[0] + 0.25f * va[1];
+    o[2] += 0.75f * vb[0] + 0.25f * vb[1];
+  }
+}
+
+// The correction cycle on the grids of at most kTailC cells per axis, one block per sample, in
+// shared memory: sweeps, red residuals, restriction, interpolation and the exact 2^3 solve with
+// block barriers between the passes (the batched kernels' operations). As launches these grids
+// were bound by launch latency: 37 of a cycle's 75 launches. Reads g of its finest grid, writes
+// e. C0 = 2^lc0 <= kTailC.
+constexpr int kTailC = 16, kTailThreads = 512;
+struct TailDiag {
+  float ch2[5], inv[5][4];  // per lc = 0 .. 4: c h^2 and the reciprocal diagonals of 3 .. 6 neighbours
+};
+__device__ __forceinline__ int tail_off(int lc) {  // offset of grid lc in the shared arrays
+  return lc == 4 ? 0 : lc == 3 ? 4096 : lc == 2 ? 4608 : 4672;
+}
+__global__ void __launch_bounds__(kTailThreads) k_cc_tail(int lc0, TailDiag td, const float* __restrict__ g0,
+                                                          float* __restrict__ e0, const int* __restrict__ active) {
+  __shared__ float sg[4680], se[4680];
+  const int s = blockIdx.x, tid = threadIdx.x;
+  if (!active[s]) return;
+  const int n0 = 1 << (3 * lc0);
+  for (int i = tid; i < n0; i += kTailThreads) sg[tail_off(lc0) + i] = g0[(size_t)s * n0 + i];
+  __syncthreads();
+  // one colour pass on grid lc
+  auto pass = [&](int lc, int colour, bool zero) {
+    const int C = 1 << lc, C2 = C * C;
+    const float* g = sg + tail_off(lc);
+    float* e = se + tail_off(lc);
+    const float* inv = td.inv[lc];
+    for (int i = tid; i < (C2 * C) / 2; i += kTailThreads) {
+      const int row = i >> (lc - 1), y = row & (C - 1), z = row >> lc;
+      const int x = 2 * (i & (C / 2 - 1)) + ((y + z + colour) & 1), p = (row << lc) + x;
+      float acc = g[p];
+      if (!zero) {
+        if (x > 0) acc += e[p - 1];
+        if (x < C - 1) acc += e[p + 1];
+        if (y > 0) acc += e[p - C];
+        if (y < C - 1) acc += e[p + C];
+        if (z > 0) acc += e[p - C2];
+        if (z < C - 1) acc += e[p + C2];
+      }
+      const int np = (x > 0) + (x < C - 1) + (y > 0) + (y < C - 1) + (z > 0) + (z < C - 1);
+      e[p] = acc * inv[np - 3];
+    }
+    __syncthreads();
+  };
+  for (int lc = lc0; lc > 1; --lc) {
+    pass(lc, 0, true);
+    pass(lc, 1, false);
+    pass(lc, 0, false);
+    pass(lc, 1, false);
+    const int C = 1 << lc, C2 = C * C, lcc = lc - 1, Cc = 1 << lcc;
+    const float* g = sg + tail_off(lc);
+    const float* e = se + tail_off(lc);
+    const float ch2 = td.ch2[lc];
+    for (int i = tid; i < Cc * Cc * Cc; i += kTailThreads) {
+      const int X = i & (Cc - 1), Y = (i >> lcc) & (Cc - 1), Z = i >> (2 * lcc);
+      float sum = 0.0f;
+      for (int k = 0; k < 4; ++k) {
+        const int c = k >> 1, b = k & 1, x = 2 * X + ((b + c) & 1), y = 2 * Y + b, z = 2 * Z + c;
+        const int p = (((z << lc) + y) << lc) + x;
+        float nb = (z > 0 ? e[p - C2] : 0.0f) + (z < C - 1 ? e[p + C2] : 0.0f);
+        if (x > 0) nb += e[p - 1];
+        if (x < C - 1) nb += e[p + 1];
+        if (y > 0) nb += e[p - C];
+        if (y < C - 1) nb += e[p + C];
+        const int np = (x > 0) + (x < C - 1) + (y > 0) + (y < C - 1) + (z > 0) + (z < C - 1);
+        sum += g[p] - ((ch2 + (float)np) * e[p] - nb);
+      }
+      sg[tail_off(lcc) + i] = 0.5f * sum;
+    }
+    __syncthreads();
+  }
+  if (tid < 8) {  // k_cc_coarse, one cell per thread
+    const float* g = sg + tail_off(1);
+    float a = 0.0f;
+    for (int m = 0; m < 8; ++m) {
+      float G = 0.0f;
+      for (int p = 0; p < 8; ++p) G += (__popc(m & p) & 1) ? -g[p] : g[p];
+      G /= td.ch2[1] + 2.0f * (float)__popc(m);
+      a += (__popc(m & tid) & 1) ? -G : G;
+    }
+    se[tail_off(1) + tid] = 0.125f * a;
+  }
+  __syncthreads();
+  for (int lc = 2; lc <= lc0; ++lc) {
+    const int C = 1 << lc, lcc = lc - 1, Cc = 1 << lcc;
+    const float* ec = se + tail_off(lcc);
+    float* e = se + tail_off(lc);
+    for (int i = tid; i < (C * C * C) / 2; i += kTailThreads) {
+      const int row = i >> (lc - 1), y = row & (C - 1), z = row >> lc;
+      const int x = 2 * (i & (C / 2 - 1)) + ((y + z + 1) & 1);
+      const int X = x >> 1, Y = y >> 1, Z = z >> 1;
+      int nx = (x & 1) ? X + 1 : X - 1, ny = (y & 1) ? Y + 1 : Y - 1, nz = (z & 1) ? Z + 1 : Z - 1;
+      if (nx < 0 || nx >= Cc) nx = X;
+      if (ny < 0 || ny >= Cc) ny = Y;
+      if (nz < 0 || nz >= Cc) nz = Z;
+      auto row_lerp = [&](int zz, int yy) {
+        const float* r = ec + (((zz << lcc) + yy) << lcc);
+        return 0.75f * r[X] + 0.25f * r[nx];
+      };
+      const float v0 = 0.75f * row_lerp(Z, Y) + 0.25f * row_lerp(Z, ny);
+      const float v1 = 0.75f * row_lerp(nz, Y) + 0.25f * row_lerp(nz, ny);
+      e[(row << lc) + x] += 0.75f * v0 + 0.25f * v1;
+    }
+    __syncthreads();
+    pass(lc, 0, false);
+    pass(lc, 1, false);
+    pass(lc, 0, false);
+    pass(lc, 1, false);
+  }
+  for (int i = tid; i < n0; i += kTailThreads) e0[(size_t)s * n0 + i] = se[tail_off(lc0) + i];
+}
+
 int log2i(int c) {
   int l = 0;
   while ((1 << l) < c) ++l;
@@ -487,44 +739,51 @@ int log2i(int c) {
 // Grid of a per-sample cell kernel: enough blocks for `per` items, samples on y.
 dim3 cell_grid(size_t per, int B) { return dim3((unsigned)((per + kT - 1) / kT), (unsigned)(B < 65535 ? B : 65535)); }
 
-// FP32 V(2,2) cycle on grid l: e_l ~ A_l^-1 g_l (e_l zero on entry).
+// FP32 V(2,2) cycle on grid l: e_l ~ A_l^-1 g_l (e_l's values on entry are not used).
 int vcycle32(const SpdeLevels& L, int l, int B, double kappa, double h0, cudaStream_t st) {
   const int C = L.C[l], lc = log2i(C);
-  const double hl = h0 * (double)(1 << l), ch2d = kappa * kappa * hl * hl;
+  auto ch2_of = [&](int j) {
+    const double hj = h0 * (double)(1 << j);
+    return kappa * kappa * hj * hj;
+  };
+  const double ch2d = ch2_of(l);
   const float ch2 = (float)ch2d;
   const size_t cells = (size_t)B * C * C * C;
-  if (C == 2) {
-    MLMC_LAUNCH("spde_coarse", cells * 8.0, cells * 64.0, st,
-                (k_cc_coarse<float><<<(B + 127) / 128, 128, 0, st>>>(B, ch2, L.g[l], L.e[l], L.active)));
+  if (C <= kTailC) {
+    TailDiag td{};
+    for (int j = l, k = lc; k >= 1; ++j, --k) {
+      td.ch2[k] = (float)ch2_of(j);
+      for (int np = 3; np <= 6; ++np) td.inv[k][np - 3] = (float)(1.0 / (ch2_of(j) + (double)np));
+    }
+    MLMC_LAUNCH("spde_tail", cells * 8.0, cells * 60.0, st,
+                (k_cc_tail<<<B, kTailThreads, 0, st>>>(lc, td, L.g[l], L.e[l], L.active)));
     return MLMC_OK;
   }
   const float i3 = (float)(1.0 / (ch2d + 3.0)), i4 = (float)(1.0 / (ch2d + 4.0)), i5 = (float)(1.0 / (ch2d + 5.0)),
               i6 = (float)(1.0 / (ch2d + 6.0));
-  auto sweep = [&]() {
-    for (int colour = 0; colour < 2; ++colour)
+  const dim3 quads = cell_grid(((size_t)C * C * C) / 4, B);
+  auto sweep = [&](bool zero) {
+    if (zero)
+      MLMC_LAUNCH("spde_rbgs", cells * 4.0, cells * 0.5, st,
+                  (k_cc_rbgs4<true><<<quads, kT, 0, st>>>(0, lc, B, i3, i4, i5, i6, L.g[l], L.e[l], L.active)));
+    else
       MLMC_LAUNCH("spde_rbgs", cells * 6.0, cells * 4.0, st,
-                  (k_cc_rbgs<float><<<cell_grid(((size_t)C * C * C) / 2, B), kT, 0, st>>>(
-                      colour, lc, B, i3, i4, i5, i6, L.g[l], L.e[l], L.active)));
+                  (k_cc_rbgs4<false><<<quads, kT, 0, st>>>(0, lc, B, i3, i4, i5, i6, L.g[l], L.e[l], L.active)));
+    MLMC_LAUNCH("spde_rbgs", cells * 6.0, cells * 4.0, st,
+                (k_cc_rbgs4<false><<<quads, kT, 0, st>>>(1, lc, B, i3, i4, i5, i6, L.g[l], L.e[l], L.active)));
   };
-  sweep();
-  sweep();
-  int zs = 0;
-  const int slabs = zslabs(C, &zs);
-  MLMC_LAUNCH("spde_residual", cells * 12.0, cells * 9.0, st,
-              (k_cc_residual<float, float><<<dim3(col_blocks(C), slabs, B), 128, 0, st>>>(
-                  lc, zs, ch2, L.g[l], L.e[l], L.r[l], nullptr, L.active)));
+  sweep(true);
+  sweep(false);
   const int Cc = L.C[l + 1];
   const size_t ccells = (size_t)B * Cc * Cc * Cc;
-  MLMC_LAUNCH("spde_restrict", cells * 4.0 + ccells * 4.0, cells * 1.0, st,
-              (k_cc_restrict<float><<<cell_grid((size_t)Cc * Cc * Cc, B), kT, 0, st>>>(lc - 1, B, L.r[l], L.g[l + 1],
-                                                                                        L.active)));
-  MLMC_CUDA_TRY(cudaMemsetAsync(L.e[l + 1], 0, ccells * sizeof(float), st));
+  MLMC_LAUNCH("spde_restrict", cells * 6.0 + ccells * 4.0, cells * 5.0, st,
+              (k_cc_restrict_red<<<cell_grid(((size_t)Cc * Cc * Cc) / 2, B), kT, 0, st>>>(lc, B, ch2, L.g[l], L.e[l],
+                                                                                           L.g[l + 1], L.active)));
   MLMC_TRY(vcycle32(L, l + 1, B, kappa, h0, st));
-  MLMC_LAUNCH("spde_prolong", cells * 8.0 + ccells * 4.0, cells * 10.0, st,
-              (k_cc_prolong<float><<<cell_grid((size_t)C * C * C, B), kT, 0, st>>>(lc, B, L.e[l + 1], L.e[l],
-                                                                                    L.active)));
-  sweep();
-  sweep();
+  MLMC_LAUNCH("spde_prolong", cells * 4.0 + ccells * 4.0, cells * 7.0, st,
+              (k_cc_prolong_black<<<quads, kT, 0, st>>>(lc, B, L.e[l + 1], L.e[l], L.active)));
+  sweep(false);
+  sweep(false);
   return MLMC_OK;
 }
 
@@ -575,7 +834,6 @@ int spde_field_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, in
     MLMC_CUDA_TRY(cudaMemcpyAsync(&flag, L.flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     MLMC_CUDA_TRY(cudaStreamSynchronize(st));
     if (!(flag & 1)) break;
-    MLMC_CUDA_TRY(cudaMemsetAsync(L.e[0], 0, cells * sizeof(float), st));
     MLMC_TRY(vcycle32(L, 0, B, kappa, h, st));
     MLMC_LAUNCH("spde_update", cells * 20.0, cells * 1.0, st,
                 (k_cc_update<<<cell_grid(C3, B), kT, 0, st>>>(lc, B, L.e[0], L.Z64, L.active)));
