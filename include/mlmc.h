@@ -162,8 +162,8 @@ typedef struct {
                           its transpose. FP64, stored-face smoothers. */
 
 /* Execution engine of a solve (no counterpart in the paper; same results bit for bit).
- * MLMC_ENGINE_BATCHED: every phase of the cycle is a kernel over the whole batch, one
- * convergence test per cycle on the host. MLMC_ENGINE_CTA (finite volumes, stationary
+ * MLMC_ENGINE_BATCHED: every phase of the cycle is a kernel over the whole batch (the cycle
+ * below the finest grid, from 17^3 down, is one), one convergence test per cycle on the host. MLMC_ENGINE_CTA (finite volumes, stationary
  * cycles, refinement or CG, grids up to 33^3; otherwise the batched engine runs): one
  * persistent launch for the whole solve, each CTA taking the next sample from a device
  * counter and running all of its cycles, the convergence tests and the CG recurrences

@@ -26,6 +26,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -1945,6 +1946,7 @@ struct Hier {
   bool nodal[kMaxLevels] = {};    // two-pass sweep on the nodal coefficient (FP32)
   bool p1 = false;                // P1 finite elements: P1 transfers instead of FW / trilinear
   bool split = false;             // FP32 hierarchy in colour-split storage (MLMC_SMOOTH_SPLIT)
+  bool tail_finest = false;       // the one-launch cycle may start on the finest grid (FMG)
 };
 
 // Lays out the workspace. Level-0 u of FP64 solves is the caller's array (not carved).
@@ -2064,6 +2066,332 @@ cudaError_t clear_guess(const Hier<T>& H, int j, int nu1, cudaStream_t st) {
 // zero: u is zero on entry (cleared by clear_guess, where that is needed).
 template <typename T>
 void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero);
+
+// ---------------------------------------------------------------------------------
+// The V-cycle below a grid of at most 17^3 nodes as one launch, one block per sample.
+// As launches its 20 (9^3: 10) passes are bound by launch latency, about 2.3 us each, for any
+// batch up to a few hundred samples. Here the iterate, the right-hand side and the red residuals
+// of every grid sit in shared memory (FP64: 112 KB from 17^3, two blocks per SM) and the passes
+// are separated by block barriers; FP32 coefficients are staged too (nodal 1/k or stored faces),
+// FP64 faces are read from L2 in the storage they have (plain or colour-split). Every node takes
+// the batched kernels' operations in their order, so the iterates are theirs bit for bit. A red
+// node (x, y, z) has an even linear index (N is odd), hence the half-size residual array. What
+// bounds it: FP64 one SM's FP64 pipe (about 26 us a V(2,2) cycle from 17^3, whatever the batch up
+// to two blocks an SM), FP32 the barriers. A mixed 33^3 x 48 solve 4.81 -> 3.81 ms (608 -> 256
+// launches), an FP64 65^3 x 19 solve 9.03 -> 8.57, the 65^3 P1 / FMG level of 108 samples 21.9 ->
+// 20.3, the 129^3 level of 24 66.0 -> 65.3; one launch takes 33 us (FP32, 2 samples) to 94 us
+// (FP64 V(4,4), 108 samples).
+// ---------------------------------------------------------------------------------
+constexpr int kTailN = 17, kTailThreads = 512;
+template <typename T>
+struct TailLevel {
+  const T *Kx, *Ky, *Kz, *D, *Dinv, *kn;  // kn: the nodal sweep of FP32 grids, else NULL
+  const T* g;
+  T* u;
+};
+template <typename T>
+struct TailArgs {
+  TailLevel<T> lv[2];  // from the finest grid of the tail (17^3 or 9^3)
+  const double* Ainv;
+  const int* active;
+  int nu1, nu2, zero;
+};
+
+// One grid of the tail in a block: shared u, g, r and its coefficients (CS: colour-split FP64
+// arrays in global memory; otherwise plain, shared for FP32 and global for FP64).
+template <typename T, int N, bool CS>
+struct TailGrid {
+  T *u, *g, *r;
+  const T *Kx, *Ky, *Kz, *D, *Dinv, *kn;
+  static constexpr int N1 = N, N2 = N * N, N3 = N * N * N, M = N - 2, HALF = (N - 1) / 2;
+  static constexpr int P = (((N + 1) / 2) + 3) & ~3, BLK = N * N * P;
+  static constexpr int shared_iter = 2 * N3 + (N3 + 1) / 2;  // elements of u, g, r
+  __device__ static __forceinline__ int at(int x, int y, int z) {
+    return CS ? ((x + y + z) & 1) * BLK + (z * N + y) * P + (x >> 1) : (z * N + y) * N + x;
+  }
+  // node `it` of the colour, or false where the row has no such node
+  __device__ static __forceinline__ bool node(int it, int colour, int& x, int& y, int& z) {
+    const int zi = it / (M * HALF), q = it - zi * (M * HALF), yi = q / HALF;
+    z = 1 + zi;
+    y = 1 + yi;
+    x = (((1 + y + z) & 1) == colour ? 1 : 2) + 2 * (q - yi * HALF);
+    return x <= N - 2;
+  }
+  __device__ void pass(int colour, bool zero) const {
+    for (int it = threadIdx.x; it < M * M * HALF; it += kTailThreads) {
+      int x, y, z;
+      if (!node(it, colour, x, y, z)) continue;
+      const int p = (z * N + y) * N + x;
+      if constexpr (sizeof(T) == 4) {
+        if (kn) {
+          u[p] = zero ? nodal_update<true>(kn[p], g[p], kn[p - 1], 0.f, kn[p + 1], 0.f, kn[p - N], 0.f, kn[p + N], 0.f,
+                                           kn[p - N2], 0.f, kn[p + N2], 0.f)
+                      : nodal_update(kn[p], g[p], kn[p - 1], u[p - 1], kn[p + 1], u[p + 1], kn[p - N], u[p - N],
+                                     kn[p + N], u[p + N], kn[p - N2], u[p - N2], kn[p + N2], u[p + N2]);
+          continue;
+        }
+      }
+      const int o = at(x, y, z);
+      T acc = g[p];
+      if (!zero) {
+        acc = fma(Kx[at(x - 1, y, z)], u[p - 1], acc);
+        acc = fma(Kx[o], u[p + 1], acc);
+        acc = fma(Ky[at(x, y - 1, z)], u[p - N], acc);
+        acc = fma(Ky[o], u[p + N], acc);
+        acc = fma(Kz[at(x, y, z - 1)], u[p - N2], acc);
+        acc = fma(Kz[o], u[p + N2], acc);
+      }
+      u[p] = acc * Dinv[o];
+    }
+    __syncthreads();
+  }
+  __device__ void red_residual() const {
+    for (int it = threadIdx.x; it < M * M * HALF; it += kTailThreads) {
+      int x, y, z;
+      if (!node(it, 0, x, y, z)) continue;
+      const int p = (z * N + y) * N + x;
+      if constexpr (sizeof(T) == 4) {
+        if (kn) {
+          r[p >> 1] = nodal_residual(kn[p], g[p], u[p], kn[p - 1], u[p - 1], kn[p + 1], u[p + 1], kn[p - N], u[p - N],
+                                     kn[p + N], u[p + N], kn[p - N2], u[p - N2], kn[p + N2], u[p + N2]);
+          continue;
+        }
+      }
+      const int o = at(x, y, z);
+      T rr = fma(-D[o], u[p], g[p]);
+      rr = fma(Kx[at(x - 1, y, z)], u[p - 1], rr);
+      rr = fma(Kx[o], u[p + 1], rr);
+      rr = fma(Ky[at(x, y - 1, z)], u[p - N], rr);
+      rr = fma(Ky[o], u[p + N], rr);
+      rr = fma(Kz[at(x, y, z - 1)], u[p - N2], rr);
+      rr = fma(Kz[o], u[p + N2], rr);
+      r[p >> 1] = rr;
+    }
+    __syncthreads();
+  }
+  // g of the coarse grid from the red residuals (k_restrict_red, P1: k_restrict_p1_red)
+  template <bool P1>
+  __device__ void restrict_to(T* gc) const {
+    constexpr int NC = (N + 1) / 2, MC = NC - 2;
+    for (int it = threadIdx.x; it < MC * MC * MC; it += kTailThreads) {
+      const int Z = 1 + it / (MC * MC), q = it % (MC * MC), Y = 1 + q / MC, X = 1 + q % MC;
+      const int p = (2 * Z * N + 2 * Y) * N + 2 * X;
+      auto R = [&](int dx, int dy, int dz) { return r[(p + (dz * N + dy) * N + dx) >> 1]; };
+      T v = 0;
+      if (P1) {
+        T acc = R(-1, -1, 0) + R(1, 1, 0);
+        acc += R(0, -1, -1) + R(0, 1, 1);
+        acc += R(-1, 0, -1) + R(1, 0, 1);
+        v = T(0.5) * R(0, 0, 0) + T(0.25) * acc;
+      } else {
+#pragma unroll
+        for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+          for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+            for (int dx = -1; dx <= 1; ++dx) {
+              if ((dx + dy + dz) & 1) continue;
+              const T wgt = (T)((2 - abs(dx)) * (2 - abs(dy)) * (2 - abs(dz))) * (T)(1.0 / 16.0);
+              v = fma(wgt, R(dx, dy, dz), v);
+            }
+      }
+      gc[(Z * NC + Y) * NC + X] = v;
+    }
+    __syncthreads();
+  }
+  // u += the interpolated coarse correction at the black nodes (k_prolong_blk, k_prolong_p1_black)
+  template <bool P1>
+  __device__ void prolong_from(const T* ec) const {
+    constexpr int NC = (N + 1) / 2, MC = NC - 1;
+    if (P1) {
+      for (int it = threadIdx.x; it < M * M * HALF; it += kTailThreads) {
+        int x, y, z;
+        if (!node(it, 1, x, y, z)) continue;
+        const int dx = x & 1, dy = y & 1, dz = z & 1, c = ((z >> 1) * NC + (y >> 1)) * NC + (x >> 1);
+        u[(z * N + y) * N + x] += T(0.5) * (ec[c] + ec[c + (dz * NC + dy) * NC + dx]);
+      }
+    } else {
+      for (int it = threadIdx.x; it < MC * MC * MC; it += kTailThreads) {
+        const int Z = it / (MC * MC), q = it % (MC * MC), Y = q / MC, X = q % MC;
+        const T* e = ec + (Z * NC + Y) * NC + X;
+        const T c[8] = {e[0], e[1], e[NC], e[NC + 1], e[NC * NC], e[NC * NC + 1], e[NC * NC + NC], e[NC * NC + NC + 1]};
+        T v[8];
+        prolong_block_sums(c, v);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
+          if (!((dx + dy + dz) & 1)) continue;
+          const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
+          if (x < 1 || y < 1 || z < 1 || x > N - 2 || y > N - 2 || z > N - 2) continue;
+          const T w = dx + dy + dz == 1 ? T(0.5) : T(0.125);
+          u[(z * N + y) * N + x] += w * v[k];
+        }
+      }
+    }
+    __syncthreads();
+  }
+};
+
+// FP32 coefficients staged in shared memory: nodal 1/k, or Kx, Ky, Kz, D, 1/D
+inline int tail_coef_arrays(bool f32, bool nodal) { return f32 ? (nodal ? 1 : 5) : 0; }
+
+template <typename T, int N0, bool SPLIT, bool P1>
+__global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> A) {
+  constexpr bool F32 = sizeof(T) == 4, CS = SPLIT && !F32;
+  constexpr int LV = N0 == 17 ? 2 : 1;
+  using G0 = TailGrid<T, N0, CS>;
+  using G1 = TailGrid<T, 9, CS>;
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  const int s = blockIdx.x, tid = threadIdx.x;
+  if (!A.active[s]) return;
+  T* sm = reinterpret_cast<T*>(tail_smem);
+  T* const base = sm;
+  G0 a;
+  G1 b;
+  auto carve = [&](auto& G) {
+    using G_ = typename std::remove_reference<decltype(G)>::type;
+    G.u = sm;
+    G.g = sm + G_::N3;
+    G.r = sm + 2 * G_::N3;
+    sm += G_::shared_iter;
+  };
+  carve(a);
+  if (LV == 2) carve(b);
+  T* const u5 = sm;
+  T* const g5 = sm + 125;
+  sm += 250;
+  for (int i = tid; i < (int)(sm - base); i += kTailThreads) base[i] = T(0);
+  // the coefficients: plain FP32 copies in shared memory, FP64 where they are
+  auto coefs = [&](auto& G, const TailLevel<T>& L) {
+    using G_ = typename std::remove_reference<decltype(G)>::type;
+    constexpr size_t NS = SPLIT ? (size_t)2 * G_::BLK : (size_t)G_::N3;
+    const size_t o = (size_t)s * NS;
+    G.kn = nullptr;
+    if constexpr (!F32) {
+      G.Kx = L.Kx + o;
+      G.Ky = L.Ky + o;
+      G.Kz = L.Kz + o;
+      G.D = L.D + o;
+      G.Dinv = L.Dinv + o;
+    } else {
+      auto stage = [&](const T* src) -> const T* {
+        T* dst = sm;
+        for (int i = tid; i < G_::N3; i += kTailThreads) {
+          const int z = i / G_::N2, q = i - z * G_::N2, y = q / G_::N1, x = q - y * G_::N1;
+          dst[i] = src[o + (SPLIT ? ((x + y + z) & 1) * G_::BLK + (z * G_::N1 + y) * G_::P + (x >> 1) : i)];
+        }
+        sm += G_::N3;
+        return dst;
+      };
+      if (L.kn) {
+        G.kn = stage(L.kn);
+      } else {
+        G.Kx = stage(L.Kx);
+        G.Ky = stage(L.Ky);
+        G.Kz = stage(L.Kz);
+        G.D = stage(L.D);
+        G.Dinv = stage(L.Dinv);
+      }
+    }
+  };
+  coefs(a, A.lv[0]);
+  if (LV == 2) coefs(b, A.lv[1]);
+  __syncthreads();
+  // interior nodes of the finest grid of the tail: its g and, from a non-zero guess, its u
+  auto each = [&](auto fn) {
+    constexpr int M = N0 - 2;
+    for (int i = tid; i < M * M * M; i += kTailThreads) {
+      const int z = 1 + i / (M * M), q = i % (M * M), y = 1 + q / M, x = 1 + q % M;
+      const size_t o = SPLIT ? (size_t)s * 2 * G0::BLK + (size_t)(((x + y + z) & 1) * G0::BLK + (z * N0 + y) * G0::P + (x >> 1))
+                             : (size_t)s * G0::N3 + (size_t)((z * N0 + y) * N0 + x);
+      fn((z * N0 + y) * N0 + x, o);
+    }
+  };
+  each([&](int p, size_t o) {
+    a.g[p] = A.lv[0].g[o];
+    if (!A.zero) a.u[p] = A.lv[0].u[o];
+  });
+  __syncthreads();
+  auto down = [&](auto& G, T* gc, bool zero) {
+    for (int k = 0; k < A.nu1; ++k)
+      for (int c = 0; c < 2; ++c) G.pass(c, zero && k == 0 && c == 0);
+    G.red_residual();
+    G.template restrict_to<P1>(gc);
+  };
+  auto up = [&](auto& G, const T* ec) {
+    G.template prolong_from<P1>(ec);
+    for (int k = 0; k < A.nu2; ++k)
+      for (int c = 0; c < 2; ++c) G.pass(c, false);
+  };
+  down(a, LV == 2 ? b.g : g5, A.zero != 0);
+  if constexpr (LV == 2) down(b, g5, true);
+  if (tid < 27) {  // the exact solve (k_coarse_apply)
+    const double* X = A.Ainv + (size_t)s * 729 + (size_t)tid * 27;
+    double v = 0.0;
+    for (int q = 0; q < 27; ++q)
+      v = fma(X[q], (double)g5[((1 + q / 9) * 5 + 1 + (q / 3) % 3) * 5 + 1 + q % 3], v);
+    u5[((1 + tid / 9) * 5 + 1 + (tid / 3) % 3) * 5 + 1 + tid % 3] = (T)v;
+  }
+  __syncthreads();
+  if constexpr (LV == 2) up(b, u5);
+  up(a, LV == 2 ? b.u : u5);
+  each([&](int p, size_t o) { A.lv[0].u[o] = a.u[p]; });
+}
+
+// Whether the cycle from grid j down runs as one launch: grids of 17^3 or 9^3 below the finest
+// (for an FMG cycle, which has no small-grid engine, also the finest grid, unless the batched
+// engine is asked for), with both pre- and post-smoothing (the red-black shortcuts).
+template <typename T>
+inline bool tail_applies(const Hier<T>& H, int j, int nu1, int nu2) {
+  const int n = H.lv[j].n;
+  return (n == 17 || n == 9) && (j > 0 || H.tail_finest) && nu1 > 0 && nu2 > 0;
+}
+
+template <typename T, int N0, bool SPLIT, bool P1>
+cudaError_t tail_launch(const TailArgs<T>& A, int B, int coef0, int coef1, cudaStream_t st) {
+  constexpr int N1 = 9;
+  const size_t elems = (size_t)TailGrid<T, N0, false>::shared_iter + 250 + (size_t)coef0 * N0 * N0 * N0 +
+                       (N0 == 17 ? (size_t)TailGrid<T, N1, false>::shared_iter + (size_t)coef1 * N1 * N1 * N1 : 0);
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      k_vcycle_tail<T, N0, SPLIT, P1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (attr != cudaSuccess) return attr;
+  k_vcycle_tail<T, N0, SPLIT, P1><<<B, kTailThreads, elems * sizeof(T), st>>>(A);
+  return cudaSuccess;
+}
+
+template <typename T>
+void vcycle_tail(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
+  TailArgs<T> A{};
+  const int n = H.lv[j].n, B = H.B;
+  int coef[2] = {0, 0};
+  for (int k = 0; k < (n == 17 ? 2 : 1); ++k) {
+    const Level<T>& v = H.lv[j + k];
+    const bool nodal = sizeof(T) == 4 && (H.split || H.nodal[j + k]);
+    A.lv[k] = {v.Kx, v.Ky, v.Kz, v.D, v.Dinv, nodal ? v.kn : nullptr, v.g, v.u};
+    coef[k] = tail_coef_arrays(sizeof(T) == 4, nodal);
+  }
+  A.Ainv = H.Ainv;
+  A.active = H.active;
+  A.nu1 = nu1;
+  A.nu2 = nu2;
+  A.zero = zero ? 1 : 0;
+  const double Ba = (double)H.n_act, nodes = interior(n) * 8.0 / 7.0;
+  auto go = [&](auto n0) {
+    constexpr int N0 = decltype(n0)::value;
+    if constexpr (sizeof(T) == 8) {
+      if (H.split && H.p1) return tail_launch<T, N0, true, true>(A, B, 0, 0, st);
+      if (H.split) return tail_launch<T, N0, true, false>(A, B, 0, 0, st);
+      if (H.p1) return tail_launch<T, N0, false, true>(A, B, 0, 0, st);
+      return tail_launch<T, N0, false, false>(A, B, 0, 0, st);
+    } else {
+      if (H.split) return tail_launch<T, N0, true, false>(A, B, coef[0], coef[1], st);
+      return tail_launch<T, N0, false, false>(A, B, coef[0], coef[1], st);
+    }
+  };
+  MLMC_LAUNCH(prof::sized(sizeof(T) == 8 ? "vcycle_tail_f64" : "vcycle_tail_f32", n),
+              Ba * nodes * (nu1 + nu2) * 7.0 * (double)sizeof(T), Ba * nodes * ((nu1 + nu2) * 13.0 + 14.0), st,
+              (n == 17 ? go(std::integral_constant<int, 17>()) : go(std::integral_constant<int, 9>())));
+}
 
 // One level of the V-cycle on colour-split FP32 storage: nodal-coefficient colour passes,
 // the residual into the plain r, full weighting into the coarse grid's split g, the
@@ -2253,6 +2581,10 @@ void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
     else
       MLMC_LAUNCH(Names<T>::coarse, Ba * (729.0 * 8 + 54 * W), Ba * 27 * 54.0, st,
                   (k_coarse_apply<T><<<(B * 27 + 127) / 128, 128, 0, st>>>(B, H.Ainv, v.g, v.u, act)));
+    return;
+  }
+  if (tail_applies(H, j, nu1, nu2)) {
+    vcycle_tail(H, j, nu1, nu2, st, zero);
     return;
   }
   if (H.split) {
@@ -3077,6 +3409,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   Carver c(ws);
   layout<T>(H, c, a.B, a.n, mixed, cg);
   H.p1 = a.cfg.disc == MLMC_DISC_FE;
+  H.tail_finest = fmg && a.cfg.engine != MLMC_ENGINE_BATCHED;
   const int B = a.B;
   const double W = (double)sizeof(T);
   // the sweep count of the cycle (tuned for the finest grid, or as given) and whether the
