@@ -43,6 +43,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxLevels = 12;
 constexpr int kPlaneThreads = 128;
+constexpr int kCtaMaxN = 33;  // largest grid of the small-grid engine
 
 // Plane launches: blockIdx.x (with threadIdx.x) enumerates the work items of one z-plane,
 // blockIdx.y strides over the (sample, z) planes, so every in-sample index is 32-bit
@@ -977,12 +978,13 @@ __device__ __forceinline__ double block_sum(double v) {
 }
 
 // Blocks per sample of the deterministic reductions: a function of the grid size only
-// (never of the batch), so that a sample's sums do not depend on its batch; up to 1024
-// blocks so that one or two large samples still fill the GPU.
-inline int reduce_blocks(size_t work) {
+// (never of the batch), so that a sample's sums do not depend on its batch; up to per_sm
+// blocks for each of the 152 SMs (what is resident at once: one large sample then runs as one
+// whole wave).
+inline int reduce_blocks(size_t work, int per_sm = 8) {
   size_t nb = (work + 4095) / 4096;
   if (nb < 1) nb = 1;
-  if (nb > 1024) nb = 1024;
+  if (nb > (size_t)(152 * per_sm)) nb = 152 * per_sm;
   return (int)nb;
 }
 
@@ -1518,6 +1520,31 @@ __global__ void __launch_bounds__(kThreads) k_qoi_flux(int n, const double* __re
 // preconditioner). All vectors are FP64 on the finest grid; per-sample scalars.
 // ---------------------------------------------------------------------------------
 
+// True in every thread of the block of a sample's grid that finishes last: `total` blocks count
+// themselves in *tick, which the last one resets for the next kernel. Thread 0 has written the
+// block's partials before the call. The last block then does the per-sample scalar work, so no
+// launch of its own is needed for it.
+__device__ __forceinline__ bool last_block(int* tick, int total) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(tick, 1) == total - 1;
+    if (last) *tick = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return last != 0;
+}
+// warp_sum_partials of partials that other blocks of this launch wrote (read past the L1)
+__device__ __forceinline__ double warp_sum_fresh(const double* p, int NB) {
+  double t = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x & 31; b < NB; b += 32) t += __ldcg(p + b);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
 // q = A~ p on interior nodes (0 on the boundary): v = D p, then the six faces in the order
 // -x, +x, -y, +y, -z, +z, and partials of p.q, by column z-marches: a thread owns one
 // (x, y) column of a z-slab and carries p and Kz of the planes below and above in
@@ -1566,6 +1593,15 @@ __global__ void __launch_bounds__(128)
   }
   const double bs = block_sum<128>(acc);
   if (threadIdx.x == 0) partial[(size_t)s * nb + b] = bs;
+}
+
+// alpha = rz / p.q from k_apply_dot_z's partials, one warp per sample.
+__global__ void k_cg_alpha(int B, int NB, const double* __restrict__ part, const double* __restrict__ rz,
+                           double* __restrict__ alpha, const int* __restrict__ active) {
+  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (s >= B || !active[s]) return;
+  const double t = warp_sum_partials(part + (size_t)s * NB, NB);
+  if ((threadIdx.x & 31) == 0) alpha[s] = t != 0.0 ? rz[s] / t : 0.0;
 }
 
 // z-slabs of the column z-march kernels: a function of n only (so a sample's sums do not
@@ -1779,87 +1815,192 @@ inline dim3 zmarch_grid(int n, int B, int* zslab) {
   return dim3((unsigned)((n * n + 127) / 128), (unsigned)slabs, (unsigned)B);
 }
 
-// x += alpha p, r -= alpha q; partials of r.r and r.z (z: the previous preconditioned
-// residual); optionally r32 = (float) r for an FP32 preconditioner (SPLIT: in colour-split
-// storage). Grid (NB, B).
+// A node index that steps by the block size through a flat chunk of a sample: the index of its
+// FP32 value (plain, or SPLIT: colour-split) without a division per node.
 template <bool SPLIT>
-__global__ void __launch_bounds__(kThreads)
-    k_cg_update(int n, const double* __restrict__ alpha, const double* __restrict__ p,
-                const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                const double* __restrict__ z, float* __restrict__ r32, double* __restrict__ part_rr,
-                double* __restrict__ part_rz, const int* __restrict__ active) {
-  const int s = blockIdx.y;
-  if (!active[s]) return;
+struct FlatWalk {
+  unsigned n, dq, dr, x, y, z, ns;
+  __device__ __forceinline__ FlatWalk(int n_, unsigned i) {
+    if (!SPLIT) return;
+    n = (unsigned)n_;
+    dq = kThreads / n;
+    dr = kThreads - dq * n;
+    z = i / (n * n);
+    const unsigned rem = i - z * n * n;
+    y = rem / n;
+    x = rem - y * n;
+  }
+  __device__ __forceinline__ size_t at(unsigned i) const {
+    return SPLIT ? (size_t)split_index((int)n, (int)x, (int)y, (int)z) : (size_t)i;
+  }
+  __device__ __forceinline__ void step() {
+    if (!SPLIT) return;
+    x += dr;
+    y += dq;
+    if (x >= n) {
+      x -= n;
+      ++y;
+    }
+    while (y >= n) {
+      y -= n;
+      ++z;
+    }
+  }
+};
+
+// The preconditioned residual z of a node: the FP32 correction of the V-cycle as it lies in the
+// finest grid's iterate (MIX; SPLIT: in colour-split storage), or the FP64 one.
+template <bool MIX, bool SPLIT>
+struct PrecondZ {
+  const void* z;
+  __device__ __forceinline__ double at(int n, int s, size_t n3, unsigned i, const FlatWalk<SPLIT>& w) const {
+    if (MIX) return widen(__ldg((const float*)z + (size_t)s * (SPLIT ? split_elems(n) : n3) + w.at(i)));
+    return ((const double*)z)[(size_t)s * n3 + i];
+  }
+};
+
+// r -= alpha q; r32 = (float) r for an FP32 preconditioner; partials of r.r and r.z (z: the
+// previous preconditioned residual). The last block of a sample sums them and decides: the
+// relative residual, the cycle count, whether the sample goes on (n_active) or is done with this
+// iteration (fin, for k_cg_finish), and r.z (rzo). x is updated with p in k_p_update, which reads
+// p anyway: 32 instead of 60 bytes per node here, bound by HBM. Grid (NB, B).
+template <bool MIX, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 4)
+    k_cg_update(int n, const double* __restrict__ alpha, const double* __restrict__ q, double* __restrict__ r,
+                PrecondZ<MIX, SPLIT> z, float* __restrict__ r32, double* part_rr, double* part_rz,
+                double* __restrict__ rzo, const double* __restrict__ g2, double* __restrict__ relres,
+                int* __restrict__ cycles, int* active, int* __restrict__ fin, double rtol, int max_cycles,
+                int* __restrict__ n_active, int* tick) {
+  const int s = blockIdx.y, NB = gridDim.x;
+  if (!active[s]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) fin[s] = 0;
+    return;
+  }
   const unsigned n3 = (unsigned)n * n * n;
   const unsigned chunk = (n3 + gridDim.x - 1) / gridDim.x;
   const unsigned lo = blockIdx.x * chunk, hi = lo + chunk < n3 ? lo + chunk : n3;
   const double a = alpha[s];
   double rr = 0.0, rz = 0.0;
-  for (unsigned i = lo + threadIdx.x; i < hi; i += kThreads) {
-    const size_t t = (size_t)s * n3 + i;
-    x[t] = fma(a, p[t], x[t]);
-    const double rn = fma(-a, q[t], r[t]);  // q and p vanish on the boundary
-    r[t] = rn;
-    if (r32) {
-      if (SPLIT) {
-        const unsigned zq = i / (unsigned)(n * n), rem = i - zq * (unsigned)(n * n), yq = rem / (unsigned)n;
-        r32[(size_t)s * split_elems(n) + split_index(n, (int)(rem - yq * (unsigned)n), (int)yq, (int)zq)] = (float)rn;
-      } else {
-        r32[t] = (float)rn;
-      }
+  FlatWalk<SPLIT> w(n, lo + threadIdx.x);
+  float* f = MIX ? r32 + (size_t)s * (SPLIT ? split_elems(n) : (size_t)n3) : nullptr;
+  const double* qs = q + (size_t)s * n3;
+  double* rs = r + (size_t)s * n3;
+  // four nodes a thread at a time: all their loads before the stores
+  for (unsigned i = lo + threadIdx.x; i < hi;) {
+    double qv[4], rv[4], zv[4];
+    size_t fo[4];
+    unsigned t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k, i += kThreads) {
+      t[k] = i;
+      const bool on = i < hi;
+      fo[k] = w.at(i);
+      qv[k] = on ? qs[i] : 0.0;  // q vanishes on the boundary
+      rv[k] = on ? rs[i] : 0.0;
+      zv[k] = on ? z.at(n, s, n3, i, w) : 0.0;
+      w.step();
     }
-    rr = fma(rn, rn, rr);
-    rz = fma(rn, z[t], rz);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (t[k] >= hi) break;
+      const double rn = fma(-a, qv[k], rv[k]);
+      rs[t[k]] = rn;
+      if (MIX) f[fo[k]] = (float)rn;
+      rr = fma(rn, rn, rr);
+      rz = fma(rn, zv[k], rz);
+    }
   }
   const double b1 = block_sum<kThreads>(rr);
-  if (threadIdx.x == 0) part_rr[(size_t)s * gridDim.x + blockIdx.x] = b1;
   const double b2 = block_sum<kThreads>(rz);
-  if (threadIdx.x == 0) part_rz[(size_t)s * gridDim.x + blockIdx.x] = b2;
+  if (threadIdx.x == 0) {
+    part_rr[(size_t)s * NB + blockIdx.x] = b1;
+    part_rz[(size_t)s * NB + blockIdx.x] = b2;
+  }
+  if (last_block(tick + s, NB) && threadIdx.x < 32) {
+    const double tz = warp_sum_fresh(part_rz + (size_t)s * NB, NB);
+    const double tr = warp_sum_fresh(part_rr + (size_t)s * NB, NB);
+    if (threadIdx.x == 0) {
+      rzo[s] = tz;
+      const double rel = g2[s] > 0.0 ? sqrt(tr / g2[s]) : 0.0;
+      relres[s] = rel;
+      const int c = cycles[s] + 1;
+      cycles[s] = c;
+      const int still = (rtol > 0.0) ? (rel > rtol && c < max_cycles) : (c < max_cycles);
+      active[s] = still;
+      fin[s] = !still;
+      if (still) atomicAdd(n_active, 1);
+    }
+  }
 }
 
-// z = (double) e (when e32 is given; SPLIT: in colour-split storage) and partial sums of
-// r.z. Grid (NB, B).
-template <bool SPLIT>
-__global__ void __launch_bounds__(kThreads)
-    k_precond_dot(int n, const float* __restrict__ e32, double* __restrict__ z, const double* __restrict__ r,
-                  double* __restrict__ partial, const int* __restrict__ active) {
-  const int s = blockIdx.y;
+// r.z of the new preconditioned residual z; the last block sets beta = (r.z - r.z_old) / rz (the
+// flexible beta; not the first time) and rz = r.z. Grid (NB, B).
+template <bool MIX, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 8)
+    k_precond_dot(int n, PrecondZ<MIX, SPLIT> z, const double* __restrict__ r, double* partial, int first,
+                  const double* __restrict__ rzo, double* __restrict__ rz, double* __restrict__ beta, int* tick,
+                  const int* __restrict__ active) {
+  const int s = blockIdx.y, NB = gridDim.x;
   if (!active[s]) return;
   const unsigned n3 = (unsigned)n * n * n;
   const unsigned chunk = (n3 + gridDim.x - 1) / gridDim.x;
   const unsigned lo = blockIdx.x * chunk, hi = lo + chunk < n3 ? lo + chunk : n3;
   double acc = 0.0;
+  const double* rs = r + (size_t)s * n3;
+  FlatWalk<SPLIT> w(n, lo + threadIdx.x);
+#pragma unroll 4
   for (unsigned i = lo + threadIdx.x; i < hi; i += kThreads) {
-    const size_t t = (size_t)s * n3 + i;
-    double zv;
-    if (e32) {
-      if (SPLIT) {
-        const unsigned zq = i / (unsigned)(n * n), rem = i - zq * (unsigned)(n * n), yq = rem / (unsigned)n;
-        zv = widen(e32[(size_t)s * split_elems(n) + split_index(n, (int)(rem - yq * (unsigned)n), (int)yq, (int)zq)]);
-      } else {
-        zv = widen(e32[t]);
-      }
-      z[t] = zv;
-    } else {
-      zv = z[t];
-    }
-    acc = fma(r[t], zv, acc);
+    acc = fma(rs[i], z.at(n, s, n3, i, w), acc);
+    w.step();
   }
   const double b = block_sum<kThreads>(acc);
-  if (threadIdx.x == 0) partial[(size_t)s * gridDim.x + blockIdx.x] = b;
+  if (threadIdx.x == 0) partial[(size_t)s * NB + blockIdx.x] = b;
+  if (last_block(tick + s, NB) && threadIdx.x < 32) {
+    const double t = warp_sum_fresh(partial + (size_t)s * NB, NB);
+    if (threadIdx.x == 0) {
+      if (!first) beta[s] = rz[s] != 0.0 ? (t - rzo[s]) / rz[s] : 0.0;
+      rz[s] = t;
+    }
+  }
 }
 
-// p = z + beta p (beta = 0: p = z).
-__global__ void k_p_update(int n, int B, const double* __restrict__ beta, const double* __restrict__ z,
-                           double* __restrict__ p, const int* __restrict__ active) {
+// The iteration's x += alpha p and the next direction p = z + beta p (first: p = z alone).
+// Planes of active samples.
+template <bool MIX, bool SPLIT>
+__global__ void k_p_update(int n, int B, int first, const double* __restrict__ alpha, const double* __restrict__ beta,
+                           const void* __restrict__ z, double* __restrict__ p, double* __restrict__ x,
+                           const int* __restrict__ active) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;  // node of the plane
   if (q >= n * n) return;
+  const int y = q / n, xx = q - y * n;
   const size_t n3 = (size_t)n * n * n;
   for (int zz = blockIdx.y; zz < B * n; zz += gridDim.y) {
     const int s = zz / n, zp = zz - s * n;
     if (!active[s]) continue;
     const size_t t = (size_t)s * n3 + (size_t)(zp * n * n + q);
-    p[t] = beta ? fma(beta[s], p[t], z[t]) : z[t];
+    const double zv = MIX ? widen(((const float*)z)[SPLIT ? (size_t)s * split_elems(n) + split_index(n, xx, y, zp) : t])
+                          : ((const double*)z)[t];
+    if (first) {
+      p[t] = zv;
+    } else {
+      const double pv = p[t];
+      x[t] = fma(alpha[s], pv, x[t]);
+      p[t] = fma(beta[s], pv, zv);
+    }
+  }
+}
+
+// x += alpha p of the samples that the iteration finished.
+__global__ void k_cg_finish(int n, int B, const double* __restrict__ alpha, const double* __restrict__ p,
+                            double* __restrict__ x, const int* __restrict__ fin) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // node of the plane
+  if (q >= n * n) return;
+  const size_t n3 = (size_t)n * n * n;
+  for (int zz = blockIdx.y; zz < B * n; zz += gridDim.y) {
+    const int s = zz / n, zp = zz - s * n;
+    if (!fin[s]) continue;
+    const size_t t = (size_t)s * n3 + (size_t)(zp * n * n + q);
+    x[t] = fma(alpha[s], p[t], x[t]);
   }
 }
 
@@ -1877,30 +2018,6 @@ __global__ void k_to_f32_split(int n, int B, const double* __restrict__ a, float
   for (int zz = blockIdx.y; zz < B * n; zz += gridDim.y) {
     const int s = zz / n, z = zz - s * n;
     b[(size_t)s * ns + split_index(n, x, y, z)] = (float)a[(size_t)s * n3 + (size_t)(z * n * n + q)];
-  }
-}
-
-// Per-sample CG scalars from block partials (fixed order).
-//   mode 0: rz = sum(part)                         (after the first preconditioning)
-//   mode 1: alpha = rz / sum(part)                 (part = p.q)
-//   mode 2: beta = (sum(part) - rzo) / rz, rz = sum (part = r.z_new; flexible beta)
-//   mode 3: rzo = sum(part)                        (part = r_new.z_old)
-__global__ void k_cg_scalar(int B, int NB, int mode, const double* __restrict__ part, double* __restrict__ rz,
-                            double* __restrict__ rzo, double* __restrict__ alpha, double* __restrict__ beta,
-                            const int* __restrict__ active) {
-  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp per sample
-  if (s >= B || !active[s]) return;
-  const double t = warp_sum_partials(part + (size_t)s * NB, NB);
-  if ((threadIdx.x & 31) != 0) return;
-  if (mode == 0) {
-    rz[s] = t;
-  } else if (mode == 1) {
-    alpha[s] = t != 0.0 ? rz[s] / t : 0.0;
-  } else if (mode == 2) {
-    beta[s] = rz[s] != 0.0 ? (t - rzo[s]) / rz[s] : 0.0;
-    rz[s] = t;
-  } else {
-    rzo[s] = t;
   }
 }
 
@@ -1936,11 +2053,13 @@ struct Hier {
   int* cand = nullptr;      // candidates to stop
   int* err = nullptr;  // device error word of bounded waits
   int NB = 1;   // partials per sample of the flat-chunk reductions (reduce_blocks)
+  int NBu = 1;  // the same for k_cg_update (four blocks per SM)
   int NBz = 1;  // partials per sample of the column z-march kernels (apply_blocks)
   // flexible PCG (FP64 vectors on the finest grid) and per-sample scalars
   double *R = nullptr, *P = nullptr, *Q = nullptr, *Z = nullptr;
   double *part2 = nullptr, *rz = nullptr, *rzo = nullptr, *alpha = nullptr, *beta = nullptr;
   double* part_apply = nullptr;  // partials of p.q (k_apply_dot_z's partition)
+  int* tick = nullptr;           // blocks of a sample that have finished (last_block)
   int tile[kMaxLevels] = {};      // fused-sweep tile shape per level
   bool fused[kMaxLevels] = {};    // fused (one pass) or two-pass smoother per level
   bool nodal[kMaxLevels] = {};    // two-pass sweep on the nodal coefficient (FP32)
@@ -1991,6 +2110,7 @@ void layout(Hier<T>& H, Carver& c, int B, int n, bool mixed, bool cg) {
   }
   H.Ainv = c.template take<double>((size_t)B * 729);
   H.NB = reduce_blocks(cube(n));
+  H.NBu = reduce_blocks(cube(n), 4);
   H.NBz = apply_blocks(n);
   H.partial = c.template take<double>((size_t)B * (H.NB > H.NBz ? H.NB : H.NBz));
   H.g2 = c.template take<double>(B);
@@ -2004,7 +2124,8 @@ void layout(Hier<T>& H, Carver& c, int B, int n, bool mixed, bool cg) {
     H.R = c.template take<double>(e0);
     H.P = c.template take<double>(e0);
     H.Q = c.template take<double>(e0);
-    if (mixed) H.Z = c.template take<double>(e0);
+    if (mixed && n <= kCtaMaxN) H.Z = c.template take<double>(e0);  // the small-grid engine's
+    H.tick = c.template take<int>(B);
     H.part2 = c.template take<double>((size_t)B * H.NB);
     H.part_apply = c.template take<double>((size_t)B * apply_blocks(n));
     H.rz = c.template take<double>(B);
@@ -2738,23 +2859,61 @@ struct GraphRunner {
   }
 };
 
-template <typename T>
+// The vector kernels of flexible CG on the finest grid, FP64, with the V-cycle's result z read
+// where the cycle left it (MIX: FP32, SPLIT: in colour-split storage).
+template <typename T, bool SPLIT>
+struct CgVectors {
+  static constexpr bool MIX = sizeof(T) == 4;
+  const Hier<T>& H;
+  double* x;
+  cudaStream_t st;
+  double rtol;
+  int maxc;
+  int n() const { return H.lv[0].n; }
+  const void* z() const { return H.lv[0].u; }
+  double all() const { return (double)H.n_act * H.lv[0].n3; }
+  dim3 planes() const { return plane_grid(n() * n(), (long long)H.B * n()); }
+  void update() const {
+    MLMC_LAUNCH("cg_update", all() * (MIX ? 32.0 : 32.0), all() * 6.0, st,
+                (k_cg_update<MIX, SPLIT><<<dim3(H.NBu, H.B), kThreads, 0, st>>>(
+                    n(), H.alpha, H.Q, H.R, PrecondZ<MIX, SPLIT>{z()}, MIX ? (float*)(void*)H.lv[0].g : nullptr,
+                    H.partial, H.part2, H.rzo, H.g2, H.relres, H.cycles, H.active, H.cand, rtol, maxc, H.n_active,
+                    H.tick)));
+  }
+  void dot(bool first) const {
+    MLMC_LAUNCH("cg_precond_dot", all() * (MIX ? 12.0 : 16.0), all() * 2.0, st,
+                (k_precond_dot<MIX, SPLIT><<<dim3(H.NB, H.B), kThreads, 0, st>>>(
+                    n(), PrecondZ<MIX, SPLIT>{z()}, H.R, H.partial, first ? 1 : 0, H.rzo, H.rz, H.beta, H.tick,
+                    H.active)));
+  }
+  void direction(bool first) const {
+    MLMC_LAUNCH("cg_p_update", all() * (first ? 12.0 : (MIX ? 36.0 : 40.0)), all() * (first ? 0.0 : 4.0), st,
+                (k_p_update<MIX, SPLIT><<<planes(), kPlaneThreads, 0, st>>>(n(), H.B, first ? 1 : 0, H.alpha, H.beta,
+                                                                           z(), H.P, x, H.active)));
+  }
+  void finish(int count) const {
+    MLMC_LAUNCH("cg_finish", (double)count * H.lv[0].n3 * 24.0, (double)count * H.lv[0].n3 * 2.0, st,
+                (k_cg_finish<<<planes(), kPlaneThreads, 0, st>>>(n(), H.B, H.alpha, H.P, x, H.cand)));
+  }
+};
+
+// Flexible preconditioned CG: per iteration one operator application with p.q, one residual
+// update with r.r and r.z, the V-cycle, one dot product r.z, one update of x and p: 128 bytes and
+// 14 FP64 operations per node in mixed precision (an FP64 copy of z, and x updated beside r, made
+// it 152), one launch for the scalars (last_block does the others). The FP64 pipe bounds the
+// application (1.07 of the 1.06 TFLOP/s the FMA probe reaches at 257^3), HBM p's and x's update
+// (5.7 TB/s); r's update, 32 bytes and three FP64 operations per node, is bound by neither alone.
+// Per iteration at 257^3: 663 us of vector kernels and three of scalars -> 560. The mixed 257^3
+// solve 24.3 -> 22.1 ms, the 257^3 / 129^3 level of two 41.0 -> 39.0.
+template <typename T, bool SPLIT>
 int pcg_loop(Hier<T>& H, const MGSolveArgs& a, int nu1, int nu2, double rtol, int maxc, cudaStream_t st,
              GraphRunner<T>& gr) {
   const bool mixed = a.cfg.precision == MLMC_PREC_MIXED;
   const int B = H.B, n = a.n;
   Level<T>& l0 = H.lv[0];
-  // algorithmic work of the active samples (H.n_act, updated after every convergence test)
-  double nodes = H.n_act * interior(n), all = (double)H.n_act * l0.n3;
-  auto set_active = [&](int na) {
-    H.n_act = na;
-    nodes = na * interior(n);
-    all = (double)na * l0.n3;
-  };
-  dim3 rg(H.NB, B);
+  const CgVectors<T, SPLIT> V{H, a.u, st, rtol, maxc};
   const unsigned sb = (B + 3) / 4;  // 128-thread blocks, one warp per sample
   const unsigned g0 = blocks_for((size_t)B * l0.n3, kThreads);
-  const dim3 pg = plane_grid(n * n, (long long)B * n);
   int azslab = 0;
   const int aslabs = apply_slabs(n, &azslab), NBa = apply_blocks(n);
   const dim3 ag((unsigned)((n * n + 127) / 128), (unsigned)aslabs, (unsigned)B);
@@ -2768,22 +2927,14 @@ int pcg_loop(Hier<T>& H, const MGSolveArgs& a, int nu1, int nu2, double rtol, in
     MLMC_CUDA_TRY(cudaStreamSynchronize(st));
     return MLMC_OK;
   };
-  // z = M r: one V-cycle from zero on the (FP32 copy of the) residual; partials of r.z
-  auto precondition = [&]() {
+  // z = M r: one V-cycle from zero on the (FP32 copy of the) residual
+  auto precondition = [&]() -> int {
     MLMC_CUDA_TRY(clear_guess(H, 0, nu1, st));
-    MLMC_TRY(gr.run(H, nu1, nu2, st, true));
-    double* z = mixed ? H.Z : (double*)(void*)H.lv[0].u;
-    const float* e32 = mixed ? (const float*)(const void*)H.lv[0].u : nullptr;
-    if (H.split)
-      MLMC_LAUNCH("cg_precond_dot", all * 20.0, nodes * 2.0, st,
-                  (k_precond_dot<true><<<rg, kThreads, 0, st>>>(n, e32, z, H.R, H.partial, H.active)));
-    else
-      MLMC_LAUNCH("cg_precond_dot", all * (mixed ? 20.0 : 16.0), nodes * 2.0, st,
-                  (k_precond_dot<false><<<rg, kThreads, 0, st>>>(n, e32, z, H.R, H.partial, H.active)));
-    return MLMC_OK;
+    return gr.run(H, nu1, nu2, st, true);
   };
-  auto zcur = [&]() -> double* { return mixed ? H.Z : (double*)(void*)H.lv[0].u; };
   // r = g - A x, ||r||
+  double nodes = H.n_act * interior(n);
+  MLMC_CUDA_TRY(cudaMemsetAsync(H.tick, 0, B * sizeof(int), st));
   MLMC_CUDA_TRY(cudaMemsetAsync(H.n_active, 0, sizeof(int), st));
   MLMC_LAUNCH("cg_residual", nodes * (3 * 8.0 + 32), nodes * 16.0, st,
               (k_residual_z<double, double, double, double><<<ag, 128, 0, st>>>(n, azslab, Fx, Fy, Fz, D, H.g64,
@@ -2791,50 +2942,35 @@ int pcg_loop(Hier<T>& H, const MGSolveArgs& a, int nu1, int nu2, double rtol, in
   MLMC_LAUNCH("norm_update", B * NBa * 8.0, B * NBa * 1.0, st,
               (k_norm_update<<<sb, 128, 0, st>>>(B, NBa, H.partial, H.g2, H.relres, H.cycles, H.active, 1, 0, rtol,
                                                  maxc, H.n_active)));
-  int na = 0;
-  MLMC_TRY(sync_count(&na));
-  set_active(na);
-  if (na == 0) return MLMC_OK;
-  if (mixed && H.split)
-    MLMC_LAUNCH("to_f32", all * 12.0, 0.0, st,
-                (k_to_f32_split<<<pg, kPlaneThreads, 0, st>>>(n, B, H.R, (float*)(void*)l0.g)));
+  MLMC_TRY(sync_count(&H.n_act));
+  if (H.n_act == 0) return MLMC_OK;
+  if (mixed && SPLIT)
+    MLMC_LAUNCH("to_f32", V.all() * 12.0, 0.0, st,
+                (k_to_f32_split<<<V.planes(), kPlaneThreads, 0, st>>>(n, B, H.R, (float*)(void*)l0.g)));
   else if (mixed)
-    MLMC_LAUNCH("to_f32", all * 12.0, 0.0, st,
+    MLMC_LAUNCH("to_f32", V.all() * 12.0, 0.0, st,
                 (k_to_f32<<<g0, kThreads, 0, st>>>((size_t)B * l0.n3, H.R, (float*)(void*)l0.g)));
   MLMC_TRY(precondition());
-  MLMC_LAUNCH("cg_scalar", B * H.NB * 8.0, 0.0, st,
-              (k_cg_scalar<<<sb, 128, 0, st>>>(B, H.NB, 0, H.partial, H.rz, H.rzo, H.alpha, H.beta, H.active)));
-  MLMC_LAUNCH("cg_p_update", all * 16.0, 0.0, st,
-              (k_p_update<<<pg, kPlaneThreads, 0, st>>>(n, B, nullptr, zcur(), H.P, H.active)));
+  V.dot(true);
+  V.direction(true);
   while (true) {
-    MLMC_LAUNCH("cg_apply_dot", nodes * (3 * 8.0 + 8 + 16), nodes * 16.0, st,
-                (k_apply_dot_z<double, double><<<ag, 128, 0, st>>>(n, azslab, Fx, Fy, Fz, D, H.P, H.Q,
-                                                                    H.part_apply, H.active)));
+    nodes = H.n_act * interior(n);
+    MLMC_LAUNCH("cg_apply_dot", nodes * 48.0, nodes * 16.0, st,
+                (k_apply_dot_z<double, double><<<ag, 128, 0, st>>>(n, azslab, Fx, Fy, Fz, D, H.P, H.Q, H.part_apply,
+                                                                    H.active)));
     MLMC_LAUNCH("cg_scalar", B * NBa * 8.0, 0.0, st,
-                (k_cg_scalar<<<sb, 128, 0, st>>>(B, NBa, 1, H.part_apply, H.rz, H.rzo, H.alpha, H.beta, H.active)));
-    if (H.split)
-      MLMC_LAUNCH("cg_update", all * 60.0, nodes * 8.0, st,
-                  (k_cg_update<true><<<rg, kThreads, 0, st>>>(n, H.alpha, H.P, H.Q, a.u, H.R, zcur(),
-                                                              (float*)(void*)l0.g, H.partial, H.part2, H.active)));
-    else
-      MLMC_LAUNCH("cg_update", all * (mixed ? 60.0 : 56.0), nodes * 8.0, st,
-                  (k_cg_update<false><<<rg, kThreads, 0, st>>>(n, H.alpha, H.P, H.Q, a.u, H.R, zcur(),
-                                                               mixed ? (float*)(void*)l0.g : nullptr, H.partial,
-                                                               H.part2, H.active)));
-    MLMC_LAUNCH("cg_scalar", B * H.NB * 8.0, 0.0, st,
-                (k_cg_scalar<<<sb, 128, 0, st>>>(B, H.NB, 3, H.part2, H.rz, H.rzo, H.alpha, H.beta, H.active)));
+                (k_cg_alpha<<<sb, 128, 0, st>>>(B, NBa, H.part_apply, H.rz, H.alpha, H.active)));
     MLMC_CUDA_TRY(cudaMemsetAsync(H.n_active, 0, sizeof(int), st));
-    MLMC_LAUNCH("norm_update", B * H.NB * 8.0, B * H.NB * 1.0, st,
-                (k_norm_update<<<sb, 128, 0, st>>>(B, H.NB, H.partial, H.g2, H.relres, H.cycles, H.active, 1, 1,
-                                                   rtol, maxc, H.n_active)));
+    V.update();
+    int na = 0;
     MLMC_TRY(sync_count(&na));
-    set_active(na);
+    const int done = H.n_act - na;
+    H.n_act = na;
+    if (done > 0) V.finish(done);
     if (na == 0) break;
     MLMC_TRY(precondition());
-    MLMC_LAUNCH("cg_scalar", B * H.NB * 8.0, 0.0, st,
-                (k_cg_scalar<<<sb, 128, 0, st>>>(B, H.NB, 2, H.partial, H.rz, H.rzo, H.alpha, H.beta, H.active)));
-    MLMC_LAUNCH("cg_p_update", all * 24.0, nodes * 2.0, st,
-                (k_p_update<<<pg, kPlaneThreads, 0, st>>>(n, B, H.beta, zcur(), H.P, H.active)));
+    V.dot(false);
+    V.direction(false);
   }
   return MLMC_OK;
 }
@@ -2851,7 +2987,6 @@ int pcg_loop(Hier<T>& H, const MGSolveArgs& a, int nu1, int nu2, double rtol, in
 // path.
 // ---------------------------------------------------------------------------------
 constexpr int kCtaThreads = 256;
-constexpr int kCtaMaxN = 33;
 
 // MLMC_ENGINE_CTA where it applies (finite volumes, stationary cycles, refinement or CG,
 // grids up to 33^3); MLMC_ENGINE_AUTO takes it for grids up to 17^3 (measured 1.15-1.4x
@@ -3693,7 +3828,8 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     MLMC_CUDA_TRY(cudaGetLastError());
   }
   if (cg && !use_cta) {
-    const int st_pcg = pcg_loop<T>(H, a, nu1, nu2, rtol, maxc, st, gr);
+    const int st_pcg = H.split ? pcg_loop<T, true>(H, a, nu1, nu2, rtol, maxc, st, gr)
+                               : pcg_loop<T, false>(H, a, nu1, nu2, rtol, maxc, st, gr);
     if (st_pcg < 0) return st_pcg;
   }
   if (fmg) {
