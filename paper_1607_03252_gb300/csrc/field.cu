@@ -13,6 +13,7 @@
 
 #include <atomic>
 #include <cstdlib>
+#include <type_traits>
 
 #include "bulk.cuh"
 #include "common.cuh"
@@ -746,20 +747,32 @@ int field_tc_dispatch(const float4* xsplit, const float4* pt, const uint4* Xf, c
   return field_tc_launch<TOut, 1, FACE>(xsplit, pt, Xf, e2tab, M, n, KS, B, scale, kout, bytes, flops, st, share);
 }
 
-// The volume product on the fifth-generation tensor cores (grids from n = 65): one block
-// computes 128 lines by 64 x-values with tcgen05.mma (M = 128, N = 64, K = 16, bf16 operands
-// from shared memory, FP32 accumulators in tensor memory: the seven slice groups take 7 x 64
-// of the 512 columns). The A operand (the line factors' slices) is staged by all 256 threads
-// into K-major core matrices; the B operand (the x-phasors' slices, the same for every line
-// of a sample) is laid out in that form once per sample (k_uxslices) and brought in by one
-// bulk copy per chunk. Chunks of two k-steps are double-buffered: one thread issues the 56
-// products of a chunk and commits them to the buffer's mbarrier while the block stages the
-// next chunk, so the staging's FP32 work runs under the tensor cores' work. Every 256
-// features (and at the end) the group sums are read from tensor memory and folded into a
-// double-float; the next product overwrites them. Every wait is bounded: a block whose wait
-// runs out records *err, drains its copies and products, writes NaN to its nodes and frees
-// its tensor memory.
-constexpr int kUmM = 128, kUmN = 64, kUmKC = 2;
+// The volume and the face x = n - 1 on the fifth-generation tensor cores: one block computes 128
+// lines by N x-values (N = 64, or n - 1 on the 17^3 and 33^3 grids) with tcgen05.mma (M = 128,
+// K = 16, bf16 operands from shared memory, FP32 accumulators in tensor memory: the seven slice
+// groups take 7 N of the 512 columns). The A operand (the line factors' slices) is staged by SW
+// warps into K-major core matrices; the B operand (the x-phasors' slices, the same for every line
+// of a sample) is laid out in that form once per sample (k_uxslices) and brought in by one bulk
+// copy per k-step. The face is further line tiles of the same launch: rows z, factors X_m[n - 1]
+// Z_m[z], the y-phasors' slices for B.
+//
+// The staging (about 190 FP32 and integer instructions per line and feature) is what bounds the
+// kernel, so it must not stop: NS k-steps are in flight, each a stage with two mbarriers. A
+// staging warp waits for the products of the stage's last use (empty), writes its share, and
+// arrives (full); one thread of the last warp waits for full and for the bulk copy, issues the
+// products and commits them to empty. Staging warps never wait for each other. A slice of A times
+// all slices of B that it meets is one product of up to 256 columns (10 per k-step instead of 28
+// of 64 columns, which read A from shared memory 28 times and took 3300 clocks a k-step, more than
+// the staging). Volume and face, 129^3 x 8 (M = 256): 1042 us with a block barrier per two k-steps
+// and 28 products, 818 without the barrier, 631 now; 65^3 x 5 (M = 1024) 747 -> 340. Below 65^3 a
+// block is small enough for three (N = 16) or two (N = 32) per SM; the warp-level mma.sync form
+// ran there with 8 warps per SM: 17^3 x 4096 6.7 -> 2.5 ms, 33^3 x 103 494 -> 193 us.
+//
+// Every 256 features (and at the end) the group sums are read from tensor memory and folded into
+// a double-float; the next product overwrites them. Every wait is bounded: a block whose wait
+// runs out records *err, drains its copies and products, writes NaN to its nodes and frees its
+// tensor memory.
+constexpr int kUmM = 128;
 
 // Set to 1 by a tensor-core field block whose bounded wait ran out (field_wait_error_take).
 __device__ int g_field_wait_err = 0;
@@ -779,29 +792,50 @@ int field_wait_error_take(cudaStream_t st) {
   }
   return v;
 }
-constexpr unsigned kUmCols = 512;
-constexpr int kUmATile = kUmM * 32, kUmBTile = kUmN * 32;  // bytes of one (k-step, slice) tile
-constexpr int kUmAChunk = kUmKC * kTcSlices * kUmATile, kUmBChunk = kUmKC * kTcSlices * kUmBTile;
-constexpr int kUmStage = kUmAChunk + kUmBChunk;
-constexpr size_t kUmSmem = 2 * (size_t)kUmStage + 128 + kUmM * sizeof(int2) + 64 * sizeof(float) + 64;
+constexpr int kUmATile = kUmM * 32;  // bytes of one (k-step, slice) tile of A
+// Block shape by x-values per block: staging warps, stages in flight, blocks per SM.
+template <int N>
+struct UmShape {
+  static constexpr int SW = N == 64 ? 16 : 8, NS = N == 64 ? 4 : (N == 32 ? 3 : 2), BPS = N == 64 ? 1 : (N == 32 ? 2 : 3);
+  static constexpr int threads = 32 * (SW + 1);
+  static constexpr int XW = N / (SW / 4);  // x-values of a thread
+  static constexpr unsigned cols = N == 64 ? 512 : (N == 32 ? 256 : 128);
+  static constexpr int a_stage = kTcSlices * kUmATile, b_stage = kTcSlices * N * 32, stage = a_stage + b_stage;
+  static constexpr size_t smem = (size_t)NS * stage + 128 + kUmM * sizeof(int2) + 64 * sizeof(float) + 128;
+};
 
-static bool umma_applies(int n) { return n >= 65 && (n - 1) % kUmN == 0; }
-
-size_t tc_uxslice_bytes(int B, int M, int n) {
-  return umma_applies(n) ? (size_t)B * ((n - 1) / kUmN) * ((M + 7) / 8) * kTcSlices * kUmBTile : 0;
+// x-values per block of the tcgen05 form on grid n, 0 where it does not apply.
+static int umma_n(int n) {
+  if (n < 17 || (n - 1) % 16 != 0) return 0;
+  return (n - 1) % 64 == 0 ? 64 : ((n - 1) % 32 == 0 ? 32 : 16);
 }
 
-// XU[s][x block][k-step][slice]: 64 x-rows by 16 k in K-major core matrices, (Re X, -Im X) of
-// feature 8 ks + fl at k = 2 fl, 2 fl + 1. One thread per (sample, x block, k-step, x, feature).
-__global__ void k_uxslices(const float4* __restrict__ xsplit, int B, int M, int n, int KS,
-                           unsigned char* __restrict__ XU) {
-  const int XB = (n - 1) / kUmN;
-  const size_t total = (size_t)B * XB * KS * kUmN * 8;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+// bytes of the slices of one axis
+size_t tc_uxslice_bytes(int B, int M, int n) {
+  return umma_n(n) ? (size_t)B * ((n - 1) / umma_n(n)) * ((M + 7) / 8) * kTcSlices * umma_n(n) * 32 : 0;
+}
+
+// XU[axis][s][block][k-step][slice], axis 0 (x) and 1 (y): N rows by 16 k in K-major core
+// matrices, (Re X, -Im X) of feature 8 ks + fl at k = 2 fl, 2 fl + 1. One thread per (axis, sample,
+// block, k-step, row, feature). Threads 0..31 also write 2^(j/32) as double-floats (e2tab[j],
+// e2tab[32 + j]) for the exp.
+__global__ void k_uxslices(const float4* __restrict__ xsplit, int B, int M, int n, int N, int KS,
+                           unsigned char* __restrict__ XU, float* __restrict__ e2tab) {
+  const int XB = (n - 1) / N, tile = N * 32;
+  const size_t per_axis = (size_t)B * XB * KS * N * 8;
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t0 < 32) {
+    const double v = exp2((double)t0 / 32.0);
+    const float h = narrow(v);
+    e2tab[t0] = h;
+    e2tab[32 + t0] = narrow(v - widen(h));
+  }
+  for (size_t t = t0; t < 2 * per_axis; t += (size_t)gridDim.x * blockDim.x) {
+    const int axis = t < per_axis ? 0 : 1;
     const int fl = (int)(t & 7);
-    size_t r = t >> 3;
-    const int xr = (int)(r % kUmN);
-    r /= kUmN;
+    size_t r = (t - axis * per_axis) >> 3;
+    const int xr = (int)(r % N);
+    r /= N;
     const int ks = (int)(r % KS);
     r /= KS;
     const int xb = (int)(r % XB);
@@ -809,252 +843,261 @@ __global__ void k_uxslices(const float4* __restrict__ xsplit, int B, int M, int 
     const int f = ks * 8 + fl;
     float re[kTcSlices], im[kTcSlices];
     if (f < M) {
-      const float4 v = xsplit[((size_t)s * 3 * M + f) * n + xb * kUmN + xr];
+      const float4 v = xsplit[(((size_t)s * 3 + axis) * M + f) * n + xb * N + xr];
       df::slice7(v.x, v.y, re);
       df::slice7(-v.z, -v.w, im);
     } else {
 #pragma unroll
       for (int i = 0; i < kTcSlices; ++i) re[i] = im[i] = 0.f;
     }
-    unsigned char* o = XU + (((size_t)(s * XB + xb) * KS + ks) * kTcSlices) * kUmBTile + umma::pair_offset(xr, fl);
+    unsigned char* o =
+        XU + ((((size_t)axis * B + s) * XB + xb) * KS + ks) * kTcSlices * tile + umma::pair_offset(xr, fl);
 #pragma unroll
-    for (int i = 0; i < kTcSlices; ++i)
-      *reinterpret_cast<uint32_t*>(o + (size_t)i * kUmBTile) = pack_bf16x2(re[i], im[i]);
+    for (int i = 0; i < kTcSlices; ++i) *reinterpret_cast<uint32_t*>(o + (size_t)i * tile) = pack_bf16x2(re[i], im[i]);
   }
 }
 
-template <typename TOut, bool MULTI, int SW>
-__global__ void __launch_bounds__(32 * (SW + 1), 1) k_field_umma(const float4* __restrict__ tsplit,
-                                                               const unsigned char* __restrict__ XU,
-                                                               const float* __restrict__ e2tab, int M, int n, int KS,
-                                                               double scale, long long budget, int inject, int* err,
-                                                               TOut* __restrict__ kout) {
+// Grid (x-blocks, volume line tiles then face line tiles, samples).
+template <typename TOut, int N, bool MULTI>
+__global__ void __launch_bounds__(UmShape<N>::threads, UmShape<N>::BPS)
+    k_field_umma(const float4* __restrict__ tsplit, const unsigned char* __restrict__ XU,
+                 const float* __restrict__ e2tab, int M, int n, int KS, double scale, long long budget, int inject,
+                 int* err, TOut* __restrict__ kout) {
+  using S = UmShape<N>;
+  constexpr int NS = S::NS, SW = S::SW, XW = S::XW;
+  constexpr int kFoldSteps = kTcFold / 8;  // k-steps per exact group sum
   extern __shared__ unsigned char um_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)um_raw + 127) & ~(uintptr_t)127);
-  int2* sline = reinterpret_cast<int2*>(sm + 2 * kUmStage);  // (y, z) of line slot l, y = -1: none
+  int2* sline = reinterpret_cast<int2*>(sm + (size_t)NS * S::stage);  // table offsets of line slot l's two factors
   float* se2 = reinterpret_cast<float*>(sline + kUmM);
-  uint64_t* bfull = reinterpret_cast<uint64_t*>(se2 + 64);  // [2]: B chunk landed
-  uint64_t* mdone = bfull + 2;                               // [2]: the chunk's products done
-  uint64_t* never = mdone + 2;                               // fault injection: nothing arrives
+  uint64_t* full = reinterpret_cast<uint64_t*>(se2 + 64);  // [NS]: A staged
+  uint64_t* bfull = full + NS;                              // [NS]: B landed
+  uint64_t* empty = bfull + NS;                             // [NS]: the stage's products done
+  uint64_t* accf = empty + NS;                              // the group sums of a fold period complete
+  uint64_t* acce = accf + 1;                                // they have been read
+  uint64_t* never = acce + 1;                               // fault injection: nothing arrives
   uint32_t* tslot = reinterpret_cast<uint32_t*>(never + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int s = blockIdx.z, xb = blockIdx.x, XB = (n - 1) / kUmN;
-  const size_t n2 = (size_t)n * n, L0 = (size_t)blockIdx.y * kUmM;
-  if (tid < kUmM) {
-    const size_t line = L0 + tid;
-    sline[tid] = line < n2 ? make_int2((int)(line % n), (int)(line / n)) : make_int2(-1, 0);
+  const int s = blockIdx.z, xb = blockIdx.x, XB = (n - 1) / N;
+  const size_t n2 = (size_t)n * n;
+  const int vtiles = (int)((n2 + kUmM - 1) / kUmM);
+  const bool face = (int)blockIdx.y >= vtiles;
+  const size_t L0 = (size_t)(face ? (int)blockIdx.y - vtiles : (int)blockIdx.y) * kUmM;
+  const size_t nlines = face ? (size_t)n : n2;
+  const int nvalid = (int)(nlines - L0 < (size_t)kUmM ? nlines - L0 : (size_t)kUmM);
+  if (tid < kUmM) {  // line l = (z, y) of the volume: Y_m[y], Z_m[z]; line z of the face: X_m[n - 1], Z_m[z]
+    const size_t line = tid < nvalid ? L0 + tid : L0;
+    const int y = (int)(line % n), z = (int)(face ? line : line / n);
+    sline[tid] = make_int2(face ? n - 1 : M * n + y, 2 * M * n + z);
   }
   if (tid < 64) se2[tid] = e2tab[tid];
   if (tid == 0) {
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < NS; ++q) {
+      mbar_init(&full[q], SW);
       mbar_init(&bfull[q], 1);
-      mbar_init(&mdone[q], 1);
+      mbar_init(&empty[q], 1);
     }
+    mbar_init(accf, 1);
+    mbar_init(acce, SW);
     mbar_init(never, 1);
     mbar_fence_init();
   }
-  if (warp == 0) umma::alloc(tslot, kUmCols);
+  if (warp == 0) umma::alloc(tslot, S::cols);
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
   const uint32_t tmem = *tslot;
-  const float4* Ty = tsplit + ((size_t)s * 3 + 1) * M * n;
-  const float4* Tz = Ty + (size_t)M * n;
-  const unsigned char* xu = XU + ((size_t)(s * XB + xb) * KS) * kTcSlices * kUmBTile;
-  const uint32_t idesc = umma::idesc_bf16_f32(kUmM, kUmN);
-  const int nchunks = (KS + kUmKC - 1) / kUmKC;
-  // the thread's outputs: tensor-memory lane 32 (warp % 4) + lane, XW x-values from XW (warp / 4)
-  // SW staging warps (they also read the accumulators out) and one issuing warp, warp SW
-  constexpr int STAGERS = 32 * SW;
-  const bool stager = warp < SW;
-  const int issuer = STAGERS;  // the thread that issues the copies and the products
-  constexpr int XW = kUmN / (SW / 4);
+  const float4* tab = tsplit + (size_t)s * 3 * M * n;
+  const unsigned char* xu =
+      XU + ((((size_t)(face ? gridDim.z : 0) + s) * XB + xb) * (size_t)KS) * kTcSlices * (N * 32);
   const int myl = 32 * (warp & 3) + lane, xh = XW * (warp >> 2);
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)xh;
-  // MULTI (more than 256 features): the double-float running sums of the folds
-  float th[MULTI ? XW : 1], tl[MULTI ? XW : 1];
-#pragma unroll
-  for (int q = 0; q < (MULTI ? XW : 1); ++q) th[q] = tl[q] = 0.f;
-  int last_commit = -1, last_copy = -1;  // (thread 0's) the last chunk whose products / copy were issued
-  bool bad = false;                       // a bounded wait of this thread ran out
-  auto wait = [&](uint64_t* mb, int chunk, long long bud) {
-    if (!mbar_wait_bounded(mb, (unsigned)((chunk >> 1) & 1), bud)) {
+  bool bad = false;  // a bounded wait of this thread ran out
+  auto wait = [&](uint64_t* mb, int use, long long bud) {  // the use-th completion of the barrier
+    if (!mbar_wait_bounded(mb, (unsigned)(use & 1), bud)) {
       bad = true;
       atomicExch(err, 1);
     }
+    return !bad;
   };
-  const float sch = narrow(scale), scl = narrow(scale - widen(sch));
-  const size_t myline = L0 + myl;
-  TOut* out = kout + (size_t)s * n2 * n + myline * n + xb * kUmN + xh;
-  // the groups' current sums of the thread's 32 x-values: folded into (th, tl) (last = false)
-  // or, with the earlier folds, turned into k and stored (last = true)
-  auto fold = [&](bool last) {
+  if (warp < SW) {
+    // MULTI (more than 256 features): the double-float running sums of the folds
+    float th[MULTI ? XW : 1], tl[MULTI ? XW : 1];
 #pragma unroll
-    for (int c0 = 0; c0 < XW; c0 += 8) {
-      float v[kTcSlices][8];
+    for (int q = 0; q < (MULTI ? XW : 1); ++q) th[q] = tl[q] = 0.f;
+    const float sch = narrow(scale), scl = narrow(scale - widen(sch));
+    const bool mine = myl < nvalid;
+    TOut* const out = kout + (size_t)s * n2 * n;
+    auto wait_warp = [&](uint64_t* mb, int use) {  // one outcome for the whole warp
+      wait(mb, use, budget);
+      bad = __any_sync(0xffffffffu, bad);
+      return !bad;
+    };
+    // the groups' sums of the thread's x-values: folded into (th, tl) (last = false) or, with
+    // the earlier folds, turned into k and stored (last = true)
+    auto fold = [&](bool last) {
+      if (32 * (warp & 3) >= nvalid) return;  // no line of this warp exists
 #pragma unroll
-      for (int g = 0; g < kTcSlices; ++g) umma::ld8(trow + (uint32_t)(g * kUmN + c0), v[g]);
+      for (int c0 = 0; c0 < XW; c0 += 8) {
+        float v[kTcSlices][8];
+        __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        float gs[kTcSlices], sh, sl;
+        for (int g = 0; g < kTcSlices; ++g) umma::ld8(trow + (uint32_t)(g * N + c0), v[g]);
 #pragma unroll
-        for (int g = 0; g < kTcSlices; ++g) gs[g] = v[g][q];
-        df::sum7(gs, sh, sl);
-        if (MULTI) df::add(th[c0 + q], tl[c0 + q], sh, sl, sh, sl);
-        if (!last) {
-          if (MULTI) {
-            th[c0 + q] = sh;
-            tl[c0 + q] = sl;
+        for (int q = 0; q < 8; ++q) {
+          float gs[kTcSlices], sh, sl;
+#pragma unroll
+          for (int g = 0; g < kTcSlices; ++g) gs[g] = v[g][q];
+          df::sum7(gs, sh, sl);
+          if (MULTI) df::add(th[c0 + q], tl[c0 + q], sh, sl, sh, sl);
+          if (!last) {
+            if (MULTI) {
+              th[c0 + q] = sh;
+              tl[c0 + q] = sl;
+            }
+            continue;
           }
-          continue;
-        }
-        if (myline >= n2) continue;
-        float yh, yl, eh, el;
-        int m;
-        df::mul(sh, sl, sch, scl, yh, yl);
-        df::exp_df(yh, yl, se2, se2 + 32, eh, el, m);
-        if constexpr (sizeof(TOut) == 8)
-          out[c0 + q] = (widen(eh) + widen(el)) * __hiloint2double((m + 1023) << 20, 0);
-        else
-          out[c0 + q] = (m > -126 && m < 128) ? __fmul_rn(eh, __int_as_float((m + 127) << 23)) : ldexpf(eh, m);
-      }
-    }
-  };
-  // (thread 0) the bulk copy of chunk cc's x-slices into its buffer
-  auto issue_copy = [&](int cc) {
-    const int k0 = cc * kUmKC, kk = min(kUmKC, KS - k0);
-    const unsigned bytes = (unsigned)(kk * kTcSlices * kUmBTile);
-    mbar_arrive_expect_tx(&bfull[cc & 1], bytes);
-    bulk_g2s(sm + (size_t)(cc & 1) * kUmStage + kUmAChunk, xu + (size_t)k0 * kTcSlices * kUmBTile, bytes,
-             &bfull[cc & 1]);
-    last_copy = cc;
-  };
-  if (tid == issuer) {
-    issue_copy(0);
-    if (inject) wait(never, 0, budget);  // injected failure: runs out after the budget
-  }
-  for (int c = 0; c < nchunks; ++c) {
-    const int b = c & 1;
-    const int ks0 = c * kUmKC, kn = min(kUmKC, KS - ks0);
-    unsigned char* sA = sm + (size_t)b * kUmStage;
-    unsigned char* sB = sA + kUmAChunk;
-    // the buffer is free once the products of chunk c - 2 are done
-    if (c >= 2) wait(&mdone[b], c - 2, budget);
-    umma::fence_after_sync();
-    // staging: 2048 / STAGERS (line, feature) items per staging thread, their table loads
-    // issued four at a time
-#pragma unroll 1
-    for (int h = 0; h < 2048 / STAGERS / 4 && stager && !bad; ++h) {
-      float4 bq[4], dq[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int it = tid + (4 * h + r) * STAGERS;
-        const int fl4 = it & 3, rr = (it >> 2) & 7, kg = (it >> 5) & 1, rg = (it >> 6) & 15, ksl = it >> 10;
-        const int f = (ks0 + ksl) * 8 + kg * 4 + fl4;
-        const int2 yz = sline[rg * 8 + rr];
-        if (ksl < kn && yz.x >= 0 && f < M) {
-          bq[r] = Ty[(size_t)f * n + yz.x];
-          dq[r] = Tz[(size_t)f * n + yz.y];
-        } else {
-          bq[r] = dq[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (!mine) continue;
+          float yh, yl, eh, el;
+          int m;
+          df::mul(sh, sl, sch, scl, yh, yl);
+          df::exp_df(yh, yl, se2, se2 + 32, eh, el, m);
+          const size_t x = (size_t)(xb * N + xh + c0 + q);
+          const size_t o = face ? ((L0 + myl) * n + x) * n + (n - 1) : (L0 + myl) * n + x;
+          if constexpr (sizeof(TOut) == 8)
+            out[o] = (widen(eh) + widen(el)) * __hiloint2double((m + 1023) << 20, 0);
+          else
+            out[o] = (m > -126 && m < 128) ? __fmul_rn(eh, __int_as_float((m + 127) << 23)) : ldexpf(eh, m);
         }
       }
+    };
+    // a warp stages groups of eight lines by four features (kg: the k-step's half): 32 / SW
+    // groups per k-step; groups without a line are left out (their rows of A only reach
+    // accumulator rows that nothing reads)
+    constexpr int G = 32 / SW;
+    const int fl4 = lane & 3, rr = lane >> 2;
+    for (int ks = 0; ks < KS; ++ks) {
+      const int st = ks % NS;
+      float4 bq[G], dq[G];  // (loading them a k-step ahead measured no faster)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int it = tid + (4 * h + r) * STAGERS;
-        const int fl4 = it & 3, rr = (it >> 2) & 7, kg = (it >> 5) & 1, rg = (it >> 6) & 15, ksl = it >> 10;
-        if (ksl >= kn) continue;
+      for (int r = 0; r < G; ++r) {
+        const int pair = warp + SW * r, kg = pair & 1, rg = pair >> 1, f = ks * 8 + kg * 4 + fl4;
+        bq[r] = dq[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (rg * 8 < nvalid && f < M) {
+          const int2 o = sline[rg * 8 + rr];
+          bq[r] = tab[(size_t)f * n + o.x];
+          dq[r] = tab[(size_t)f * n + o.y];
+        }
+      }
+      if (ks >= NS && !wait_warp(&empty[st], ks / NS - 1)) break;
+      unsigned char* sA = sm + (size_t)st * S::stage;
+#pragma unroll
+      for (int r = 0; r < G; ++r) {
+        const int pair = warp + SW * r, kg = pair & 1, rg = pair >> 1;
+        if (rg * 8 >= nvalid) continue;
         uint32_t q[kTcSlices];
         q_slices(bq[r], dq[r], q);  // zero tables give zero slices
-        unsigned char* dst = sA + (size_t)ksl * kTcSlices * kUmATile + umma::pair_offset(rg * 8 + rr, kg * 4 + fl4);
+        unsigned char* dst = sA + umma::pair_offset(rg * 8 + rr, kg * 4 + fl4);
 #pragma unroll
         for (int j = 0; j < kTcSlices; ++j) *reinterpret_cast<uint32_t*>(dst + (size_t)j * kUmATile) = q[j];
       }
-    }
-    fence_proxy_async();
-    umma::fence_before_sync();
-    bad = __syncthreads_or(bad);
-    if (bad) break;
-    if (tid == issuer) {
-      // the x-slices of chunk c + 1 go to the other buffer once the products of chunk c - 1,
-      // its last readers, are done (they are by now as a rule), a chunk ahead of their use
-      if (c + 1 < nchunks) {
-        if (c >= 1) wait(&mdone[b ^ 1], c - 1, budget);
-        if (!bad) issue_copy(c + 1);
-      }
-      if (!bad) wait(&bfull[b], c, budget);
-      if (!bad) {
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[st]);
+      if (MULTI && (ks + 1) % kFoldSteps == 0 && ks + 1 < KS) {
+        if (!wait_warp(accf, (ks + 1) / kFoldSteps - 1)) break;
         umma::fence_after_sync();
-        const bool fresh = (ks0 * 8) % kTcFold == 0;  // the first chunk of a fold period
-        // a tile's descriptor is the chunk base's plus its byte offset / 16 (shared-memory
-        // addresses stay below 2^18, so the 14-bit address field does not carry)
-        const uint64_t ad0 = umma::smem_desc(smem_addr(sA), umma::kLeadingBytes, umma::kStrideBytes);
-        const uint64_t bd0 = umma::smem_desc(smem_addr(sB), umma::kLeadingBytes, umma::kStrideBytes);
-#pragma unroll
-        for (int ksl = 0; ksl < kUmKC; ++ksl) {
-          if (ksl >= kn) break;
-#pragma unroll
-          for (int j = 0; j < kTcSlices; ++j)
-#pragma unroll
-            for (int i = kTcSlices - 1 - j; i >= 0; --i)
-              umma::mma_bf16(tmem + (uint32_t)((i + j) * kUmN),
-                             ad0 + (uint64_t)(((ksl * kTcSlices + i) * kUmATile) >> 4),
-                             bd0 + (uint64_t)(((ksl * kTcSlices + j) * kUmBTile) >> 4), idesc,
-                             (fresh && ksl == 0 && j == 0) ? 0u : 1u);
-        }
-        umma::commit(&mdone[b]);
-        last_commit = c;
+        fold(false);
+        umma::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce);
       }
     }
-    // every 256 features, before the next chunk overwrites the groups: fold them
-    if (((ks0 + kn) * 8) % kTcFold == 0 && c + 1 < nchunks) {
-      bad = __syncthreads_or(bad);
-      if (bad) break;
-      wait(&mdone[b], c, budget);
-      umma::fence_after_sync();
-      bad = __syncthreads_or(bad);
-      if (bad) break;
-      if (stager) fold(false);
-      umma::fence_before_sync();
-      __syncthreads();
+    if (!bad) wait_warp(accf, MULTI ? (KS - 1) / kFoldSteps : 0);
+    umma::fence_after_sync();
+    if (bad) {
+      if (mine)
+        for (int q = 0; q < XW; ++q) {
+          const size_t x = (size_t)(xb * N + xh + q);
+          out[face ? ((L0 + myl) * n + x) * n + (n - 1) : (L0 + myl) * n + x] = (TOut)__int_as_float(0x7fc00000);
+        }
+    } else {
+      fold(true);
     }
-  }
-  bad = __syncthreads_or(bad);
-  if (!bad) wait(&mdone[(nchunks - 1) & 1], nchunks - 1, budget);
-  bad = __syncthreads_or(bad);
-  if (bad && tid == issuer) {
-    // drain: the last issued products and copy land before the block leaves
-    if (last_commit >= 0) mbar_wait_bounded(&mdone[last_commit & 1], (unsigned)((last_commit >> 1) & 1), kDrainBudget);
-    for (int cc = last_copy - 1; cc <= last_copy; ++cc)  // the copies run up to one chunk ahead
-      if (cc >= 0) mbar_wait_bounded(&bfull[cc & 1], (unsigned)((cc >> 1) & 1), kDrainBudget);
-  }
-  umma::fence_after_sync();
-  if (!stager) {
-  } else if (!bad) {
-    fold(true);
-  } else if (myline < n2) {
-#pragma unroll 4
-    for (int q = 0; q < XW; ++q) out[q] = (TOut)__int_as_float(0x7fc00000);
+  } else if (lane == 0) {
+    int last_copy = -1, last_commit = -1;
+    auto issue_copy = [&](int c) {  // the bulk copy of k-step c's x-slices into its stage
+      mbar_arrive_expect_tx(&bfull[c % NS], (unsigned)S::b_stage);
+      bulk_g2s(sm + (size_t)(c % NS) * S::stage + S::a_stage, xu + (size_t)c * S::b_stage, (unsigned)S::b_stage,
+               &bfull[c % NS]);
+      last_copy = c;
+    };
+    for (int c = 0; c < NS && c < KS; ++c) issue_copy(c);
+    if (inject) wait(never, 0, budget);  // injected failure: runs out after the budget
+    for (int ks = 0; ks < KS && !bad; ++ks) {
+      const int st = ks % NS, use = ks / NS;
+      if (MULTI && ks > 0 && ks % kFoldSteps == 0 && !wait(acce, ks / kFoldSteps - 1, budget)) break;
+      if (!wait(&bfull[st], use, budget) || !wait(&full[st], use, budget)) break;
+      umma::fence_after_sync();
+      const bool fresh = ks % kFoldSteps == 0;  // the first k-step of a fold period
+      // a tile's descriptor is the stage base's plus its byte offset / 16 (shared-memory
+      // addresses stay below 2^18, so the 14-bit address field does not carry)
+      const unsigned char* sA = sm + (size_t)st * S::stage;
+      const uint64_t ad0 = umma::smem_desc(smem_addr(sA), umma::kLeadingBytes, umma::kStrideBytes);
+      const uint64_t bd0 = umma::smem_desc(smem_addr(sA + S::a_stage), umma::kLeadingBytes, umma::kStrideBytes);
+      // A's slice i times B's slices 0 .. 6 - i at once: their tiles follow each other in shared
+      // memory (rows 32 bytes apart throughout) as their groups i .. 6 do in tensor memory, so it
+      // is one product of (7 - i) N columns, cut at the instruction's 256
+#pragma unroll
+      for (int i = 0; i < kTcSlices; ++i)
+#pragma unroll
+        for (int c0 = 0; c0 < (kTcSlices - i) * N; c0 += 256) {
+          const int cols = (kTcSlices - i) * N - c0 < 256 ? (kTcSlices - i) * N - c0 : 256;
+          umma::mma_bf16(tmem + (uint32_t)(i * N + c0), ad0 + (uint64_t)((i * kUmATile) >> 4),
+                         bd0 + (uint64_t)((c0 * 32) >> 4), umma::idesc_bf16_f32(kUmM, cols),
+                         fresh && i == 0 ? 0u : 1u);
+        }
+      umma::commit(&empty[st]);
+      last_commit = ks;
+      if (MULTI && (ks + 1) % kFoldSteps == 0 && ks + 1 < KS) umma::commit(accf);
+      // the stage of k-step ks - 1 gets its next x-slices once its products are done
+      if (ks >= 1 && ks - 1 + NS < KS) {
+        if (!wait(&empty[(ks - 1) % NS], (ks - 1) / NS, budget)) break;
+        issue_copy(ks - 1 + NS);
+      }
+    }
+    if (!bad) {
+      umma::commit(accf);
+    } else {
+      // drain: the last issued products and copies land before the block leaves
+      if (last_commit >= 0) mbar_wait_bounded(&empty[last_commit % NS], (unsigned)((last_commit / NS) & 1), kDrainBudget);
+      for (int c = max(0, last_copy - NS + 1); c <= last_copy; ++c)
+        mbar_wait_bounded(&bfull[c % NS], (unsigned)((c / NS) & 1), kDrainBudget);
+    }
   }
   umma::fence_before_sync();
   __syncthreads();
-  if (warp == 0) umma::dealloc(tmem, kUmCols);
+  if (warp == 0) umma::dealloc(tmem, S::cols);
+}
+
+template <typename TOut, int N, bool MULTI>
+int field_umma_launch(const float4* xsplit, const unsigned char* XU, const float* e2tab, int M, int n, int KS, int B,
+                      double scale, int inject, int* err, TOut* kout, double bytes, double flops, cudaStream_t st) {
+  using S = UmShape<N>;
+  static const cudaError_t attr = cudaFuncSetAttribute(k_field_umma<TOut, N, MULTI>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
+  MLMC_CUDA_TRY(attr);
+  const size_t tiles = ((size_t)n * n + kUmM - 1) / kUmM + (n + kUmM - 1) / kUmM;
+  MLMC_LAUNCH("field_tc", bytes, flops, st,
+              (k_field_umma<TOut, N, MULTI><<<dim3((unsigned)((n - 1) / N), (unsigned)tiles, (unsigned)B), S::threads,
+                                              S::smem, st>>>(xsplit, XU, e2tab, M, n, KS, scale, wait_budget_clocks(),
+                                                             inject, err, kout)));
+  return MLMC_OK;
 }
 
 template <typename TOut>
-int field_umma_launch(const float4* xsplit, const unsigned char* XU, const float* e2tab, int M, int n,
-                      int KS, int B, double scale, void* kout, double bytes, double flops, cudaStream_t st,
-                      double share) {
-  // one fold (up to 256 features): 16 staging warps at 120 registers; more: 8, which also hold
-  // the running double-float sums; and the issuing warp
-  static const cudaError_t attr1 = cudaFuncSetAttribute(k_field_umma<TOut, false, 16>,
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUmSmem);
-  static const cudaError_t attr2 = cudaFuncSetAttribute(k_field_umma<TOut, true, 8>,
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUmSmem);
-  MLMC_CUDA_TRY(attr1);
-  MLMC_CUDA_TRY(attr2);
-  const dim3 grid((unsigned)((n - 1) / kUmN), (unsigned)(((size_t)n * n + kUmM - 1) / kUmM), (unsigned)B);
-  const long long budget = wait_budget_clocks();
+int field_umma(const float4* xsplit, const unsigned char* XU, const float* e2tab, int M, int n, int KS, int B,
+               double scale, void* kout, double bytes, double flops, cudaStream_t st) {
   int inject = 0;
   for (int left = g_inject_wait.load(); left > 0; left = g_inject_wait.load())
     if (g_inject_wait.compare_exchange_weak(left, left - 1)) {
@@ -1069,46 +1112,45 @@ int field_umma_launch(const float4* xsplit, const unsigned char* XU, const float
     set_error("field: no address for the wait-error flag");
     return MLMC_ERR_CUDA;
   }
-  if (M > kTcFold)
-    MLMC_LAUNCH("field_tc", bytes * share, flops * share, st,
-                (k_field_umma<TOut, true, 8><<<grid, 32 * 9, kUmSmem, st>>>(xsplit, XU, e2tab, M, n, KS, scale, budget,
-                                                                             inject, err, (TOut*)kout)));
-  else
-    MLMC_LAUNCH("field_tc", bytes * share, flops * share, st,
-                (k_field_umma<TOut, false, 16><<<grid, 32 * 17, kUmSmem, st>>>(xsplit, XU, e2tab, M, n, KS, scale,
-                                                                                budget, inject, err, (TOut*)kout)));
-  return MLMC_OK;
+  auto go = [&](auto N, auto multi) {
+    return field_umma_launch<TOut, decltype(N)::value, decltype(multi)::value>(
+        xsplit, XU, e2tab, M, n, KS, B, scale, inject, err, (TOut*)kout, bytes, flops, st);
+  };
+  auto pick = [&](auto multi) {
+    switch (umma_n(n)) {
+      case 16: return go(std::integral_constant<int, 16>(), multi);
+      case 32: return go(std::integral_constant<int, 32>(), multi);
+      default: return go(std::integral_constant<int, 64>(), multi);
+    }
+  };
+  return M > kTcFold ? pick(std::true_type()) : pick(std::false_type());
 }
 
-// All of the tensor-core form: slices of the x- and y-phasors, the face factors, the volume
-// x < n - 1 (tcgen05 from n = 65 unless warp_mma, warp-level mma.sync otherwise), the face
-// x = n - 1 (y < n - 1), the edge x = y = n - 1.
+// All of the tensor-core form: the phasors' slices, the volume x < n - 1 and the face x = n - 1
+// (y < n - 1) in one tcgen05 launch (warp_mma: on the warp-level mma.sync, with the face factors,
+// in two), the edge x = y = n - 1.
 template <typename TOut>
 int field_tc_all(const double2* tab, const float4* xsplit, float4* pt, uint4* Xf, unsigned char* XU, float* e2tab, int M, int n, int B, double scale, void* kout, double bytes, double flops,
                  cudaStream_t st, bool warp_mma) {
   const int KS = (M + 7) / 8;
-  const size_t nxs = (size_t)B * ((n - 1) / 16) * KS * 32;
-  const bool umma_volume = !warp_mma && umma_applies(n);
-  const int axis0 = umma_volume ? 1 : 0;  // the tcgen05 volume takes its x-slices from k_uxslices
-  MLMC_LAUNCH("xslices", (double)nxs * (2 - axis0) * 112.0, (double)nxs * (2 - axis0) * 500.0, st,
-              (k_xslices<<<blocks_for((2 - axis0) * nxs, 256), 256, 0, st>>>(xsplit, B, M, n, KS, axis0, Xf,
-                                                                               e2tab)));
-  const size_t nf = (size_t)B * M * n;
-  MLMC_LAUNCH("face_factors", (double)nf * 48.0, (double)nf * 40.0, st,
-              (k_face_factors<<<blocks_for(nf, 256), 256, 0, st>>>(xsplit, B, M, n, pt)));
   const double n3 = (double)n * n * n;
-  const double vshare = (double)(n - 1) * n * n / n3;
-  if (umma_volume) {
-    const size_t nux = (size_t)B * ((n - 1) / kUmN) * KS * kUmN * 8;
+  if (!warp_mma) {
+    const size_t nux = (size_t)2 * B * (n - 1) * KS * 8;
     MLMC_LAUNCH("xslices", (double)nux * 28.0, (double)nux * 250.0, st,
-                (k_uxslices<<<blocks_for(nux, 256), 256, 0, st>>>(xsplit, B, M, n, KS, XU)));
-    MLMC_TRY(field_umma_launch<TOut>(xsplit, XU, e2tab, M, n, KS, B, scale, kout, bytes, flops, st, vshare));
+                (k_uxslices<<<blocks_for(nux, 256), 256, 0, st>>>(xsplit, B, M, n, umma_n(n), KS, XU, e2tab)));
+    MLMC_TRY(field_umma<TOut>(xsplit, XU, e2tab, M, n, KS, B, scale, kout, bytes * (1.0 - n / n3),
+                              flops * (1.0 - n / n3), st));
   } else {
+    const size_t nxs = (size_t)B * ((n - 1) / 16) * KS * 32, nf = (size_t)B * M * n;
+    MLMC_LAUNCH("xslices", (double)nxs * 2 * 112.0, (double)nxs * 2 * 500.0, st,
+                (k_xslices<<<blocks_for(2 * nxs, 256), 256, 0, st>>>(xsplit, B, M, n, KS, 0, Xf, e2tab)));
+    MLMC_LAUNCH("face_factors", (double)nf * 48.0, (double)nf * 40.0, st,
+                (k_face_factors<<<blocks_for(nf, 256), 256, 0, st>>>(xsplit, B, M, n, pt)));
     MLMC_TRY((field_tc_dispatch<TOut, false>(xsplit, pt, Xf, e2tab, M, n, KS, B, scale, kout, bytes, flops, st,
-                                             vshare)));
+                                             (double)(n - 1) * n * n / n3)));
+    MLMC_TRY((field_tc_dispatch<TOut, true>(xsplit, pt, Xf + nxs * kTcSlices, e2tab, M, n, KS, B, scale, kout, bytes,
+                                            flops, st, (double)(n - 1) * n / n3)));
   }
-  MLMC_TRY((field_tc_dispatch<TOut, true>(xsplit, pt, Xf + nxs * kTcSlices, e2tab, M, n, KS, B, scale, kout, bytes,
-                                          flops, st, (double)(n - 1) * n / n3)));
   MLMC_LAUNCH("field_edge", bytes * n / n3, flops * n / n3, st,
               (k_field_edge<TOut><<<(unsigned)(((size_t)B * n + 3) / 4), 128, 0, st>>>(tab, B, M, n, scale,
                                                                                        (TOut*)kout)));
@@ -1118,12 +1160,17 @@ int field_tc_all(const double2* tab, const float4* xsplit, float4* pt, uint4* Xf
 // The tensor-core form applies where the x-values below n - 1 make whole row tiles.
 static bool tc_applies(int n) { return n >= 17 && (n - 1) % 16 == 0; }
 
+// Bytes of the pieces that only one tensor-core form uses: the tcgen05 form's operand tiles of
+// both axes, or the mma.sync form's fragments and face factors.
+static size_t tc_form_bytes(int B, int M, int n, bool warp_mma) {
+  return warp_mma ? a256(2 * tc_xslice_bytes(B, M, n)) + a256((size_t)B * M * n * sizeof(float4))
+                  : a256(2 * tc_uxslice_bytes(B, M, n));
+}
+
 size_t field_scratch_bytes(int B, int M, int n) {
   return a256((size_t)B * M * 3 * sizeof(double)) + a256((size_t)B * M * sizeof(double)) +
          a256((size_t)B * 3 * M * n * sizeof(double2)) + a256((size_t)B * 3 * M * n * sizeof(float4)) +
-         (tc_applies(n) ? a256(2 * tc_xslice_bytes(B, M, n)) + a256(64 * sizeof(float)) +
-                              a256((size_t)B * M * n * sizeof(float4)) + a256(tc_uxslice_bytes(B, M, n))
-                        : 0);
+         (tc_applies(n) ? a256(64 * sizeof(float)) + tc_form_bytes(B, M, n, field_arith_default() == kFieldTCWarp) : 0);
 }
 
 int field_arith_default() {
@@ -1136,8 +1183,8 @@ int field_arith_default() {
 }
 
 int field_eval_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, int n, int dtype, void* kout,
-                   void* scratch, cudaStream_t st, int arith) {
-  if (arith < 0) arith = field_arith_default();
+                   void* scratch, cudaStream_t st) {
+  const int arith = field_arith_default();
   char* p = (char*)scratch;
   auto carve = [&](size_t bytes) {
     void* r = p;
@@ -1148,10 +1195,17 @@ int field_eval_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, in
   double* bph = (double*)carve((size_t)B * cfg.M * sizeof(double));
   double2* tab = (double2*)carve((size_t)B * 3 * cfg.M * n * sizeof(double2));
   float4* xsplit = (float4*)carve((size_t)B * 3 * cfg.M * n * sizeof(float4));
-  uint4* Xf = tc_applies(n) ? (uint4*)carve(2 * tc_xslice_bytes(B, cfg.M, n)) : nullptr;
+  const bool warp_mma = field_arith_default() == kFieldTCWarp;
   float* e2tab = tc_applies(n) ? (float*)carve(64 * sizeof(float)) : nullptr;
-  float4* pt = tc_applies(n) ? (float4*)carve((size_t)B * cfg.M * n * sizeof(float4)) : nullptr;
-  unsigned char* XU = tc_applies(n) ? (unsigned char*)carve(tc_uxslice_bytes(B, cfg.M, n)) : nullptr;
+  uint4* Xf = nullptr;
+  float4* pt = nullptr;
+  unsigned char* XU = nullptr;
+  if (tc_applies(n) && warp_mma) {
+    Xf = (uint4*)carve(2 * tc_xslice_bytes(B, cfg.M, n));
+    pt = (float4*)carve((size_t)B * cfg.M * n * sizeof(float4));
+  } else if (tc_applies(n)) {
+    XU = (unsigned char*)carve(2 * tc_uxslice_bytes(B, cfg.M, n));
+  }
   const size_t nf = (size_t)B * cfg.M;
   MLMC_LAUNCH("features", nf * 40.0, nf * 200.0, st,
               (k_features<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(ids_dev, B, cfg.M, cfg.run_seed,
@@ -1186,7 +1240,6 @@ int field_eval_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, in
     const int MCl = cfg.M < 64 ? cfg.M : 64;
     const unsigned lines = (unsigned)(((size_t)n * n + kFieldThreads - 1) / kFieldThreads);
     if ((arith == kFieldTC || arith == kFieldTCWarp) && tc_applies(n)) {
-      const bool warp_mma = arith == kFieldTCWarp;
       if (dtype == MLMC_F64)
         MLMC_TRY(field_tc_all<double>(tab, xsplit, pt, Xf, XU, e2tab, cfg.M, n, B, scale, kout, bytes, flops, st,
                                       warp_mma));
