@@ -400,13 +400,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // (The paired FP32 instructions, f32x2, with Re and Im as the two lanes measured slower here:
 // the packing of the lanes costs more integer instructions than the pairing saves.)
 __device__ __forceinline__ void q_slices(const float4& y, const float4& z, uint32_t (&q)[kTcSlices]) {
-  float t1h, t1l, t2h, t2l, rh, rl, ih, il, qr[kTcSlices], qi[kTcSlices];
-  df::mul(y.x, y.y, z.x, z.y, t1h, t1l);
-  df::mul(y.z, y.w, z.z, z.w, t2h, t2l);
-  df::add(t1h, t1l, -t2h, -t2l, rh, rl);
-  df::mul(y.x, y.y, z.z, z.w, t1h, t1l);
-  df::mul(y.z, y.w, z.x, z.y, t2h, t2l);
-  df::add(t1h, t1l, t2h, t2l, ih, il);
+  float rh, rl, ih, il, qr[kTcSlices], qi[kTcSlices];
+  df::cmul(y.x, y.y, y.z, y.w, z.x, z.y, z.z, z.w, rh, rl, ih, il);
   df::slice7(rh, rl, qr);
   df::slice7(ih, il, qi);
 #pragma unroll
@@ -484,13 +479,8 @@ __global__ void k_face_factors(const float4* __restrict__ xsplit, int B, int M, 
     const int s = (int)(sm / M);
     const float4 a = xsplit[((size_t)s * 3 * M + m) * n + (n - 1)];
     const float4 d = xsplit[(((size_t)s * 3 + 2) * M + m) * n + z];
-    float t1h, t1l, t2h, t2l, rh, rl, ih, il;
-    df::mul(a.x, a.y, d.x, d.y, t1h, t1l);
-    df::mul(a.z, a.w, d.z, d.w, t2h, t2l);
-    df::add(t1h, t1l, -t2h, -t2l, rh, rl);
-    df::mul(a.x, a.y, d.z, d.w, t1h, t1l);
-    df::mul(a.z, a.w, d.x, d.y, t2h, t2l);
-    df::add(t1h, t1l, t2h, t2l, ih, il);
+    float rh, rl, ih, il;
+    df::cmul(a.x, a.y, a.z, a.w, d.x, d.y, d.z, d.w, rh, rl, ih, il);
     pt[t] = make_float4(rh, rl, ih, il);
   }
 }
@@ -971,35 +961,41 @@ __global__ void __launch_bounds__(UmShape<N>::threads, UmShape<N>::BPS)
         }
       }
     };
-    // a warp stages groups of eight lines by four features (kg: the k-step's half): 32 / SW
-    // groups per k-step; groups without a line are left out (their rows of A only reach
-    // accumulator rows that nothing reads)
-    constexpr int G = 32 / SW;
-    const int fl4 = lane & 3, rr = lane >> 2;
+    // a warp stages groups of eight lines by the k-step's eight features, two adjacent features
+    // (eight bytes of a row of A) per lane: 16 / SW groups per k-step; groups without a line are
+    // left out (their rows of A only reach accumulator rows that nothing reads)
+    constexpr int G = 16 / SW;
+    const int f2 = 2 * (lane & 3), rr = lane >> 2;
     for (int ks = 0; ks < KS; ++ks) {
       const int st = ks % NS;
-      float4 bq[G], dq[G];  // (loading them a k-step ahead measured no faster)
+      float4 bq[G][2], dq[G][2];  // (loading them a k-step ahead measured no faster)
 #pragma unroll
       for (int r = 0; r < G; ++r) {
-        const int pair = warp + SW * r, kg = pair & 1, rg = pair >> 1, f = ks * 8 + kg * 4 + fl4;
-        bq[r] = dq[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (rg * 8 < nvalid && f < M) {
-          const int2 o = sline[rg * 8 + rr];
-          bq[r] = tab[(size_t)f * n + o.x];
-          dq[r] = tab[(size_t)f * n + o.y];
+        const int rg = warp + SW * r;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int f = ks * 8 + f2 + e;
+          bq[r][e] = dq[r][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (rg * 8 < nvalid && f < M) {
+            const int2 o = sline[rg * 8 + rr];
+            bq[r][e] = tab[(size_t)f * n + o.x];
+            dq[r][e] = tab[(size_t)f * n + o.y];
+          }
         }
       }
       if (ks >= NS && !wait_warp(&empty[st], ks / NS - 1)) break;
       unsigned char* sA = sm + (size_t)st * S::stage;
 #pragma unroll
       for (int r = 0; r < G; ++r) {
-        const int pair = warp + SW * r, kg = pair & 1, rg = pair >> 1;
+        const int rg = warp + SW * r;
         if (rg * 8 >= nvalid) continue;
-        uint32_t q[kTcSlices];
-        q_slices(bq[r], dq[r], q);  // zero tables give zero slices
-        unsigned char* dst = sA + umma::pair_offset(rg * 8 + rr, kg * 4 + fl4);
+        uint32_t q0[kTcSlices], q1[kTcSlices];
+        q_slices(bq[r][0], dq[r][0], q0);  // zero tables give zero slices
+        q_slices(bq[r][1], dq[r][1], q1);
+        unsigned char* dst = sA + umma::pair_offset(rg * 8 + rr, f2);
 #pragma unroll
-        for (int j = 0; j < kTcSlices; ++j) *reinterpret_cast<uint32_t*>(dst + (size_t)j * kUmATile) = q[j];
+        for (int j = 0; j < kTcSlices; ++j)
+          *reinterpret_cast<uint2*>(dst + (size_t)j * kUmATile) = make_uint2(q0[j], q1[j]);
       }
       fence_proxy_async();
       __syncwarp();
