@@ -68,42 +68,48 @@ __global__ void k_features(const uint64_t* __restrict__ ids, int B, int M, uint6
 }
 
 // Phasor tables tab[s][axis][m][i] = (cos, sin) of (w_axis x_i (+ b_m on axis 0)), and
-// the same pre-split for the double-float kernels, xs = (Re hi, Re lo, Im hi, Im lo). A
-// thread fills a run of kPhRun consecutive i of one (sample, axis, feature) row: the first
-// entry by sincos of its phase, the next ones by multiplying by the step e^{i w h} (one
-// sincos per run), so each entry costs one complex product instead of a sincos on the FP64
-// unit; over a run the products add a few ulps (below 2e-15 relative). The split is done
-// by the integer-pipe narrowing (hi = fl32(v), lo = fl32(v - hi), the difference exact in
-// FP64).
+// the same pre-split for the double-float sums, xs = (Re hi, Re lo, Im hi, Im lo). A row (one
+// sample, axis and feature) is cut into runs of kPhRun entries (the last takes the row's remainder:
+// nine on every grid from n = 9); a run's first entry is the sincos of its phase, the next ones are
+// products with the step e^{i w h} (over a run the products add a few ulps, below 2e-15 relative).
+// A thread fills `group` consecutive runs of a row with one sincos of the step between them. The
+// FP64 pipe bounds it (one sincos is worth about 40 operations, a product 4); the split runs on the
+// integer pipe. `all` = false leaves out the entries of tab that the tensor-core form does not read
+// (it takes tab only for the edge x = y = n - 1: axis 2 and the last entries of the others), a
+// third of the bytes. 17^3 x 4096: 1.78 ms with a step sincos per run, FP64 splits and runs of 8, 8
+// and 1, 0.88 now; 33^3 x 103 72 -> 45 us.
 constexpr int kPhRun = 8;
+__device__ __forceinline__ int phasor_runs(int n) { return n > 2 * kPhRun ? (n - 1) / kPhRun : 1; }
 __global__ void k_phasors(const double* __restrict__ w, const double* __restrict__ bph, int B, int M, int n,
-                          double h, double2* __restrict__ tab, float4* __restrict__ xs) {
-  const int runs = (n + kPhRun - 1) / kPhRun;
-  const size_t total = (size_t)B * 3 * M * runs;
+                          double h, double2* __restrict__ tab, float4* __restrict__ xs, int group = 1,
+                          bool all = true) {
+  const int runs = phasor_runs(n), groups = (runs + group - 1) / group;
+  const size_t total = (size_t)B * 3 * M * groups;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-    const int run = (int)(t % runs);
-    const size_t r = t / runs;  // row (s, axis, m)
+    const size_t r = t / groups;  // row (s, axis, m)
+    const int run0 = (int)(t - r * groups) * group, run1 = run0 + group < runs ? run0 + group : runs;
     const int m = (int)(r % M);
     const size_t r2 = r / M;
     const int axis = (int)(r2 % 3);
     const int s = (int)(r2 / 3);
     const size_t f = (size_t)s * M + m;
     const double wa = w[3 * f + axis];
-    const int i0 = run * kPhRun;
-    double ph = wa * ((double)i0 * h);
-    if (axis == 0) ph += bph[f];
-    double sn, cs, ds, dc;
-    sincos(ph, &sn, &cs);
+    double ds, dc;
     sincos(wa * h, &ds, &dc);
-    const int i1 = i0 + kPhRun < n ? i0 + kPhRun : n;
-    for (int i = i0; i < i1; ++i) {
-      const size_t o = r * n + i;
-      tab[o] = make_double2(cs, sn);
-      const float ch = narrow(cs), sh = narrow(sn);
-      xs[o] = make_float4(ch, narrow(cs - widen(ch)), sh, narrow(sn - widen(sh)));
-      const double c2 = cs * dc - sn * ds, s2 = sn * dc + cs * ds;
-      cs = c2;
-      sn = s2;
+    for (int run = run0; run < run1; ++run) {
+      const int i0 = run * kPhRun, i1 = run == runs - 1 ? n : i0 + kPhRun;
+      double ph = wa * ((double)i0 * h);
+      if (axis == 0) ph += bph[f];
+      double sn, cs;
+      sincos(ph, &sn, &cs);
+      for (int i = i0; i < i1; ++i) {
+        const size_t o = r * n + i;
+        if (all || axis == 2 || i == n - 1) tab[o] = make_double2(cs, sn);
+        xs[o] = make_float4(narrow(cs), narrow_rest(cs), narrow(sn), narrow_rest(sn));
+        const double c2 = cs * dc - sn * ds, s2 = sn * dc + cs * ds;
+        cs = c2;
+        sn = s2;
+      }
     }
   }
 }
@@ -485,27 +491,43 @@ __global__ void k_face_factors(const float4* __restrict__ xsplit, int B, int M, 
   }
 }
 
-// The edge x = y = n - 1 in FP64 (n nodes per sample): one warp per (sample, z), lanes over the
-// features, log k / scale = sum_m Re(X_m[n - 1] Y_m[n - 1] Z_m[z]), a butterfly sum over the lanes.
-template <typename TOut>
+// The edge x = y = n - 1 in FP64 (n nodes per sample): one warp per sample and ZC values of z,
+// lanes over the features, log k / scale = sum_m Re(X_m[n - 1] Y_m[n - 1] Z_m[z]) with the product
+// of the first two formed once for the warp's z, a butterfly sum over the lanes. Bound by the FP64
+// pipe for many samples (there six z per warp share the product: 17^3 x 4096 282 -> 196 us), by the
+// length of one warp's chain for few (there one z: 65^3 x 5 with 1024 features 27 us, 80 with six).
+template <typename TOut, int kEdgeZ>
 __global__ void k_field_edge(const double2* __restrict__ tab, int B, int M, int n, double scale,
                              TOut* __restrict__ kout) {
   const size_t gw = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (size_t)B * n) return;
-  const int s = (int)(gw / n), z = (int)(gw % n);
+  const int lane = threadIdx.x & 31, zb = (n + kEdgeZ - 1) / kEdgeZ;
+  if (gw >= (size_t)B * zb) return;
+  const int s = (int)(gw / zb), z0 = (int)(gw % zb) * kEdgeZ;
   const double2* Tx = tab + (size_t)s * 3 * M * n;
   const double2* Ty = Tx + (size_t)M * n;
   const double2* Tz = Ty + (size_t)M * n;
-  double acc = 0.0;
+  double acc[kEdgeZ];
+#pragma unroll
+  for (int k = 0; k < kEdgeZ; ++k) acc[k] = 0.0;
   for (int m = lane; m < M; m += 32) {
-    const double2 x = Tx[(size_t)m * n + n - 1], y = Ty[(size_t)m * n + n - 1], zz = Tz[(size_t)m * n + z];
+    const double2 x = Tx[(size_t)m * n + n - 1], y = Ty[(size_t)m * n + n - 1];
     const double cr = x.x * y.x - x.y * y.y, ci = x.x * y.y + x.y * y.x;
-    acc = fma(cr, zz.x, fma(-ci, zz.y, acc));
+#pragma unroll
+    for (int k = 0; k < kEdgeZ; ++k) {
+      if (z0 + k >= n) break;
+      const double2 zz = Tz[(size_t)m * n + z0 + k];
+      acc[k] = fma(cr, zz.x, fma(-ci, zz.y, acc[k]));
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) kout[(size_t)s * n * n * n + ((size_t)z * n + n - 1) * n + n - 1] = (TOut)exp(scale * acc);
+  for (int k = 0; k < kEdgeZ; ++k) {
+    if (z0 + k >= n) break;
+    double v = acc[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0)
+      kout[(size_t)s * n * n * n + ((size_t)(z0 + k) * n + n - 1) * n + n - 1] = (TOut)exp(scale * v);
+  }
 }
 
 // Block: RX row tiles (16 rows each, from row 16 RX blockIdx.x) by 256 / RX lines (from
@@ -1147,9 +1169,15 @@ int field_tc_all(const double2* tab, const float4* xsplit, float4* pt, uint4* Xf
     MLMC_TRY((field_tc_dispatch<TOut, true>(xsplit, pt, Xf + nxs * kTcSlices, e2tab, M, n, KS, B, scale, kout, bytes,
                                             flops, st, (double)(n - 1) * n / n3)));
   }
-  MLMC_LAUNCH("field_edge", bytes * n / n3, flops * n / n3, st,
-              (k_field_edge<TOut><<<(unsigned)(((size_t)B * n + 3) / 4), 128, 0, st>>>(tab, B, M, n, scale,
-                                                                                       (TOut*)kout)));
+  // six z per warp once that leaves 32 warps for every SM
+  const size_t wide = (size_t)B * ((n + 5) / 6);
+  if (wide >= 152u * 32)
+    MLMC_LAUNCH("field_edge", bytes * n / n3, flops * n / n3, st,
+                (k_field_edge<TOut, 6><<<(unsigned)((wide + 3) / 4), 128, 0, st>>>(tab, B, M, n, scale, (TOut*)kout)));
+  else
+    MLMC_LAUNCH("field_edge", bytes * n / n3, flops * n / n3, st,
+                (k_field_edge<TOut, 1><<<(unsigned)(((size_t)B * n + 3) / 4), 128, 0, st>>>(tab, B, M, n, scale,
+                                                                                           (TOut*)kout)));
   return MLMC_OK;
 }
 
@@ -1208,8 +1236,15 @@ int field_eval_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, in
                                                                           cfg.ell, cfg.cov, w, bph)));
   const double h = 1.0 / (double)(n - 1);
   const size_t nt = (size_t)B * 3 * cfg.M * n;
-  MLMC_LAUNCH("phasors", nt * 32.0, nt * 12.0, st,
-              (k_phasors<<<blocks_for(nt / kPhRun + 1, 256), 256, 0, st>>>(w, bph, B, cfg.M, n, h, tab, xsplit)));
+  // runs per thread: as many as leave two warps for each quarter of an SM, which fill its FP64 pipe
+  const bool tc = (arith == kFieldTC || arith == kFieldTCWarp) && tc_applies(n);
+  const int runs = n > 2 * kPhRun ? (n - 1) / kPhRun : 1;
+  const size_t rows = (size_t)B * 3 * cfg.M;
+  int group = (int)(rows * runs / (152u * 4 * 2 * 32));
+  group = group < 1 ? 1 : (group > runs ? runs : group);
+  MLMC_LAUNCH("phasors", nt * (tc ? 22.0 : 32.0), nt * 12.0, st,
+              (k_phasors<<<blocks_for(rows * ((runs + group - 1) / group), 256), 256, 0, st>>>(
+                  w, bph, B, cfg.M, n, h, tab, xsplit, group, !tc)));
   int LT = 2048 / n;
   if (LT < 1) LT = 1;
   if ((size_t)LT > (size_t)n * n) LT = n * n;

@@ -40,5 +40,17 @@ __device__ __forceinline__ float narrow(double d) {
   const unsigned bits = e <= 0 ? sign : (e >= 255 ? (sign | 0x7f800000u) : (sign | (body >= 0x7f800000u ? 0x7f800000u : body)));
   return __uint_as_float(bits);
 }
+// narrow(d - widen(narrow(d))), the rounded remainder of |d| <= 1, without an FP64 operation: the 29
+// bits below narrow's last one, less the carry, as a signed integer times the ulp of d. Zero where
+// that ulp is below the smallest normal FP32 number (|d| < 2^-74).
+__device__ __forceinline__ float narrow_rest(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const unsigned rem = lo & 0x1fffffffu;
+  const bool up = rem > 0x10000000u || (rem == 0x10000000u && ((lo >> 29) & 1u));
+  const int r = (int)rem - (up ? 0x20000000 : 0);
+  const float ulp = __uint_as_float(e > 948 ? (unsigned)(e - 948) << 23 : 0u);  // 2^(e - 1023 - 52)
+  return (float)((hi & 0x80000000u) ? -r : r) * ulp;
+}
 
 }  // namespace mlmc
