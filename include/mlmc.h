@@ -106,7 +106,9 @@ typedef struct {
 } mlmc_field_cfg;
 
 /* Smoother implementations (all compute the same red-black sweep, bit for bit). */
-#define MLMC_SMOOTH_AUTO 0      /* the tuned choice for the grid size (mlmc_autotune), else a default */
+#define MLMC_SMOOTH_AUTO 0      /* the tuned choice for the grid size (mlmc_autotune), else a default:
+                                    MLMC_SMOOTH_SPLIT from 33^3 (FP32 correction cycles) or 65^3
+                                    (FP64), MLMC_SMOOTH_TWO_PASS below */
 #define MLMC_SMOOTH_TWO_PASS 1  /* one kernel per colour */
 #define MLMC_SMOOTH_FUSED_32x8 2  /* both colours in one z-marching pass, 32x8 x-y tiles */
 #define MLMC_SMOOTH_FUSED_32x16 3

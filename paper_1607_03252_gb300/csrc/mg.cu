@@ -3553,8 +3553,8 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   int nu1 = a.cfg.nu1, nu2 = a.cfg.nu2;
   // the small-grid engine: one persistent launch for the whole solve (grids up to 33^3)
   const bool use_cta = cta_engine_chosen(a.cfg, a.n, a.B);
+  int sm0 = a.cfg.smoother;
   {
-    int sm0 = a.cfg.smoother;
     resolve_tuning(a.n, a.cfg.precision, &sm0, &nu1, &nu2);
     // FP32 correction cycles on finite volumes (mixed), or FP64 stationary and FMG cycles
     // on finite volumes or P1 elements (the split kernels are instantiated for n = 5 .. 1025)
@@ -3626,7 +3626,9 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     }
     int sm = a.cfg.smoother, d1 = 1, d2 = 1;
     resolve_tuning(v.n, a.cfg.precision, &sm, &d1, &d2);
-    if (sm == MLMC_SMOOTH_SPLIT) sm = MLMC_SMOOTH_NODAL;  // split storage only for the whole hierarchy
+    // split storage only for the whole hierarchy; where the finest grid's choice was that, every
+    // grid takes its arithmetic
+    if (sm == MLMC_SMOOTH_SPLIT || sm0 == MLMC_SMOOTH_SPLIT) sm = MLMC_SMOOTH_NODAL;
     // the small-grid engine runs the two-pass arithmetic (bit for bit that of the fused and
     // bulk sweeps) or the nodal one
     if (use_cta && sm != MLMC_SMOOTH_NODAL) sm = MLMC_SMOOTH_TWO_PASS;
