@@ -8,6 +8,7 @@
 
 #include <atomic>
 #include <chrono>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -40,6 +41,62 @@ long long wait_budget_clocks() { return g_wait_budget.load(); }
 // number of further allocations that still succeed before every later one fails.
 static std::atomic<long long> g_alloc_budget{-1};
 
+// The library's own stream-ordered memory pool of a device, created on its first use. The
+// default pool gives every freed byte back to the system at the next synchronisation, so each call
+// of a blocking API mapped its workspace again (a 65^3 field alone 0.3 ms of 1.2, a level of 5 GB 6
+// ms of 29). This one keeps up to a sixteenth of the device's memory between calls; what is freed
+// beyond that goes back at the next synchronisation, all of it when an allocation fails
+// (DevBuf::alloc) or the device runs low (pool_give_back). Pools are safe with any number of
+// threads and streams. NULL (the default pool is used) where the device offers none.
+constexpr int kMaxDevices = 64;
+static cudaMemPool_t device_pool(int dev) {
+  static std::mutex mu;
+  static bool made[kMaxDevices] = {};
+  static cudaMemPool_t pools[kMaxDevices] = {};
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!made[dev]) {
+    made[dev] = true;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    size_t fr = 0, tot = 0;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && cudaMemPoolCreate(&p, &props) == cudaSuccess) {
+      uint64_t keep = tot / 16;
+      if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        pools[dev] = p;
+      else
+        cudaMemPoolDestroy(p);
+    }
+    cudaGetLastError();
+  }
+  return pools[dev];
+}
+
+static cudaMemPool_t current_pool() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess ? device_pool(dev) : nullptr;
+}
+
+// Bytes the pool holds that no allocation uses.
+static size_t pool_idle_bytes() {
+  cudaMemPool_t p = current_pool();
+  uint64_t have = 0, used = 0;
+  if (!p || cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &have) != cudaSuccess ||
+      cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return 0;
+  return have > used ? (size_t)(have - used) : 0;
+}
+
+// Returns the pool's unused memory to the system when less than an eighth of the device is free
+// (called where a call has looked up the free memory).
+static void pool_give_back(size_t fr, size_t tot) {
+  cudaMemPool_t p = current_pool();
+  if (p && fr < tot / 8) cudaMemPoolTrimTo(p, 0);
+}
+
 int DevBuf::alloc(size_t bytes, cudaStream_t st) {
   release();
   st_ = st;
@@ -51,7 +108,15 @@ int DevBuf::alloc(size_t bytes, cudaStream_t st) {
     }
     if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
   }
-  cudaError_t e = cudaMallocAsync(&p_, bytes, st);
+  cudaMemPool_t pool = current_pool();
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p_, bytes, pool, st) : cudaMallocAsync(&p_, bytes, st);
+  if (e == cudaErrorMemoryAllocation && pool) {
+    // what earlier calls left, in this pool and in its fragments, goes back before giving up
+    cudaGetLastError();
+    cudaStreamSynchronize(st);
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(&p_, bytes, pool, st);
+  }
   if (e != cudaSuccess) {
     p_ = nullptr;
     set_error("cudaMallocAsync(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
@@ -454,6 +519,9 @@ static int choose_batch(const mlmc_cfg* cfg, int N, int nf, int nc, int* B) {
   if (b == 0) {
     size_t fr = 0, tot = 0;
     MLMC_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+    const size_t idle = pool_idle_bytes();
+    pool_give_back(fr, tot);
+    fr += idle;
     const size_t per = LevelBatch::bytes_for(1, nf, nc, cfg->field, cfg->mg.precision, cfg->mg.accel);
     size_t fit = (size_t)(0.6 * (double)fr) / (per + 1);
     if (fit < 1) fit = 1;
