@@ -3534,6 +3534,384 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
   }
 }
 
+// ---------------------------------------------------------------------------------
+// The small-grid engine on 17^3 grids: one block of 512 threads per SM with the whole cycle in
+// registers and shared memory. A thread owns up to four nodes of either colour for the whole
+// solve and keeps their six faces in registers; 1/D,
+// iterate, right-hand side and red residuals of 17^3, 9^3 and 5^3 and the 9^3 coefficients are in
+// shared memory (222 KB in FP64). Operations, partitions and trees are k_solve_cta's (which keeps everything in
+// global memory, read through L2 in every pass, and serves 9^3 and 33^3), so results are bit for
+// bit the same. Bound by the chain of passes, one sample per SM. A served request (one mixed CG
+// sample) 1.12 -> 0.57 ms in this kernel, 1.38 -> 0.87 in all.
+// ---------------------------------------------------------------------------------
+template <typename T>
+struct Solve17 {
+  static constexpr int N = 17;
+  using G0 = TailGrid<T, 17, false>;
+  using G1 = TailGrid<T, 9, false>;
+  static constexpr int items = G0::M * G0::M * G0::HALF, per = (items + kTailThreads - 1) / kTailThreads;
+  // shared memory in elements of T: u, g, r of both grids, u and g of 5^3, five 9^3 coefficients,
+  // and 1/D of 17^3
+  static constexpr size_t elems = (size_t)G0::shared_iter + G1::shared_iter + 250 + 5 * G1::N3 + G0::N3;
+  G0 a;
+  G1 b;
+  T *u5, *g5;
+  T c[2][per][6];  // faces -x, +x, -y, +y, -z, +z of the thread's nodes
+  const T* D;      // diagonal of the sample (global)
+
+  __device__ __forceinline__ int item(int k, int colour, bool& on) const {  // linear index of node k
+    int x, y, z;
+    const int it = threadIdx.x + k * kTailThreads;
+    on = it < items && G0::node(it, colour, x, y, z);
+    return on ? (z * N + y) * N + x : 0;
+  }
+  __device__ void load(const CtaArgs<T>& A, int s, T* sm) {
+    T* p = sm;
+    a.u = p;
+    a.g = p + G0::N3;
+    a.r = p + 2 * G0::N3;
+    p += G0::shared_iter;
+    b.u = p;
+    b.g = p + G1::N3;
+    b.r = p + 2 * G1::N3;
+    p += G1::shared_iter;
+    u5 = p;
+    g5 = p + 125;
+    p += 250;
+    T* const c9 = p;
+    p += 5 * G1::N3;
+    T* const dinv = p;
+    for (int i = threadIdx.x; i < (int)(c9 - sm); i += kTailThreads) sm[i] = T(0);
+    const CtaLevel<T>&v = A.lv[0], &w = A.lv[1];
+    const size_t o = (size_t)s * G0::N3, o9 = (size_t)s * G1::N3;
+    D = v.D + o;
+#pragma unroll
+    for (int col = 0; col < 2; ++col)
+#pragma unroll
+      for (int k = 0; k < per; ++k) {
+        bool on;
+        const size_t q = o + item(k, col, on);
+        if (!on) continue;
+        c[col][k][0] = v.Kx[q - 1];
+        c[col][k][1] = v.Kx[q];
+        c[col][k][2] = v.Ky[q - N];
+        c[col][k][3] = v.Ky[q];
+        c[col][k][4] = v.Kz[q - G0::N2];
+        c[col][k][5] = v.Kz[q];
+      }
+    for (int i = threadIdx.x; i < G0::N3; i += kTailThreads) dinv[i] = v.Dinv[o + i];
+    a.Dinv = dinv;
+    const T* src[5] = {w.Kx, w.Ky, w.Kz, w.D, w.Dinv};
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      for (int i = threadIdx.x; i < G1::N3; i += kTailThreads) c9[q * G1::N3 + i] = src[q][o9 + i];
+    a.kn = b.kn = nullptr;
+    b.Kx = c9;
+    b.Ky = c9 + G1::N3;
+    b.Kz = c9 + 2 * G1::N3;
+    b.D = c9 + 3 * G1::N3;
+    b.Dinv = c9 + 4 * G1::N3;
+    __syncthreads();
+  }
+  __device__ __forceinline__ T faces(const T (&f)[6], int p, T acc) const {
+    const T* u = a.u;
+    acc = fma(f[0], u[p - 1], acc);
+    acc = fma(f[1], u[p + 1], acc);
+    acc = fma(f[2], u[p - N], acc);
+    acc = fma(f[3], u[p + N], acc);
+    acc = fma(f[4], u[p - G0::N2], acc);
+    return fma(f[5], u[p + G0::N2], acc);
+  }
+  template <int COL>
+  __device__ void pass(bool zero) {
+#pragma unroll
+    for (int k = 0; k < per; ++k) {
+      bool on;
+      const int p = item(k, COL, on);
+      if (on) a.u[p] = (zero ? a.g[p] : faces(c[COL][k], p, a.g[p])) * a.Dinv[p];
+    }
+    __syncthreads();
+  }
+  // red residuals into r; returns the thread's sum of their squares
+  __device__ double red_residual(bool store) {
+    double sq = 0.0;
+#pragma unroll
+    for (int k = 0; k < per; ++k) {
+      bool on;
+      const int p = item(k, 0, on);
+      if (!on) continue;
+      const T rr = faces(c[0][k], p, fma(-D[p], a.u[p], a.g[p]));
+      if (store) a.r[p >> 1] = rr;
+      else sq += (double)rr * (double)rr;
+    }
+    if (store) __syncthreads();
+    return sq;
+  }
+  // one cycle on a.u for the right-hand side a.g (without pre- or post-smoothing the full
+  // residual or interpolation would be needed: k_solve_cta takes those)
+  __device__ void cycle(const CtaArgs<T>& A, int s, bool zero) {
+    for (int k = 0; k < A.nu1; ++k) {
+      pass<0>(zero && k == 0);
+      pass<1>(false);
+    }
+    red_residual(true);
+    a.template restrict_to<false>(b.g);
+    for (int k = 0; k < A.nu1; ++k) {
+      b.pass(0, k == 0);
+      b.pass(1, false);
+    }
+    b.red_residual();
+    b.template restrict_to<false>(g5);
+    if (threadIdx.x < 27) {  // the exact solve (k_coarse_apply)
+      const int i = threadIdx.x;
+      const double* X = A.Ainv + (size_t)s * 729 + (size_t)i * 27;
+      double v = 0.0;
+      for (int q = 0; q < 27; ++q) v = fma(X[q], (double)g5[((1 + q / 9) * 5 + 1 + (q / 3) % 3) * 5 + 1 + q % 3], v);
+      u5[((1 + i / 9) * 5 + 1 + (i / 3) % 3) * 5 + 1 + i % 3] = (T)v;
+    }
+    __syncthreads();
+    b.template prolong_from<false>(u5);
+    for (int k = 0; k < A.nu2; ++k) {
+      b.pass(0, false);
+      b.pass(1, false);
+    }
+    a.template prolong_from<false>(b.u);
+    for (int k = 0; k < A.nu2; ++k) {
+      pass<0>(false);
+      pass<1>(false);
+    }
+  }
+};
+
+// block_sum of each group of 32 W threads: the same trees; valid in the group's first thread.
+template <int W>
+__device__ __forceinline__ double group_sum(double v, double* warp_part) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if (lane == 0) warp_part[wid] = v;
+  __syncthreads();
+  double r = 0.0;
+  if (wid % W == 0) {
+    r = lane < W ? warp_part[wid + lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+  }
+  return r;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTailThreads, 1) k_solve17(CtaArgs<T> A) {
+  constexpr bool MIX = sizeof(T) == 4;
+  constexpr int N = 17, N2 = N * N, N3 = N * N2;
+  constexpr int VB = (N2 + 127) / 128;               // k_residual_z's blocks: one z-slab (apply_slabs(17))
+  static_assert(VB * 128 <= kTailThreads, "one column per thread");
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  __shared__ double part[kCtaMaxPartials], part2[kCtaMaxPartials], warp_part[kTailThreads / 32], bcast[2];
+  __shared__ int s_next, cyc, act, go_on;
+  __shared__ double rel;
+  const int tid = threadIdx.x;
+  Solve17<T> S;
+  for (;;) {
+    if (tid == 0) s_next = atomicAdd(A.work, 1);
+    __syncthreads();
+    const int s = s_next;
+    __syncthreads();
+    if (s >= A.B) return;
+    const size_t b0 = (size_t)s * N3;
+    S.load(A, s, reinterpret_cast<T*>(tail_smem));
+    const double* Fx = A.Fx + b0;
+    const double* Fy = A.Fy + b0;
+    const double* Fz = A.Fz + b0;
+    const double* D = A.D + b0;
+    // column z-march of k_residual_z (APPLY: k_apply_dot_z) over v; fn(index, value) stores;
+    // partials of r~^2 (p.q) into part
+    auto zmarch = [&](bool apply, const double* g, auto v, auto store) {
+      double acc = 0.0;
+      const int y = tid / N, x = tid - y * N;
+      const bool col = tid < N2, in = col && x > 0 && y > 0 && x < N - 1 && y < N - 1;
+      if (in) {
+        double pm = v(tid), pc = v(tid + N2), kzm = Fz[tid];
+        static_assert((N - 2) % 3 == 0, "planes in threes");
+        for (int z = 1; z <= N - 2; z += 3) {  // the loads of three planes, then their sums and stores
+          double pp[3], kzp[3], w[3][4], f[3][4], d[3], gg[3], r[3];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const int t = tid + (z + k) * N2;
+            pp[k] = v(t + N2);
+            kzp[k] = Fz[t];
+            f[k][0] = Fx[t - 1];
+            f[k][1] = Fx[t];
+            f[k][2] = Fy[t - N];
+            f[k][3] = Fy[t];
+            w[k][0] = v(t - 1);
+            w[k][1] = v(t + 1);
+            w[k][2] = v(t - N);
+            w[k][3] = v(t + N);
+            d[k] = D[t];
+            gg[k] = apply ? 0.0 : g[t];
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            if (apply) {
+              r[k] = d[k] * pc;
+#pragma unroll
+              for (int q = 0; q < 4; ++q) r[k] = fma(-f[k][q], w[k][q], r[k]);
+              r[k] = fma(-kzm, pm, r[k]);
+              r[k] = fma(-kzp[k], pp[k], r[k]);
+              acc = fma(pc, r[k], acc);
+            } else {
+              r[k] = fma(-d[k], pc, gg[k]);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) r[k] = fma(f[k][q], w[k][q], r[k]);
+              r[k] = fma(kzm, pm, r[k]);
+              r[k] = fma(kzp[k], pp[k], r[k]);
+              acc += r[k] * r[k];
+            }
+            pm = pc;
+            pc = pp[k];
+            kzm = kzp[k];
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k) store(tid + (z + k) * N2, r[k]);
+        }
+      } else if (col) {
+        for (int z = 1; z <= N - 2; ++z) store(tid + z * N2, 0.0);
+      }
+      if (col) {
+        store(tid, 0.0);
+        store(tid + (N - 1) * N2, 0.0);
+      }
+      const double bs = group_sum<4>(acc, warp_part);
+      if ((tid & 127) == 0 && (tid >> 7) < VB) part[tid >> 7] = bs;
+    };
+    // The per-sample scalars live in shared memory and are formed by thread 0 (an FP64 division
+    // by every warp would take the FP64 pipe a tenth of a cycle).
+    const double g2 = A.g2[s];
+    if (tid == 0) {
+      rel = 0.0;
+      cyc = act = 0;
+    }
+    // convergence test of r~^2 = the sum of `count` partials after `inc` cycles: goes on?
+    auto test = [&](int count, int inc) {
+      __syncthreads();
+      if (tid < 32) {
+        const double t = warp_sum_partials(part, count);
+        if (tid == 0) act = cta_norm_update(t, g2, A.rtol, A.maxc, inc, &rel, &cyc);
+      }
+      __syncthreads();
+      return act != 0;
+    };
+    // fn(sum of `count` partials), in every thread
+    auto scalar = [&](const double* p, int count, auto fn) {
+      __syncthreads();
+      if (tid < 32) {
+        const double t = warp_sum_partials(p, count);
+        if (tid == 0) bcast[0] = fn(t);
+      }
+      __syncthreads();
+      return bcast[0];
+    };
+    auto none = [](int, double) {};
+    if (!MIX && A.mode == kCtaStationary) {
+      const double* g = A.g64 + b0;
+      const double* x0 = A.x + b0;
+      for (int i = tid; i < N3; i += kTailThreads) {
+        S.a.g[i] = (T)g[i];
+        S.a.u[i] = (T)x0[i];
+      }
+      __syncthreads();
+      auto u = [&](int i) { return (double)S.a.u[i]; };
+      for (int inc = 0;; inc = 1) {
+        // k_solve_cta's test: the red residuals let a sample go on, the full one stops it
+        if (inc > 0) {
+          const double b = A.rtol > 0.0 ? group_sum<kTailThreads / 32>(S.red_residual(false), warp_part) : 0.0;
+          if (tid == 0) {
+            go_on = cyc + 1 < A.maxc && (A.rtol <= 0.0 || (g2 > 0.0 && sqrt(b / g2) > A.rtol));
+            if (go_on) ++cyc;
+          }
+          __syncthreads();
+        }
+        if (inc == 0 || !go_on) {
+          zmarch(false, g, u, none);
+          if (!test(VB, inc)) break;
+        }
+        S.cycle(A, s, false);
+      }
+      for (int i = tid; i < N3; i += kTailThreads) A.x[b0 + i] = (double)S.a.u[i];
+    } else if (MIX && A.mode == kCtaRefinement) {
+      double* x = A.x + b0;
+      auto xv = [&](int i) { return x[i]; };
+      for (int inc = 0;; inc = 1) {
+        zmarch(false, A.g64 + b0, xv, [&](int i, double r) { S.a.g[i] = (T)r; });
+        if (!test(VB, inc)) break;
+        S.cycle(A, s, true);
+        for (int i = tid; i < N3; i += kTailThreads) x[i] += widen((float)S.a.u[i]);
+        __syncthreads();
+      }
+    } else if (A.mode == kCtaCG) {
+      double *x = A.x + b0, *R = A.R + b0, *P = A.P + b0, *Q = A.Q + b0;
+      const unsigned chunk = ((unsigned)N3 + A.NB - 1) / A.NB;  // NB = 2 chunks of 256 threads' partials
+      const unsigned grp = tid >> 8, lo = grp * chunk, hi = min(lo + chunk, (unsigned)N3);
+      auto z = [&](unsigned i) { return widen(S.a.u[i]); };
+      auto precondition = [&]() {
+        S.cycle(A, s, true);
+        double acc = 0.0;
+        for (unsigned i = lo + (tid & 255); i < hi; i += 256) acc = fma(R[i], z(i), acc);
+        const double b = group_sum<8>(acc, warp_part);
+        if ((tid & 255) == 0) part[grp] = b;
+      };
+      auto same = [](double t) { return t; };
+      double rz = 0.0, rzo = 0.0;
+      zmarch(false, A.g64 + b0, [&](int i) { return x[i]; }, [&](int i, double r) { R[i] = r; });
+      if (test(VB, 0)) {
+        for (int i = tid; i < N3; i += kTailThreads) S.a.g[i] = (T)R[i];
+        __syncthreads();
+        precondition();
+        rz = scalar(part, A.NB, same);
+        for (int i = tid; i < N3; i += kTailThreads) P[i] = z(i);
+        __syncthreads();
+        for (;;) {
+          zmarch(true, nullptr, [&](int i) { return P[i]; }, [&](int i, double q) { Q[i] = q; });
+          const double alpha = scalar(part, VB, [&](double pq) { return pq != 0.0 ? rz / pq : 0.0; });
+          double rr = 0.0, rzp = 0.0;
+          for (unsigned i = lo + (tid & 255); i < hi; i += 256) {
+            x[i] = fma(alpha, P[i], x[i]);
+            const double rn = fma(-alpha, Q[i], R[i]);
+            R[i] = rn;
+            S.a.g[i] = (T)rn;
+            rr = fma(rn, rn, rr);
+            rzp = fma(rn, z(i), rzp);
+          }
+          const double s1 = group_sum<8>(rr, warp_part);
+          const double s2 = group_sum<8>(rzp, warp_part);
+          if ((tid & 255) == 0) {
+            part[grp] = s1;
+            part2[grp] = s2;
+          }
+          rzo = scalar(part2, A.NB, same);
+          if (!test(A.NB, 1)) break;
+          precondition();
+          const double beta = scalar(part, A.NB, [&](double t) {
+            bcast[1] = t;
+            return rz != 0.0 ? (t - rzo) / rz : 0.0;
+          });
+          rz = bcast[1];
+          for (int i = tid; i < N3; i += kTailThreads) P[i] = fma(beta, P[i], z(i));
+          __syncthreads();
+        }
+      }
+    }
+    if (tid == 0) {
+      A.relres[s] = rel;
+      A.cycles[s] = cyc;
+      A.active[s] = act;
+    }
+    __syncthreads();
+  }
+}
+
 template <typename T>
 int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host, double* relres_host,
                int* n_unconv, int* cycles_dev, double* relres_dev) {
@@ -3822,11 +4200,25 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     int dev = 0, sms = 0, per_sm = 0;
     MLMC_CUDA_TRY(cudaGetDevice(&dev));
     MLMC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    MLMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_cta<T>, kCtaThreads, 0));
-    const int grid = B < sms * (per_sm > 0 ? per_sm : 1) ? B : sms * (per_sm > 0 ? per_sm : 1);
     MLMC_CUDA_TRY(cudaMemsetAsync(H.n_active, 0, sizeof(int), st));
-    MLMC_LAUNCH(prof::sized(sizeof(T) == 4 ? "solve_cta_mixed" : "solve_cta_f64", a.n), 0.0, 0.0, st,
-                (k_solve_cta<T><<<grid, kCtaThreads, 0, st>>>(A)));
+    // k_solve17 fills an SM with one sample: always the faster form for FP32 cycles (17^3 x 400
+    // mixed: 1.06 against 1.5 ms), for FP64 ones while every SM has at most one sample (one sample
+    // 0.51 ms, 4096 15.1 against k_solve_cta's 14.3, whose four samples per SM fill the FP64 pipe)
+    if (a.n == 17 && nu1 > 0 && nu2 > 0 && !H.nodal[0] && !H.nodal[1] && A.NB == 2 && A.slabs == 1 && (mixed || B <= sms)) {
+      const size_t smem = Solve17<T>::elems * sizeof(T);
+      static const cudaError_t attr =
+          cudaFuncSetAttribute(k_solve17<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      MLMC_CUDA_TRY(attr);
+      MLMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve17<T>, kTailThreads, smem));
+      const int grid = B < sms * (per_sm > 0 ? per_sm : 1) ? B : sms * (per_sm > 0 ? per_sm : 1);
+      MLMC_LAUNCH(prof::sized(sizeof(T) == 4 ? "solve_cta_mixed" : "solve_cta_f64", a.n), 0.0, 0.0, st,
+                  (k_solve17<T><<<grid, kTailThreads, smem, st>>>(A)));
+    } else {
+      MLMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_cta<T>, kCtaThreads, 0));
+      const int grid = B < sms * (per_sm > 0 ? per_sm : 1) ? B : sms * (per_sm > 0 ? per_sm : 1);
+      MLMC_LAUNCH(prof::sized(sizeof(T) == 4 ? "solve_cta_mixed" : "solve_cta_f64", a.n), 0.0, 0.0, st,
+                  (k_solve_cta<T><<<grid, kCtaThreads, 0, st>>>(A)));
+    }
     MLMC_CUDA_TRY(cudaGetLastError());
   }
   if (cg && !use_cta) {
