@@ -462,6 +462,11 @@ template <int LG>
 struct SplitGeo {
   static constexpr int n = (1 << LG) + 1, m = n - 2, P = (((n + 1) / 2) + 3) & ~3, NP = n * P, BLK = n * n * P;
   static constexpr int Q4 = P / 4;               // four-slot groups per row
+  // four- and two-slot groups that hold an interior node (x = 1 .. n - 2) of either parity: the
+  // passes give threads to these only (of the padded row's 9 four-slot groups at 65^3 to 8, of its
+  // 18 two-slot groups to 16; an idle lane costs the FP64 pipe as much as a busy one: the colour
+  // passes of a 129^3 / 65^3 level of 24 samples 31.0 -> 29.5 ms, FP32 ones of 33^3 x 48 1.15 -> 1.06)
+  static constexpr int A4 = n > 9 ? (n - 1) / 8 : 1, A2 = (n - 1) / 4;
   static constexpr size_t NS = (size_t)2 * BLK;  // elements per sample
 };
 
@@ -533,10 +538,10 @@ __global__ void __launch_bounds__(128) k_rbgs_split(int colour, const float* __r
                                                     const int* __restrict__ active) {
   using G = SplitGeo<LG>;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;  // group of an interior row
-  if (q >= G::m * G::Q4) return;
+  if (q >= G::m * G::A4) return;
   const int s = blockIdx.z;
   if (active && !active[s]) return;
-  const int yi = q / G::Q4, qi = q - yi * G::Q4, y = 1 + yi, z = 1 + (int)blockIdx.y;
+  const int yi = q / G::A4, qi = q - yi * G::A4, y = 1 + yi, z = 1 + (int)blockIdx.y;
   const int par = (colour + y + z) & 1, xi0 = 4 * qi, x0 = 2 * xi0 + par;  // node i: x = x0 + 2 i
   if (x0 > G::n - 2) return;  // boundary and padding slots only
   const int o = (z * G::n + y) * G::P + xi0;
@@ -592,10 +597,10 @@ __global__ void __launch_bounds__(128, 8) k_residual_split(const float* __restri
                                                         const int* __restrict__ active) {
   using G = SplitGeo<LG>;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= G::m * G::Q4) return;
+  if (q >= G::m * G::A4) return;
   const int s = blockIdx.z, colour = RED ? 0 : blockIdx.y & 1;
   if (active && !active[s]) return;
-  const int yi = q / G::Q4, qi = q - yi * G::Q4, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
+  const int yi = q / G::A4, qi = q - yi * G::A4, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
   const int par = (colour + y + z) & 1, xi0 = 4 * qi, x0 = 2 * xi0 + par;
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
@@ -682,10 +687,10 @@ __global__ void __launch_bounds__(128) k_prolong_split(const float* __restrict__
   using F = SplitGeo<LG>;
   using C = SplitGeo<LG - 1>;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= F::m * F::Q4) return;
+  if (q >= F::m * F::A4) return;
   const int s = BLACK ? blockIdx.z : blockIdx.z >> 1, colour = BLACK ? 1 : blockIdx.z & 1;
   if (active && !active[s]) return;
-  const int yi = q / F::Q4, qi = q - yi * F::Q4, y = 1 + yi, z = 1 + (int)blockIdx.y;
+  const int yi = q / F::A4, qi = q - yi * F::A4, y = 1 + yi, z = 1 + (int)blockIdx.y;
   const int xo = (colour + y + z) & 1, xi0 = 4 * qi, x0 = 2 * xi0 + xo;
   if (x0 > F::n - 2) return;
   const int yo = y & 1, zo = z & 1, Y = y >> 1, Z = z >> 1;
@@ -822,12 +827,11 @@ __global__ void __launch_bounds__(128) k_rbgs_split64(int colour, const double* 
                                                       const double* __restrict__ Dinv, const double* __restrict__ g,
                                                       double* __restrict__ u, const int* __restrict__ active) {
   using G = SplitGeo<LG>;
-  constexpr int Q2 = G::P / 2;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= G::m * Q2) return;
+  if (q >= G::m * G::A2) return;
   const int s = blockIdx.z;
   if (active && !active[s]) return;
-  const int yi = q / Q2, qi = q - yi * Q2, y = 1 + yi, z = 1 + (int)blockIdx.y;
+  const int yi = q / G::A2, qi = q - yi * G::A2, y = 1 + yi, z = 1 + (int)blockIdx.y;
   const int par = (colour + y + z) & 1, xi0 = 2 * qi, x0 = 2 * xi0 + par;  // node i: x = x0 + 2 i
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
@@ -896,12 +900,11 @@ __global__ void __launch_bounds__(128) k_residual_split64(const double* __restri
                                                           const double* __restrict__ g, const double* __restrict__ u,
                                                           double* __restrict__ r, const int* __restrict__ active) {
   using G = SplitGeo<LG>;
-  constexpr int Q2 = G::P / 2;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= G::m * Q2) return;
+  if (q >= G::m * G::A2) return;
   const int s = blockIdx.z, colour = RED ? 0 : blockIdx.y & 1;
   if (active && !active[s]) return;
-  const int yi = q / Q2, qi = q - yi * Q2, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
+  const int yi = q / G::A2, qi = q - yi * G::A2, y = 1 + yi, z = 1 + (int)(RED ? blockIdx.y : blockIdx.y >> 1);
   const int par = (colour + y + z) & 1, xi0 = 2 * qi, x0 = 2 * xi0 + par;
   if (x0 > G::n - 2) return;
   const int o = (z * G::n + y) * G::P + xi0;
@@ -1763,15 +1766,14 @@ __global__ void __launch_bounds__(128)
                      const double* __restrict__ Kz, const double* __restrict__ D, const double* __restrict__ g,
                      const double* __restrict__ u, double* __restrict__ partial, const int* __restrict__ active) {
   using G = SplitGeo<LG>;
-  constexpr int Q2 = G::P / 2;
   const int s = blockIdx.z;
   if (!active[s]) return;
   const int q = blockIdx.x * 128 + threadIdx.x;
   const int zlo = 1 + blockIdx.y * zslab, zhi = min(G::n - 2, zlo + zslab - 1);
   const size_t cb = (size_t)s * G::NS, ob = cb + G::BLK;
   double sq = 0.0;
-  if (q < G::m * Q2) {
-    const int yi = q / Q2, qi = q - yi * Q2, y = 1 + yi, xi0 = 2 * qi;
+  if (q < G::m * G::A2) {
+    const int yi = q / G::A2, qi = q - yi * G::A2, y = 1 + yi, xi0 = 2 * qi;
     for (int z = zlo; z <= zhi; ++z) {
       const int par = (y + z) & 1, x0 = 2 * xi0 + par;
       if (x0 > G::n - 2) continue;
@@ -2158,6 +2160,9 @@ struct Names<float> {
   static constexpr const char* coarse = "coarse_apply_f32";
 };
 
+// groups of a colour row with an interior node, `nodes` values of x each (SplitGeo's A4, A2)
+inline int split_groups(int n, int nodes) { return n > nodes + 1 ? (n - 1) / nodes : 1; }
+
 inline double interior(int n) { return (double)(n - 2) * (n - 2) * (n - 2); }
 
 // Red-black sweeps start on red and end on black, and a colour pass reads the other colour
@@ -2527,7 +2532,7 @@ void vcycle_split(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zer
   float* u = (float*)(void*)v.u;
   const float* g = (const float*)(const void*)v.g;
   const float* kn = (const float*)(const void*)v.kn;
-  const dim3 gs((unsigned)((m * (split_pitch(v.n) / 4) + 127) / 128), (unsigned)m, (unsigned)B);
+  const dim3 gs((unsigned)((m * split_groups(v.n, 8) + 127) / 128), (unsigned)m, (unsigned)B);
   auto smooth = [&](int sweeps, bool from_zero) {
     for (int s = 0; s < sweeps; ++s)
       for (int c = 0; c < 2; ++c) {
@@ -2540,7 +2545,7 @@ void vcycle_split(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zer
       }
   };
   smooth(nu1, zero);
-  const unsigned groups = (unsigned)((m * (split_pitch(v.n) / 4) + 127) / 128);
+  const unsigned groups = (unsigned)((m * split_groups(v.n, 8) + 127) / 128);
   float* r = (float*)(void*)v.r;  // colour-split r~ (room for n^2 (n+1) elements: carved as n^3 + slack)
   const dim3 rg((unsigned)(((w.n - 2) * (w.n - 2) + 127) / 128), (unsigned)(w.n - 2), (unsigned)B);
   if (nu1 > 0) {
@@ -2639,7 +2644,7 @@ void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool z
   const double* g = (const double*)(const void*)v.g;
   double* u = (double*)(void*)v.u;
   double* r = (double*)(void*)v.r;
-  const unsigned pairs = (unsigned)((m * (split_pitch(v.n) / 2) + 127) / 128);
+  const unsigned pairs = (unsigned)((m * split_groups(v.n, 4) + 127) / 128);
   const dim3 gs(pairs, (unsigned)m, (unsigned)B);
   auto smooth = [&](int sweeps, bool from_zero) {
     for (int s = 0; s < sweeps; ++s)
@@ -4130,7 +4135,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                   (k_norm_update<<<sb, 128, 0, st>>>(B, H.NBz, H.partial, H.g2, H.relres, H.cycles, H.active, 1, inc,
                                                      rtol, maxc, H.n_active)));
     } else if (inc > 0 && nu1 + nu2 > 0 && H.L > 1) {
-      const int slots = H.split ? (a.n - 2) * (split_pitch(a.n) / 2) : (a.n - 2) * ((a.n - 1) / 2);
+      const int slots = H.split ? (a.n - 2) * split_groups(a.n, 4) : (a.n - 2) * ((a.n - 1) / 2);
       const dim3 rr((unsigned)((slots + 127) / 128), rz.y, (unsigned)B);
       const int NBr = (int)(rr.x * rr.y);
       if (H.split)
