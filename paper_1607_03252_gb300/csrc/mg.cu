@@ -1361,11 +1361,12 @@ __global__ void k_qoi_final(int B, int NB, double scale, const double* __restric
 //   K_a(P) = (k_P + k_{P+a}) / 4 + (k_{P+a+b} + k_{P+a+c} + k_{P+a+b+c} + k_{P-b} + k_{P-c}
 //            + k_{P-b-c}) / 12      ({a, b, c} = {x, y, z}),
 // in the h^2-scaled form (FE matrix / h); the load of f = 1 is h^3 per interior node, the
-// g = h^2 f of the scaled form.
+// g = h^2 f of the scaled form. split: the faces go straight to colour-split storage (assembled in
+// plain arrays and copied, a 65^3 / 33^3 FMG level of 108 samples took 0.9 of its 17.6 ms longer).
 // ---------------------------------------------------------------------------------
 template <typename T>
 __global__ void k_faces_fe(const double* __restrict__ k0, int n0, int st0, int n, int B, T* __restrict__ Kx,
-                           T* __restrict__ Ky, T* __restrict__ Kz) {
+                           T* __restrict__ Ky, T* __restrict__ Kz, int split = 0) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;  // node of the plane
   if (q >= n * n) return;
   const int y = q / n, x = q - y * n;
@@ -1377,7 +1378,7 @@ __global__ void k_faces_fe(const double* __restrict__ k0, int n0, int st0, int n
       return kb[((size_t)(st0 * (z + dz)) * n0 + (size_t)(st0 * (y + dy))) * n0 + (size_t)(st0 * (x + dx))];
     };
     const bool ix = x >= 1 && x <= n - 2, iy = y >= 1 && y <= n - 2, iz = z >= 1 && z <= n - 2;
-    const size_t t = (size_t)s * n3 + (size_t)(z * n * n + q);
+    const size_t t = split ? (size_t)s * split_elems(n) + split_index(n, x, y, z) : (size_t)s * n3 + (size_t)(z * n * n + q);
     double fx = 0.0, fy = 0.0, fz = 0.0;
     if (x <= n - 2 && iy && iz)
       fx = (K(0, 0, 0) + K(1, 0, 0)) * 0.25 +
@@ -3970,17 +3971,12 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
       if (j < H.L - 1) {
         if constexpr (sizeof(T) == 8) {
           // FP64: stored faces, D and 1/D in the split storage (the coarsest grid keeps the
-          // plain faces its dense factorisation reads); P1 faces are assembled in the plain
-          // layout into the level's spare arrays and copied over
+          // plain faces its dense factorisation reads)
           if (a.cfg.disc == MLMC_DISC_FE) {
-            double* t[3] = {(double*)(void*)v.u2, (double*)(void*)v.r, (double*)(void*)v.u};
             MLMC_LAUNCH("faces_fe", B * (double)v.n3 * (8.0 + 3 * W), B * (double)v.n3 * 36.0, st,
-                        (k_faces_fe<double><<<gb, kPlaneThreads, 0, st>>>(a.k0, a.n_k0, stride, v.n, B, t[0], t[1],
-                                                                          t[2])));
-            double* K[3] = {(double*)(void*)v.Kx, (double*)(void*)v.Ky, (double*)(void*)v.Kz};
-            for (int d = 0; d < 3; ++d)
-              MLMC_LAUNCH("split_copy", B * (double)v.n3 * 16.0, 0.0, st,
-                          (k_split_copy<double, true><<<gb, kPlaneThreads, 0, st>>>(v.n, B, t[d], K[d])));
+                        (k_faces_fe<double><<<gb, kPlaneThreads, 0, st>>>(a.k0, a.n_k0, stride, v.n, B,
+                                                                          (double*)(void*)v.Kx, (double*)(void*)v.Ky,
+                                                                          (double*)(void*)v.Kz, 1)));
           } else {
             MLMC_LAUNCH(Names<T>::faces, B * (double)v.n3 * (8.0 + 3 * W), B * (double)v.n3 * 12.0, st,
                         (k_faces_split<<<gb, kPlaneThreads, 0, st>>>(a.k0, a.n_k0, stride, v.n, B, (double*)v.Kx,
