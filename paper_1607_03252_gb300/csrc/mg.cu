@@ -1037,11 +1037,11 @@ __device__ __forceinline__ double warp_sum_partials(const double* __restrict__ p
 
 // Per sample: total of the NB partials (fixed order). mode 0: store ||g||^2.
 // mode 1: relative residual, cycle count and active flag after `inc` cycles, of the active
-// samples (of those that `mask` names, if it is given).
+// samples (of those that `mask` names, if it is given; mask then names those of them that go on).
 __global__ void k_norm_update(int B, int NB, const double* __restrict__ partial, double* __restrict__ g2,
                               double* __restrict__ relres, int* __restrict__ cycles, int* __restrict__ active,
                               int mode, int inc, double rtol, int max_cycles, int* __restrict__ n_active,
-                              const int* __restrict__ mask = nullptr) {
+                              int* __restrict__ mask = nullptr) {
   const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp per sample
   if (s >= B) return;
   if (mode == 1 && !(mask ? mask[s] : active[s])) return;
@@ -1057,11 +1057,21 @@ __global__ void k_norm_update(int B, int NB, const double* __restrict__ partial,
   const int c = cycles[s];
   const int still = (rtol > 0.0) ? (rel > rtol && c < max_cycles) : (c < max_cycles);
   active[s] = still;
+  if (mask) mask[s] = still;
   if (still) atomicAdd(n_active, 1);
 }
 
+// What the red residuals' norm has to exceed for a sample to go on without the full test. Formed
+// in the full residual's order of operations (fused = false) they can differ from their part of it
+// by the order of the sum alone. Formed along with a red pass (fused) each differs by rounding too:
+// about 2^-55 (n - 1)^2 of |g| for a coefficient of order one, at most a sixteenth of the tolerances
+// that red_fused takes, so an eighth on top leaves the answer to the full test wherever rounding
+// could change it, and below those tolerances every test is a full one.
+__host__ __device__ inline double red_limit(double rtol, bool fused) { return rtol * (fused ? 1.125 : 1.0 + 1e-9); }
+inline bool red_fused(double rtol, int n) { return rtol >= 0x1p-51 * (n - 1) * (n - 1); }
+
 // After `inc` more cycles, from the partials of the red residuals alone (a lower bound of the
-// norm): a sample whose red residual still exceeds rtol, and which has cycles left, goes on
+// norm): a sample whose red residual exceeds `rtol` (red_limit), and which has cycles left, goes on
 // (n_active[0]); the others are candidates to stop (cand, n_active[1]), for which the full
 // residual decides (k_norm_update).
 __global__ void k_norm_red(int B, int NB, const double* __restrict__ partial, const double* __restrict__ g2,
@@ -1742,7 +1752,8 @@ __global__ void __launch_bounds__(128)
 // half the work decides whether a sample goes on. Bound by the FP64 pipe (8 operations per red
 // node). A thread takes one red slot of a plane (the split form a pair of slots on 16-byte
 // loads) through a z-slab; the partition is a function of n only. Grid (slot blocks, z-slabs,
-// samples), 128 threads.
+// samples), 128 threads. (Plain storage; the split form below takes the test along with the next
+// cycle's first red pass.)
 template <typename T>
 __global__ void __launch_bounds__(128)
     k_norm_red_z(int n, int zslab, const T* __restrict__ Kx, const T* __restrict__ Ky, const T* __restrict__ Kz,
@@ -1775,11 +1786,18 @@ __global__ void __launch_bounds__(128)
   if (threadIdx.x == 0) partial[((size_t)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = b;
 }
 
+// The next cycle's first red pass (k_rbgs_split64's operations) on colour-split storage with the
+// red residuals it passes by: with acc = g + sum K u_q, the residual is acc - D u and the update
+// acc / D, so the test costs two FP64 operations per red node instead of eight (212 us a launch on a
+// 129^3 / 65^3 level of 24 samples, 0.93 TFLOP/s; the pass alone 150, the test alone 184). The replaced red
+// values go to `old` (one colour block per sample) for the samples that turn out to be done
+// (k_restore_red).
 template <int LG>
 __global__ void __launch_bounds__(128)
-    k_norm_red_split(int zslab, const double* __restrict__ Kx, const double* __restrict__ Ky,
-                     const double* __restrict__ Kz, const double* __restrict__ D, const double* __restrict__ g,
-                     const double* __restrict__ u, double* __restrict__ partial, const int* __restrict__ active) {
+    k_rbgs_norm_split(int zslab, const double* __restrict__ Kx, const double* __restrict__ Ky,
+                      const double* __restrict__ Kz, const double* __restrict__ D, const double* __restrict__ Dinv,
+                      const double* __restrict__ g, double* __restrict__ u, double* __restrict__ old,
+                      double* __restrict__ partial, const int* __restrict__ active) {
   using G = SplitGeo<LG>;
   const int s = blockIdx.z;
   if (!active[s]) return;
@@ -1794,7 +1812,7 @@ __global__ void __launch_bounds__(128)
       if (x0 > G::n - 2) continue;
       const int o = (z * G::n + y) * G::P + xi0;
       const double2 kx2 = ld2(Kx + cb + o), ky2 = ld2(Ky + cb + o), kz2 = ld2(Kz + cb + o);
-      const double2 d2 = ld2(D + cb + o), g2 = ld2(g + cb + o), up2 = ld2(u + cb + o);
+      const double2 d2 = ld2(D + cb + o), di2 = ld2(Dinv + cb + o), g2 = ld2(g + cb + o), up2 = ld2(u + cb + o);
       const double* uo = u + ob;
       const double2 kxm2 = ld2(Kx + ob + o), kym2 = ld2(Ky + ob + o - G::P), kzm2 = ld2(Kz + ob + o - G::NP);
       const double2 um2 = ld2(uo + o), uym2 = ld2(uo + o - G::P), uyp2 = ld2(uo + o + G::P);
@@ -1806,25 +1824,43 @@ __global__ void __launch_bounds__(128)
         kext = Kx[ob + o - 1];
         uext = uo[o - 1];
       }
+      *reinterpret_cast<double2*>(old + (size_t)s * G::BLK + o) = up2;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         if (x0 + 2 * i < 1 || x0 + 2 * i > G::n - 2) continue;
         const double kl = par ? comp2(kxm2, i) : (i == 0 ? kext : comp2(kxm2, i - 1));
         const double ul = par ? comp2(um2, i) : (i == 0 ? uext : comp2(um2, i - 1));
         const double ur = par ? (i == 1 ? uext : comp2(um2, i + 1)) : comp2(um2, i);
-        double rr = fma(-comp2(d2, i), comp2(up2, i), comp2(g2, i));
-        rr = fma(kl, ul, rr);
-        rr = fma(comp2(kx2, i), ur, rr);
-        rr = fma(comp2(kym2, i), comp2(uym2, i), rr);
-        rr = fma(comp2(ky2, i), comp2(uyp2, i), rr);
-        rr = fma(comp2(kzm2, i), comp2(uzm2, i), rr);
-        rr = fma(comp2(kz2, i), comp2(uzp2, i), rr);
+        double acc = comp2(g2, i);
+        acc = fma(kl, ul, acc);
+        acc = fma(comp2(kx2, i), ur, acc);
+        acc = fma(comp2(kym2, i), comp2(uym2, i), acc);
+        acc = fma(comp2(ky2, i), comp2(uyp2, i), acc);
+        acc = fma(comp2(kzm2, i), comp2(uzm2, i), acc);
+        acc = fma(comp2(kz2, i), comp2(uzp2, i), acc);
+        const double rr = fma(-comp2(d2, i), comp2(up2, i), acc);
         sq = fma(rr, rr, sq);
+        u[cb + o + i] = acc * comp2(di2, i);
       }
     }
   }
   const double b = block_sum<128>(sq);
   if (threadIdx.x == 0) partial[((size_t)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = b;
+}
+
+// Puts back the interior red values that k_rbgs_norm_split replaced, for the samples in `cand`.
+// Grid (two-slot groups of the interior rows of a plane, interior planes, samples).
+template <int LG>
+__global__ void __launch_bounds__(128) k_restore_red(const double* __restrict__ old, double* __restrict__ u,
+                                                     const int* __restrict__ cand) {
+  using G = SplitGeo<LG>;
+  const int s = blockIdx.z, q = blockIdx.x * 128 + threadIdx.x;
+  if (!cand[s] || q >= G::m * G::A2) return;
+  const int yi = q / G::A2, xi0 = 2 * (q - yi * G::A2), y = 1 + yi, z = 1 + (int)blockIdx.y;
+  const int x0 = 2 * xi0 + ((y + z) & 1), o = (z * G::n + y) * G::P + xi0;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (x0 + 2 * i >= 1 && x0 + 2 * i <= G::n - 2) u[(size_t)s * G::NS + o + i] = old[(size_t)s * G::BLK + o + i];
 }
 
 inline dim3 zmarch_grid(int n, int B, int* zslab) {
@@ -2205,8 +2241,9 @@ cudaError_t clear_guess(const Hier<T>& H, int j, int nu1, cudaStream_t st) {
 }
 
 // zero: u is zero on entry (cleared by clear_guess, where that is needed).
+// red_done: the first red pass has been taken already (finest grid, k_rbgs_norm_split).
 template <typename T>
-void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero);
+void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero, bool red_done = false);
 
 // ---------------------------------------------------------------------------------
 // The V-cycle below a grid of at most 17^3 nodes as one launch, one block per sample.
@@ -2645,7 +2682,7 @@ void prolong_level(Hier<T>& H, int j, bool black, cudaStream_t st) {
 // sweeps, the residual into split r, full weighting into the coarse split g, the coarser
 // levels, the trilinear correction on split storage, post-smoothing.
 template <typename T>
-void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
+void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero, bool red_done) {
   Level<T>& v = H.lv[j];
   Level<T>& w = H.lv[j + 1];
   const int* act = H.active;
@@ -2661,9 +2698,10 @@ void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool z
   double* r = (double*)(void*)v.r;
   const unsigned pairs = (unsigned)((m * split_groups(v.n, 4) + 127) / 128);
   const dim3 gs(pairs, (unsigned)m, (unsigned)B);
-  auto smooth = [&](int sweeps, bool from_zero) {
+  auto smooth = [&](int sweeps, bool from_zero, bool skip_red) {
     for (int s = 0; s < sweeps; ++s)
       for (int c = 0; c < 2; ++c) {
+        if (skip_red && s == 0 && c == 0) continue;
         if (from_zero && s == 0 && c == 0)
           MLMC_LAUNCH(prof::sized("rbgs_split_f64", v.n), Ba * interior(v.n) * 1.5 * W, Ba * interior(v.n) * 0.5, st,
                       MLMC_SPLIT_DISPATCH(v.n, (k_rbgs_split64<LG, true><<<gs, 128, 0, st>>>(c, Kx, Ky, Kz, Dinv, g, u,
@@ -2674,7 +2712,7 @@ void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool z
                                                                                          act))));
       }
   };
-  smooth(nu1, zero);
+  smooth(nu1, zero, red_done);
   const bool red = nu1 > 0, black = nu2 > 0;
   double* gc = (double*)(void*)w.g;
   if (red)
@@ -2703,11 +2741,11 @@ void vcycle_split64(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool z
   clear_guess(H, j + 1, nu1, st);
   vcycle(H, j + 1, nu1, nu2, st, true);
   prolong_level(H, j, black, st);
-  smooth(nu2, false);
+  smooth(nu2, false, false);
 }
 
 template <typename T>
-void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
+void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero, bool red_done) {
   Level<T>& v = H.lv[j];
   const int* act = H.active;
   const int B = H.B;
@@ -2732,7 +2770,7 @@ void vcycle(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero) {
     if constexpr (sizeof(T) == 4)
       vcycle_split(H, j, nu1, nu2, st, zero);
     else
-      vcycle_split64(H, j, nu1, nu2, st, zero);
+      vcycle_split64(H, j, nu1, nu2, st, zero, red_done);
     return;
   }
   const int m = v.n - 2;
@@ -2850,17 +2888,17 @@ struct GraphRunner {
   ~GraphRunner() {
     if (exec) cudaGraphExecDestroy(exec);
   }
-  // one V-cycle from grid j0, from a zero guess or not (the same j0 and zero on every call of
-  // one runner)
-  int run(Hier<T>& H, int nu1, int nu2, cudaStream_t st, bool zero, int j0 = 0) {
+  // one V-cycle from grid j0, from a zero guess or not, with its first red pass or without (the
+  // same on every call of one runner)
+  int run(Hier<T>& H, int nu1, int nu2, cudaStream_t st, bool zero, int j0 = 0, bool red_done = false) {
     if (!enabled) {
-      vcycle<T>(H, j0, nu1, nu2, st, zero);
+      vcycle<T>(H, j0, nu1, nu2, st, zero, red_done);
       return MLMC_OK;
     }
     if (!exec) {
       MLMC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       prof::tape_begin();
-      vcycle<T>(H, j0, nu1, nu2, st, zero);
+      vcycle<T>(H, j0, nu1, nu2, st, zero, red_done);
       tape = prof::tape_end();
       cap_act = H.n_act > 0 ? H.n_act : 1;
       cudaGraph_t graph = nullptr;
@@ -3043,7 +3081,8 @@ enum { kCtaStationary = 0, kCtaRefinement = 1, kCtaCG = 2 };
 template <typename T>
 struct CtaArgs {
   int L = 0, B = 0, nu1 = 2, nu2 = 2, maxc = 1, mode = 0;
-  double rtol = 0.0;
+  double rtol = 0.0, red_limit = 0.0;
+  int red_fused = 0;
   CtaLevel<T> lv[4];
   const double* Ainv = nullptr;
   // outer FP64 operator (FP64 faces and diagonal of the finest grid), right-hand side, iterate
@@ -3234,12 +3273,14 @@ __device__ void cta_prolong(const CtaLevel<T>& w, const CtaLevel<T>& v, int s) {
 
 // zero: the finest iterate is zero on entry (its interior need not be: with pre-smoothing
 // the first red pass does not read it)
+// red_done: the finest grid's first red pass has been taken (cta_red_pass_norm)
 template <typename T>
-__device__ void cta_vcycle(const CtaArgs<T>& A, int s, bool zero) {
+__device__ void cta_vcycle(const CtaArgs<T>& A, int s, bool zero, bool red_done = false) {
   // down: smoothing, residual, restriction
   for (int j = 0; j < A.L - 1; ++j) {
     for (int k = 0; k < A.nu1; ++k)
       for (int c = 0; c < 2; ++c) {
+        if (red_done && j == 0 && k == 0 && c == 0) continue;
         if (k == 0 && c == 0 && (j > 0 || zero))
           cta_smooth<T, true>(A.lv[j], s, c);
         else
@@ -3361,12 +3402,14 @@ __device__ double cta_zmarch(const double* __restrict__ Fx, const double* __rest
   return *bcast;
 }
 
-// Sum of r~^2 over the red nodes of sample s (k_norm_red_z's operations), the same in every
-// thread.
+// The finest grid's red pass of sample s (cta_smooth's operations) with the sum of the squared red
+// residuals it passes by (k_rbgs_norm_split), the same in every thread; the replaced values go to
+// the grid's residual array, which the cycle has not written yet.
 template <typename T>
-__device__ double cta_red_norm(const CtaLevel<T>& v, const T* __restrict__ x, int s, double* bcast) {
+__device__ double cta_red_pass_norm(const CtaLevel<T>& v, int s, double* bcast) {
   const int n = v.n, m = n - 2, half = (n - 1) / 2, lh = 31 - __clz(half), per = m * half;
   const size_t n3 = (size_t)n * n * n, n2 = (size_t)n * n;
+  T* u = v.u;
   double sq = 0.0;
   for (int it = threadIdx.x; it < per * m; it += kCtaThreads) {
     const int zi = it / per, q = it - zi * per;
@@ -3374,20 +3417,36 @@ __device__ double cta_red_norm(const CtaLevel<T>& v, const T* __restrict__ x, in
     const int xx = 1 + ((y + z + 1) & 1) + 2 * xi;
     if (xx > n - 2) continue;
     const size_t p = (size_t)s * n3 + (size_t)(z * n * n + y * n + xx);
-    T rr = fma(-v.D[p], x[p], v.g[p]);
-    rr = fma(v.Kx[p - 1], x[p - 1], rr);
-    rr = fma(v.Kx[p], x[p + 1], rr);
-    rr = fma(v.Ky[p - n], x[p - n], rr);
-    rr = fma(v.Ky[p], x[p + n], rr);
-    rr = fma(v.Kz[p - n2], x[p - n2], rr);
-    rr = fma(v.Kz[p], x[p + n2], rr);
+    T acc = v.g[p];
+    acc = fma(v.Kx[p - 1], u[p - 1], acc);
+    acc = fma(v.Kx[p], u[p + 1], acc);
+    acc = fma(v.Ky[p - n], u[p - n], acc);
+    acc = fma(v.Ky[p], u[p + n], acc);
+    acc = fma(v.Kz[p - n2], u[p - n2], acc);
+    acc = fma(v.Kz[p], u[p + n2], acc);
+    const T up = u[p], rr = fma(-v.D[p], up, acc);
     sq += (double)rr * (double)rr;
+    v.r[p] = up;
+    u[p] = acc * v.Dinv[p];
   }
   const double b = block_sum<kCtaThreads>(sq);
   __syncthreads();
   if (threadIdx.x == 0) *bcast = b;
   __syncthreads();
   return *bcast;
+}
+
+// Puts the replaced red values back.
+template <typename T>
+__device__ void cta_restore_red(const CtaLevel<T>& v, int s) {
+  const int n = v.n, m = n - 2;
+  const size_t b = (size_t)s * n * n * n;
+  for (int it = threadIdx.x; it < m * m * m; it += kCtaThreads) {
+    const int z = 1 + it / (m * m), q = it - (z - 1) * m * m, y = 1 + q / m, x = 1 + q - (y - 1) * m;
+    const size_t p = b + (size_t)((z * n + y) * n + x);
+    if (!((x + y + z) & 1)) v.u[p] = v.r[p];
+  }
+  __syncthreads();
 }
 
 // convergence bookkeeping of one sample (k_norm_update, mode 1); returns the active flag
@@ -3416,14 +3475,15 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
     int cyc = 0, act = 0;
     if (A.mode == kCtaStationary) {
       // FP64 V-cycles on the level-0 iterate until the residual test passes
-      const bool sweeps = A.nu1 + A.nu2 > 0 && A.L > 1;
       for (int inc = 0;; inc = 1) {
-        // after a cycle the red residuals decide whether the sample goes on, the full one
-        // whether it is done (the batched test); fixed cycles need the last residual alone
-        bool go = inc > 0 && A.rtol <= 0.0 && cyc + 1 < A.maxc;
-        if (inc > 0 && A.rtol > 0.0 && sweeps && cyc + 1 < A.maxc) {
-          const double tr = cta_red_norm<T>(A.lv[0], A.lv[0].u, s, bcast);
-          go = g2 > 0.0 && sqrt(tr / g2) > A.rtol;
+        // after a cycle the red residuals, taken along with the next cycle's first red pass, decide
+        // whether the sample goes on; the full one whether it is done (the batched test); fixed
+        // cycles need the last residual alone
+        bool go = inc > 0 && A.rtol <= 0.0 && cyc + 1 < A.maxc, red_done = false;
+        if (inc > 0 && A.red_fused && A.nu1 > 0 && A.L > 1 && cyc + 1 < A.maxc) {
+          const double tr = cta_red_pass_norm<T>(A.lv[0], s, bcast);
+          go = red_done = g2 > 0.0 && sqrt(tr / g2) > A.red_limit;
+          if (!go) cta_restore_red<T>(A.lv[0], s);
         }
         if (go) {
           ++cyc;
@@ -3433,7 +3493,7 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
           act = cta_norm_update(t, g2, A.rtol, A.maxc, inc, &rel, &cyc);
           if (!act) break;
         }
-        cta_vcycle(A, s, false);
+        cta_vcycle(A, s, false, red_done);
       }
     } else if (A.mode == kCtaRefinement) {
       // FP32 V-cycles on FP64 residuals: r32 = g - A x, e = V(r32), x += e
@@ -3848,7 +3908,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_solve17(CtaArgs<T> A) {
         if (inc > 0) {
           const double b = A.rtol > 0.0 ? group_sum<kTailThreads / 32>(S.red_residual(false), warp_part) : 0.0;
           if (tid == 0) {
-            go_on = cyc + 1 < A.maxc && (A.rtol <= 0.0 || (g2 > 0.0 && sqrt(b / g2) > A.rtol));
+            go_on = cyc + 1 < A.maxc && (A.rtol <= 0.0 || (g2 > 0.0 && sqrt(b / g2) > red_limit(A.rtol, false)));
             if (go_on) ++cyc;
           }
           __syncthreads();
@@ -4106,7 +4166,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   const dim3 rz = zmarch_grid(a.n, B, &zs);
   // FP64 stationary cycles: the full residual of the samples that `mask` names (all active
   // ones), its norm and the samples that go on, added to n_active[0]
-  auto full_check = [&](int inc, const int* mask, int count) {
+  auto full_check = [&](int inc, int* mask, int count) {
     const double Ba = (double)count;
     const int* on = mask ? mask : H.active;
     if (H.split)
@@ -4122,11 +4182,26 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                 (k_norm_update<<<sb, 128, 0, st>>>(B, H.NBz, H.partial, H.g2, H.relres, H.cycles, H.active, 1, inc,
                                                    rtol, maxc, H.n_active, mask)));
   };
+  // FP64 stationary cycles on colour-split storage take the cycle's first red pass outside the
+  // cycle: with the convergence test of the cycle before (k_rbgs_norm_split), or on its own for
+  // the samples that `mask` names. Its replaced values go to the finest grid's spare iterate.
+  const bool red_first = !mixed && !cg && !fmg && H.split && nu1 > 0 && red_fused(rtol, a.n);
+  auto red_pass = [&](const int* mask, int count) {
+    if constexpr (sizeof(T) == 8) {
+      const dim3 gp((unsigned)(((a.n - 2) * split_groups(a.n, 4) + 127) / 128), (unsigned)(a.n - 2), (unsigned)B);
+      MLMC_LAUNCH(prof::sized("rbgs_split_f64", a.n), (double)count * interior(a.n) * 3.5 * W,
+                  (double)count * interior(a.n) * 0.5 * 13.0, st,
+                  MLMC_SPLIT_DISPATCH(a.n, (k_rbgs_split64<LG><<<gp, 128, 0, st>>>(0, l0.Kx, l0.Ky, l0.Kz, l0.Dinv,
+                                                                                 l0.g, l0.u, mask))));
+    }
+  };
   // Convergence test after `inc` cycles; returns the samples that go on. After an FP64 cycle
   // that ends on a black pass the red residuals decide for the samples that go on (half the FP64
   // work), the full residual for those that seem done, so cycle counts and reported residuals
-  // are those of a full test every cycle. The test of the 129^3 / 65^3 level of 24 samples took
-  // 8.25 ms and takes 6.0 (the level 75.6 -> 66.0 ms), of 65^3 x 19 0.84 and 0.75.
+  // are those of a full test every cycle. On colour-split storage the red residuals come with the
+  // next cycle's first red pass. A 129^3 / 65^3 level of 24 samples: 75.6 ms with full tests, 66.0
+  // on the red residuals; later 54.8 -> 52.5 with the pass and its test in one (6.3 ms of tests,
+  // 3.3 of them the pass); 65^3 x 19 6.72 -> 6.47.
   auto residual_check = [&](int inc) -> int {
     MLMC_CUDA_TRY(cudaMemsetAsync(H.n_active, 0, 2 * sizeof(int), st));
     const double Ba = (double)H.n_act;
@@ -4145,26 +4220,46 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                   (k_norm_update<<<sb, 128, 0, st>>>(B, H.NBz, H.partial, H.g2, H.relres, H.cycles, H.active, 1, inc,
                                                      rtol, maxc, H.n_active)));
     } else if (inc > 0 && nu1 + nu2 > 0 && H.L > 1) {
-      const int slots = H.split ? (a.n - 2) * split_groups(a.n, 4) : (a.n - 2) * ((a.n - 1) / 2);
+      const bool fused = red_first;
+      const int slots = fused ? (a.n - 2) * split_groups(a.n, 4) : (a.n - 2) * ((a.n - 1) / 2);
       const dim3 rr((unsigned)((slots + 127) / 128), rz.y, (unsigned)B);
       const int NBr = (int)(rr.x * rr.y);
-      if (H.split)
-        MLMC_LAUNCH("residual_norm_red", Ba * interior(a.n) * 4.0 * 8, Ba * interior(a.n) * 8.0, st,
-                    MLMC_SPLIT_DISPATCH(a.n, (k_norm_red_split<LG><<<rr, 128, 0, st>>>(
-                                                 zs, (const double*)l0.Kx, (const double*)l0.Ky,
-                                                 (const double*)l0.Kz, (const double*)l0.D, (const double*)l0.g,
-                                                 (const double*)l0.u, H.partial, H.active))));
-      else
+      if (H.split && !fused) {  // no pre-smoothing: the full residual
+        full_check(inc, nullptr, H.n_act);
+        MLMC_CUDA_TRY(cudaMemcpyAsync(na, H.n_active, sizeof(na), cudaMemcpyDeviceToHost, st));
+        MLMC_CUDA_TRY(cudaStreamSynchronize(st));
+        return H.n_act = na[0];
+      }
+      if constexpr (sizeof(T) == 8) {
+        if (fused)
+          MLMC_LAUNCH("rbgs_norm_f64", Ba * interior(a.n) * 4.5 * 8, Ba * interior(a.n) * 8.5, st,
+                      MLMC_SPLIT_DISPATCH(a.n, (k_rbgs_norm_split<LG><<<rr, 128, 0, st>>>(
+                                                   zs, l0.Kx, l0.Ky, l0.Kz, l0.D, l0.Dinv, l0.g, l0.u, l0.u2,
+                                                   H.partial, H.active))));
+      }
+      if (!fused)
         MLMC_LAUNCH("residual_norm_red", Ba * interior(a.n) * 4.0 * 8, Ba * interior(a.n) * 8.0, st,
                     (k_norm_red_z<T><<<rr, 128, 0, st>>>(a.n, zs, l0.Kx, l0.Ky, l0.Kz, l0.D, l0.g, l0.u, H.partial,
                                                          H.active)));
       MLMC_LAUNCH("norm_update", B * NBr * 8.0, B * NBr * 1.0, st,
-                  (k_norm_red<<<sb, 128, 0, st>>>(B, NBr, H.partial, H.g2, H.cycles, H.active, H.cand, inc, rtol,
-                                                  maxc, H.n_active)));
+                  (k_norm_red<<<sb, 128, 0, st>>>(B, NBr, H.partial, H.g2, H.cycles, H.active, H.cand, inc,
+                                                  red_limit(rtol, fused), maxc, H.n_active)));
       MLMC_CUDA_TRY(cudaMemcpyAsync(na, H.n_active, sizeof(na), cudaMemcpyDeviceToHost, st));
       MLMC_CUDA_TRY(cudaStreamSynchronize(st));
       if (na[1] == 0) return H.n_act = na[0];
+      if constexpr (sizeof(T) == 8) {
+        if (fused) {
+          const dim3 gp((unsigned)((slots + 127) / 128), (unsigned)(a.n - 2), (unsigned)B);
+          MLMC_LAUNCH("restore_red", (double)na[1] * interior(a.n) * 8.0, 0.0, st,
+                      MLMC_SPLIT_DISPATCH(a.n, (k_restore_red<LG><<<gp, 128, 0, st>>>(l0.u2, l0.u, H.cand))));
+        }
+      }
+      const int on = na[0];
       full_check(0, H.cand, na[1]);
+      MLMC_CUDA_TRY(cudaMemcpyAsync(na, H.n_active, sizeof(na), cudaMemcpyDeviceToHost, st));
+      MLMC_CUDA_TRY(cudaStreamSynchronize(st));
+      if (fused && na[0] > on) red_pass(H.cand, na[0] - on);  // candidates that go on after all
+      return H.n_act = na[0];
     } else {
       full_check(inc, nullptr, H.n_act);
     }
@@ -4180,6 +4275,8 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     A.nu2 = nu2;
     A.maxc = maxc;
     A.rtol = rtol;
+    A.red_limit = red_limit(rtol, true);
+    A.red_fused = red_fused(rtol, a.n);
     A.mode = cg ? kCtaCG : (mixed ? kCtaRefinement : kCtaStationary);
     for (int j = 0; j < H.L; ++j) {
       Level<T>& v = H.lv[j];
@@ -4285,6 +4382,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   }
   int na = cycling && (mixed || rtol > 0.0) ? residual_check(0) : 0;
   if (na < 0) return na;
+  bool first_cycle = true;
   while (na > 0) {
     if (mixed) {
       MLMC_CUDA_TRY(clear_guess(H, 0, nu1, st));
@@ -4299,7 +4397,9 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
                     (k_update_mixed<false><<<ug, kPlaneThreads, 0, st>>>(a.n, B, (const float*)H.lv[0].u, a.u,
                                                                            H.active)));
     } else {
-      MLMC_TRY(gr.run(H, nu1, nu2, st, false));
+      if (red_first && first_cycle) red_pass(H.active, H.n_act);
+      first_cycle = false;
+      MLMC_TRY(gr.run(H, nu1, nu2, st, false, 0, red_first));
     }
     na = residual_check(1);
     if (na < 0) return na;
