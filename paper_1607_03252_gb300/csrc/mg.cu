@@ -1905,10 +1905,13 @@ struct FlatWalk {
 // finest grid's iterate (MIX; SPLIT: in colour-split storage), or the FP64 one.
 template <bool MIX, bool SPLIT>
 struct PrecondZ {
+  using Raw = typename std::conditional<MIX, float, double>::type;
   const void* z;
+  __device__ __forceinline__ Raw raw(int n, int s, size_t n3, unsigned i, const FlatWalk<SPLIT>& w) const {
+    return __ldg((const Raw*)z + (size_t)s * (SPLIT ? split_elems(n) : n3) + w.at(i));
+  }
   __device__ __forceinline__ double at(int n, int s, size_t n3, unsigned i, const FlatWalk<SPLIT>& w) const {
-    if (MIX) return widen(__ldg((const float*)z + (size_t)s * (SPLIT ? split_elems(n) : n3) + w.at(i)));
-    return ((const double*)z)[(size_t)s * n3 + i];
+    return widen(raw(n, s, n3, i, w));
   }
 };
 
@@ -1916,7 +1919,7 @@ struct PrecondZ {
 // previous preconditioned residual). The last block of a sample sums them and decides: the
 // relative residual, the cycle count, whether the sample goes on (n_active) or is done with this
 // iteration (fin, for k_cg_finish), and r.z (rzo). x is updated with p in k_p_update, which reads
-// p anyway: 32 instead of 60 bytes per node here, bound by HBM. Grid (NB, B).
+// p anyway: 32 instead of 60 bytes per node here. Grid (NB, B).
 template <bool MIX, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 4)
     k_cg_update(int n, const double* __restrict__ alpha, const double* __restrict__ q, double* __restrict__ r,
@@ -1938,30 +1941,48 @@ __global__ void __launch_bounds__(kThreads, 4)
   float* f = MIX ? r32 + (size_t)s * (SPLIT ? split_elems(n) : (size_t)n3) : nullptr;
   const double* qs = q + (size_t)s * n3;
   double* rs = r + (size_t)s * n3;
-  // four nodes a thread at a time: all their loads before the stores
-  for (unsigned i = lo + threadIdx.x; i < hi;) {
-    double qv[4], rv[4], zv[4];
-    size_t fo[4];
-    unsigned t[4];
+  // Two nodes a thread at a time, the next two loaded before these are computed: with four loaded
+  // together every warp of the SM waited for memory at once and then queued at the FP64 pipe at once
+  // (257^3 x 1: 152 -> 143 us a
+  // launch, x 2: 163 -> 149; its three FP64 operations a node take 96 of them).
+  struct Nodes {
+    double q[2], r[2];
+    typename PrecondZ<MIX, SPLIT>::Raw z[2];
+    size_t f[2];
+    unsigned i[2];
+  };
+  unsigned next = lo + threadIdx.x;
+  auto fetch = [&](Nodes& v) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k, i += kThreads) {
-      t[k] = i;
-      const bool on = i < hi;
-      fo[k] = w.at(i);
-      qv[k] = on ? qs[i] : 0.0;  // q vanishes on the boundary
-      rv[k] = on ? rs[i] : 0.0;
-      zv[k] = on ? z.at(n, s, n3, i, w) : 0.0;
+    for (int k = 0; k < 2; ++k, next += kThreads) {
+      const bool on = next < hi;
+      v.i[k] = next;
+      v.f[k] = w.at(next);
+      v.q[k] = on ? qs[next] : 0.0;  // q vanishes on the boundary
+      v.r[k] = on ? rs[next] : 0.0;
+      v.z[k] = on ? z.raw(n, s, n3, next, w) : 0;
       w.step();
     }
+  };
+  auto use = [&](const Nodes& v) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (t[k] >= hi) break;
-      const double rn = fma(-a, qv[k], rv[k]);
-      rs[t[k]] = rn;
-      if (MIX) f[fo[k]] = (float)rn;
+    for (int k = 0; k < 2; ++k) {
+      if (v.i[k] >= hi) break;
+      const double rn = fma(-a, v.q[k], v.r[k]);
+      rs[v.i[k]] = rn;
+      if (MIX) f[v.f[k]] = (float)rn;
       rr = fma(rn, rn, rr);
-      rz = fma(rn, zv[k], rz);
+      rz = fma(rn, widen(v.z[k]), rz);
     }
+  };
+  Nodes v0, v1;
+  fetch(v0);
+  while (v0.i[0] < hi) {
+    fetch(v1);
+    use(v0);
+    if (v1.i[0] >= hi) break;
+    fetch(v0);
+    use(v1);
   }
   const double b1 = block_sum<kThreads>(rr);
   const double b2 = block_sum<kThreads>(rz);
