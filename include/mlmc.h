@@ -203,8 +203,8 @@ typedef struct {
  * one grid. Writes k = exp(log k) into k_out (device, batch * n^3 elements of type
  * `dtype`: MLMC_F64, or MLMC_F32 = the FP64 value rounded to FP32). The phase is
  * always evaluated in FP64; the sum over the M features runs as exact products of bf16
- * slices of the phasors on the tensor cores (tcgen05 from n = 65, the warp-level MMA
- * below; grids with n - 1 a multiple of 16, others in double-float), within ~1e-13 of the
+ * slices of the phasors on the tensor cores (tcgen05; grids with n - 1 a multiple of
+ * 16, others in double-float), within ~1e-13 of the
  * FP64 sum relative in k. sample_ids_host is host memory, read before return.
  * Errors: MLMC_ERR_INVALID for n not 2^p+1 (5 <= n <= 4097), batch < 1, M < 1,
  * ell <= 0, sigma2 < 0, unknown cov or dtype, or NULL pointers; MLMC_ERR_OOM / _CUDA;
@@ -294,7 +294,7 @@ typedef struct {
   double mean;             /* Y-hat_l = (1/N) sum Y */
   double var_biased;       /* s_l^2 with 1/N (Sec. 2.3) */
   double var_unbiased;     /* with 1/(N-1) (0 for N < 2) */
-  double sum;              /* Kahan-compensated sum of Y */
+  double sum;              /* compensated sum of Y */
   double sum_comp;         /* its compensation term */
   double M2;               /* sum (Y - mean)^2 (Welford / Chan) */
   double mean_cycles_fine; /* mean V-cycles of the fine solve */
@@ -593,7 +593,7 @@ int mlmc_tune_set(int n, int precision, int smoother, int nu);
  * default). MLMC_ERR_INVALID for after < -1. Host-only.
  *
  * mlmc_inject_wait_failure -- host-side fault injection for the tensor-core field (the
- * tcgen05 volume kernel, grids from 65^3): each of the next `launches` launches of that
+ * tcgen05 kernel, grids from 17^3): each of the next `launches` launches of that
  * kernel also waits, in its issuing thread, on an mbarrier that nothing arrives on, so the
  * wait runs out after the wait budget (mlmc_set_wait_budget); the blocks then drain their
  * copies and products, write NaN to their nodes, free their tensor memory and return, and

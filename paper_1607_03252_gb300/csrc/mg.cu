@@ -1943,8 +1943,7 @@ __global__ void __launch_bounds__(kThreads, 4)
   double* rs = r + (size_t)s * n3;
   // Two nodes a thread at a time, the next two loaded before these are computed: with four loaded
   // together every warp of the SM waited for memory at once and then queued at the FP64 pipe at once
-  // (257^3 x 1: 152 -> 143 us a
-  // launch, x 2: 163 -> 149; its three FP64 operations a node take 96 of them).
+  // (257^3 x 1: 152 -> 143 us a launch, x 2: 163 -> 149; the FP64 operations alone take 96 at x 1).
   struct Nodes {
     double q[2], r[2];
     typename PrecondZ<MIX, SPLIT>::Raw z[2];
