@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(UmShape<N>::threads, UmShape<N>::BPS)
       fold(true);
     }
   } else if (lane == 0) {
-    int last_copy = -1, last_commit = -1;
+    int last_copy = -1, last_commit = -1, last_acc = -1;
     auto issue_copy = [&](int c) {  // the bulk copy of k-step c's x-slices into its stage
       mbar_arrive_expect_tx(&bfull[c % NS], (unsigned)S::b_stage);
       bulk_g2s(sm + (size_t)(c % NS) * S::stage + S::a_stage, xu + (size_t)c * S::b_stage, (unsigned)S::b_stage,
@@ -1077,7 +1077,10 @@ __global__ void __launch_bounds__(UmShape<N>::threads, UmShape<N>::BPS)
         }
       umma::commit(&empty[st]);
       last_commit = ks;
-      if (MULTI && (ks + 1) % kFoldSteps == 0 && ks + 1 < KS) umma::commit(accf);
+      if (MULTI && (ks + 1) % kFoldSteps == 0 && ks + 1 < KS) {
+        umma::commit(accf);
+        ++last_acc;
+      }
       // the stage of k-step ks - 1 gets its next x-slices once its products are done
       if (ks >= 1 && ks - 1 + NS < KS) {
         if (!wait(&empty[(ks - 1) % NS], (ks - 1) / NS, budget)) break;
@@ -1086,12 +1089,16 @@ __global__ void __launch_bounds__(UmShape<N>::threads, UmShape<N>::BPS)
     }
     if (!bad) {
       umma::commit(accf);
-    } else {
-      // drain: the last issued products and copies land before the block leaves
-      if (last_commit >= 0) mbar_wait_bounded(&empty[last_commit % NS], (unsigned)((last_commit / NS) & 1), kDrainBudget);
-      for (int c = max(0, last_copy - NS + 1); c <= last_copy; ++c)
-        mbar_wait_bounded(&bfull[c % NS], (unsigned)((c / NS) & 1), kDrainBudget);
+      ++last_acc;
     }
+    // Drain: the products issued, their arrivals and the copies land before the block frees its
+    // tensor memory and leaves, whichever thread gave up: the staging warps may have, on a wait of
+    // theirs, while this one's all ended well (nothing is left to wait for then unless they did).
+    for (int c = max(0, last_commit - NS + 1); c <= last_commit; ++c)
+      mbar_wait_bounded(&empty[c % NS], (unsigned)((c / NS) & 1), kDrainBudget);
+    if (last_acc >= 0) mbar_wait_bounded(accf, (unsigned)(last_acc & 1), kDrainBudget);
+    for (int c = max(0, last_copy - NS + 1); c <= last_copy; ++c)
+      mbar_wait_bounded(&bfull[c % NS], (unsigned)((c / NS) & 1), kDrainBudget);
   }
   umma::fence_before_sync();
   __syncthreads();
