@@ -17,6 +17,7 @@
 #include "mg.cuh"
 #include "level.cuh"
 #include "spde.cuh"
+#include "optin.cuh"
 #include "prof.cuh"
 #include "tune.cuh"
 
@@ -48,7 +49,6 @@ static std::atomic<long long> g_alloc_budget{-1};
 // beyond that goes back at the next synchronisation, all of it when an allocation fails
 // (DevBuf::alloc) or the device runs low (pool_give_back). Pools are safe with any number of
 // threads and streams. NULL (the default pool is used) where the device offers none.
-constexpr int kMaxDevices = 64;
 static cudaMemPool_t device_pool(int dev) {
   static std::mutex mu;
   static bool made[kMaxDevices] = {};

@@ -32,6 +32,7 @@
 #include "common.cuh"
 #include "divide.cuh"
 #include "mg.cuh"
+#include "optin.cuh"
 #include "prof.cuh"
 #include "smooth.cuh"
 #include "tune.cuh"
@@ -2550,8 +2551,7 @@ cudaError_t tail_launch(const TailArgs<T>& A, int B, int coef0, int coef1, cudaS
   constexpr int N1 = 9;
   const size_t elems = (size_t)TailGrid<T, N0, false>::shared_iter + 250 + (size_t)coef0 * N0 * N0 * N0 +
                        (N0 == 17 ? (size_t)TailGrid<T, N1, false>::shared_iter + (size_t)coef1 * N1 * N1 * N1 : 0);
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_vcycle_tail<T, N0, SPLIT, P1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  const cudaError_t attr = allow_dynamic_smem<k_vcycle_tail<T, N0, SPLIT, P1>>(200 * 1024);
   if (attr != cudaSuccess) return attr;
   k_vcycle_tail<T, N0, SPLIT, P1><<<B, kTailThreads, elems * sizeof(T), st>>>(A);
   return cudaSuccess;
@@ -4338,9 +4338,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     // 0.51 ms, 4096 15.1 against k_solve_cta's 14.3, whose four samples per SM fill the FP64 pipe)
     if (a.n == 17 && nu1 > 0 && nu2 > 0 && !H.nodal[0] && !H.nodal[1] && A.NB == 2 && A.slabs == 1 && (mixed || B <= sms)) {
       const size_t smem = Solve17<T>::elems * sizeof(T);
-      static const cudaError_t attr =
-          cudaFuncSetAttribute(k_solve17<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      MLMC_CUDA_TRY(attr);
+      MLMC_CUDA_TRY(allow_dynamic_smem<k_solve17<T>>(smem));
       MLMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve17<T>, kTailThreads, smem));
       const int grid = B < sms * (per_sm > 0 ? per_sm : 1) ? B : sms * (per_sm > 0 ? per_sm : 1);
       MLMC_LAUNCH(prof::sized(sizeof(T) == 4 ? "solve_cta_mixed" : "solve_cta_f64", a.n), 0.0, 0.0, st,
