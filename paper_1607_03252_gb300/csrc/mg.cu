@@ -2140,6 +2140,7 @@ struct Hier {
   bool p1 = false;                // P1 finite elements: P1 transfers instead of FW / trilinear
   bool split = false;             // FP32 hierarchy in colour-split storage (MLMC_SMOOTH_SPLIT)
   bool tail_finest = false;       // the one-launch cycle may start on the finest grid (FMG)
+  cudaError_t failed = cudaSuccess;  // a kernel of the cycle that could not be launched (GraphRunner reports it)
 };
 
 // Lays out the workspace. Level-0 u of FP64 solves is the caller's array (not carved).
@@ -2547,13 +2548,16 @@ inline bool tail_applies(const Hier<T>& H, int j, int nu1, int nu2) {
 }
 
 template <typename T, int N0, bool SPLIT, bool P1>
-cudaError_t tail_launch(const TailArgs<T>& A, int B, int coef0, int coef1, cudaStream_t st) {
+cudaError_t tail_launch(const TailArgs<T>& A, int B, int coef0, int coef1, double nodes, cudaStream_t st) {
   constexpr int N1 = 9;
   const size_t elems = (size_t)TailGrid<T, N0, false>::shared_iter + 250 + (size_t)coef0 * N0 * N0 * N0 +
                        (N0 == 17 ? (size_t)TailGrid<T, N1, false>::shared_iter + (size_t)coef1 * N1 * N1 * N1 : 0);
   const cudaError_t attr = allow_dynamic_smem<k_vcycle_tail<T, N0, SPLIT, P1>>(200 * 1024);
   if (attr != cudaSuccess) return attr;
-  k_vcycle_tail<T, N0, SPLIT, P1><<<B, kTailThreads, elems * sizeof(T), st>>>(A);
+  const int nu = A.nu1 + A.nu2;
+  MLMC_LAUNCH(prof::sized(sizeof(T) == 8 ? "vcycle_tail_f64" : "vcycle_tail_f32", N0),
+              nodes * nu * 7.0 * (double)sizeof(T), nodes * (nu * 13.0 + 14.0), st,
+              (k_vcycle_tail<T, N0, SPLIT, P1><<<B, kTailThreads, elems * sizeof(T), st>>>(A)));
   return cudaSuccess;
 }
 
@@ -2573,22 +2577,21 @@ void vcycle_tail(Hier<T>& H, int j, int nu1, int nu2, cudaStream_t st, bool zero
   A.nu1 = nu1;
   A.nu2 = nu2;
   A.zero = zero ? 1 : 0;
-  const double Ba = (double)H.n_act, nodes = interior(n) * 8.0 / 7.0;
+  const double nodes = (double)H.n_act * interior(n) * 8.0 / 7.0;
   auto go = [&](auto n0) {
     constexpr int N0 = decltype(n0)::value;
     if constexpr (sizeof(T) == 8) {
-      if (H.split && H.p1) return tail_launch<T, N0, true, true>(A, B, 0, 0, st);
-      if (H.split) return tail_launch<T, N0, true, false>(A, B, 0, 0, st);
-      if (H.p1) return tail_launch<T, N0, false, true>(A, B, 0, 0, st);
-      return tail_launch<T, N0, false, false>(A, B, 0, 0, st);
+      if (H.split && H.p1) return tail_launch<T, N0, true, true>(A, B, 0, 0, nodes, st);
+      if (H.split) return tail_launch<T, N0, true, false>(A, B, 0, 0, nodes, st);
+      if (H.p1) return tail_launch<T, N0, false, true>(A, B, 0, 0, nodes, st);
+      return tail_launch<T, N0, false, false>(A, B, 0, 0, nodes, st);
     } else {
-      if (H.split) return tail_launch<T, N0, true, false>(A, B, coef[0], coef[1], st);
-      return tail_launch<T, N0, false, false>(A, B, coef[0], coef[1], st);
+      if (H.split) return tail_launch<T, N0, true, false>(A, B, coef[0], coef[1], nodes, st);
+      return tail_launch<T, N0, false, false>(A, B, coef[0], coef[1], nodes, st);
     }
   };
-  MLMC_LAUNCH(prof::sized(sizeof(T) == 8 ? "vcycle_tail_f64" : "vcycle_tail_f32", n),
-              Ba * nodes * (nu1 + nu2) * 7.0 * (double)sizeof(T), Ba * nodes * ((nu1 + nu2) * 13.0 + 14.0), st,
-              (n == 17 ? go(std::integral_constant<int, 17>()) : go(std::integral_constant<int, 9>())));
+  const cudaError_t e = n == 17 ? go(std::integral_constant<int, 17>()) : go(std::integral_constant<int, 9>());
+  if (e != cudaSuccess) H.failed = e;
 }
 
 // One level of the V-cycle on colour-split FP32 storage: nodal-coefficient colour passes,
@@ -2913,6 +2916,7 @@ struct GraphRunner {
   int run(Hier<T>& H, int nu1, int nu2, cudaStream_t st, bool zero, int j0 = 0, bool red_done = false) {
     if (!enabled) {
       vcycle<T>(H, j0, nu1, nu2, st, zero, red_done);
+      MLMC_CUDA_TRY(H.failed);
       return MLMC_OK;
     }
     if (!exec) {
@@ -2923,6 +2927,10 @@ struct GraphRunner {
       cap_act = H.n_act > 0 ? H.n_act : 1;
       cudaGraph_t graph = nullptr;
       MLMC_CUDA_TRY(cudaStreamEndCapture(st, &graph));
+      if (H.failed != cudaSuccess) {
+        cudaGraphDestroy(graph);
+        MLMC_CUDA_TRY(H.failed);
+      }
       const cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
       cudaGraphDestroy(graph);
       if (e != cudaSuccess) {
