@@ -20,6 +20,7 @@
 #include "dfloat.cuh"
 #include "field.cuh"
 #include "philox.cuh"
+#include "optin.cuh"
 #include "prof.cuh"
 #include "umma.cuh"
 #include "umma_layout.h"
@@ -720,9 +721,7 @@ template <typename TOut, int RX, bool FACE>
 int field_tc_launch(const float4* xsplit, const float4* pt, const uint4* Xf, const float* e2tab, int M, int n, int KS,
                     int B, double scale, void* kout, double bytes, double flops, cudaStream_t st, double share) {
   const size_t smem = TcShape<RX>::smem;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_field_tc<TOut, RX, FACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  MLMC_CUDA_TRY(attr);
+  MLMC_CUDA_TRY((allow_dynamic_smem<k_field_tc<TOut, RX, FACE>>(smem)));
   // line groups of 32 lines, ceil(lines / 32) per sample, 8 / RX per block; samples in
   // chunks that keep the grid's y-extent within 65535
   const size_t nl = FACE ? (size_t)n : (size_t)n * n;
@@ -788,6 +787,19 @@ constexpr int kUmM = 128;
 
 // Set to 1 by a tensor-core field block whose bounded wait ran out (field_wait_error_take).
 __device__ int g_field_wait_err = 0;
+
+// Its address on the device current on the calling thread, looked up once per device (NULL: none).
+static int* field_wait_flag() {
+  static std::atomic<int*> at[kMaxDevices]{};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  if (int* p = known ? at[dev].load() : nullptr) return p;
+  void* p = nullptr;
+  if (cudaGetSymbolAddress(&p, g_field_wait_err) != cudaSuccess) return nullptr;
+  if (known) at[dev].store((int*)p);
+  return (int*)p;
+}
 
 static std::atomic<int> g_inject_wait{0};
 void field_inject_wait_failure(int launches) { g_inject_wait.store(launches); }
@@ -1109,9 +1121,7 @@ template <typename TOut, int N, bool MULTI>
 int field_umma_launch(const float4* xsplit, const unsigned char* XU, const float* e2tab, int M, int n, int KS, int B,
                       double scale, int inject, int* err, TOut* kout, double bytes, double flops, cudaStream_t st) {
   using S = UmShape<N>;
-  static const cudaError_t attr = cudaFuncSetAttribute(k_field_umma<TOut, N, MULTI>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
-  MLMC_CUDA_TRY(attr);
+  MLMC_CUDA_TRY((allow_dynamic_smem<k_field_umma<TOut, N, MULTI>>(S::smem)));
   const size_t tiles = ((size_t)n * n + kUmM - 1) / kUmM + (n + kUmM - 1) / kUmM;
   MLMC_LAUNCH("field_tc", bytes, flops, st,
               (k_field_umma<TOut, N, MULTI><<<dim3((unsigned)((n - 1) / N), (unsigned)tiles, (unsigned)B), S::threads,
@@ -1129,10 +1139,7 @@ int field_umma(const float4* xsplit, const unsigned char* XU, const float* e2tab
       inject = 1;
       break;
     }
-  static int* const err = [] {
-    void* p = nullptr;
-    return cudaGetSymbolAddress(&p, g_field_wait_err) == cudaSuccess ? (int*)p : nullptr;
-  }();
+  int* const err = field_wait_flag();
   if (!err) {
     set_error("field: no address for the wait-error flag");
     return MLMC_ERR_CUDA;

@@ -29,6 +29,7 @@
 // per sweep is one read of each array and one write of u (7 words per node), against
 // 12+ words for two separate colour passes.
 #include "common.cuh"
+#include "optin.cuh"
 #include "prof.cuh"
 #include "smooth.cuh"
 #include "bulk.cuh"
@@ -566,25 +567,19 @@ int launch_shape(int n, int B, const T* Kx, const T* Ky, const T* Kz, const T* D
 
 }  // namespace
 
-// The dynamic shared-memory opt-in of each kernel instance, set once per process (the
-// library drives one device per process). Function-local statics make the first call
-// thread-safe; it happens before any stream capture because solve setup configures
-// every fused level first.
+// The dynamic shared-memory opt-in of each kernel instance, once per device; it happens before
+// any stream capture because solve setup configures every fused level first.
 template <typename T, int BX, int BY>
 int configure_shape() {
   using Lay = FusedLayout<T, BX, BY>;
-  static const cudaError_t e = cudaFuncSetAttribute(k_rbgs_fused<T, BX, BY>,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay::bytes);
-  MLMC_CUDA_TRY(e);
+  MLMC_CUDA_TRY((allow_dynamic_smem<k_rbgs_fused<T, BX, BY>>(Lay::bytes)));
   return MLMC_OK;
 }
 
 template <typename T, int BX, int BY>
 int configure_bulk() {
   using Lay = BulkLayout<T, BX, BY>;
-  static const cudaError_t e = cudaFuncSetAttribute(k_rbgs_bulk<T, BX, BY>,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay::bytes);
-  MLMC_CUDA_TRY(e);
+  MLMC_CUDA_TRY((allow_dynamic_smem<k_rbgs_bulk<T, BX, BY>>(Lay::bytes)));
   return MLMC_OK;
 }
 

@@ -1,7 +1,9 @@
 """A kernel's dynamic shared-memory limit belongs to the device it was raised on: csrc/optin.cuh,
 built with g++ against a fake runtime, raises it once per kernel and device and reports a failure
-on every call, and the solver's kernels take their limit from there and from nowhere else."""
+on every call, and every kernel takes its limit from there and from nowhere else. A device symbol's
+address belongs to its device too: the field's error flag is looked up for each."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -35,6 +37,9 @@ def test_limit_is_per_device_and_failures_are_reported(tmp_path):
     assert res.returncode == 0, res.stdout
 
 
-@pytest.mark.parametrize("name", ["mg.cu"])
+@pytest.mark.parametrize("name", ["mg.cu", "field.cu", "smooth.cu"])
 def test_no_kernel_raises_its_limit_once_per_process(name):
-    assert "cudaFuncSetAttribute" not in open(os.path.join(CSRC, name)).read()
+    text = open(os.path.join(CSRC, name)).read()
+    assert "cudaFuncSetAttribute" not in text
+    for found in re.finditer("cudaGetSymbolAddress", text):  # not in a static's initialiser
+        assert "static int* const" not in text[max(0, found.start() - 160):found.start()]
