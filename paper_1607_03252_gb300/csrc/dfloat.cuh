@@ -60,26 +60,19 @@ MLMC_DF_HD void add(float ah, float al, float bh, float bl, float& sh, float& sl
   e = add(e, add(al, bl));
   fast_two_sum(s, e, sh, sl);
 }
-// (rh + rl) + i (ih + il) = (arh + arl + i (aih + ail)) (brh + brl + i (bih + bil)) for moduli of
-// about 1: the four leading products exactly (product and FMA remainder), their sum exactly, the
-// cross terms and remainders in one FP32 sum, renormalised once; absolute error below 2^-46.
-MLMC_DF_HD void cmul_part(float p1h, float p1l, float q1h, float q1l, float p2h, float p2l, float q2h, float q2l,
-                          float& h, float& l) {  // p1 q1 + p2 q2
-  const float a = mul(p1h, q1h), ae = fma(p1h, q1h, -a);
-  const float b = mul(p2h, q2h), be = fma(p2h, q2h, -b);
-  float s, e;
-  two_sum(a, b, s, e);
-  e = add(e, add(ae, be));
-  e = fma(p1h, q1l, e);
-  e = fma(p1l, q1h, e);
-  e = fma(p2h, q2l, e);
-  e = fma(p2l, q2h, e);
-  fast_two_sum(s, e, h, l);
-}
+// (rh + rl) + i (ih + il) = (arh + arl + i (aih + ail)) (brh + brl + i (bih + bil)): the four
+// products and the two sums in double-float, each renormalised. Over random pairs of phasors the
+// error is 1.2e-15 rms and below 1e-14; with one renormalisation for each part, 38 operations
+// instead of 50, it is 1.6e-15 and up to 1.9e-14.
 MLMC_DF_HD void cmul(float arh, float arl, float aih, float ail, float brh, float brl, float bih, float bil, float& rh,
                      float& rl, float& ih, float& il) {
-  cmul_part(arh, arl, brh, brl, -aih, -ail, bih, bil, rh, rl);
-  cmul_part(arh, arl, bih, bil, aih, ail, brh, brl, ih, il);
+  float t1h, t1l, t2h, t2l;
+  mul(arh, arl, brh, brl, t1h, t1l);
+  mul(aih, ail, bih, bil, t2h, t2l);
+  add(t1h, t1l, -t2h, -t2l, rh, rl);
+  mul(arh, arl, bih, bil, t1h, t1l);
+  mul(aih, ail, brh, brl, t2h, t2l);
+  add(t1h, t1l, t2h, t2l, ih, il);
 }
 
 // Seven slices of v = h + l (|v| <= 1 + 2^-20, |l| <= ulp(h)): t[i] is an integer multiple of
