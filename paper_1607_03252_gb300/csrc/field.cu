@@ -70,9 +70,10 @@ __global__ void k_features(const uint64_t* __restrict__ ids, int B, int M, uint6
 
 // Phasor tables tab[s][axis][m][i] = (cos, sin) of (w_axis x_i (+ b_m on axis 0)), and
 // the same pre-split for the double-float sums, xs = (Re hi, Re lo, Im hi, Im lo). A row (one
-// sample, axis and feature) is cut into runs of kPhRun entries (the last takes the row's remainder:
-// nine on every grid from n = 9); a run's first entry is the sincos of its phase, the next ones are
-// products with the step e^{i w h} (over a run the products add a few ulps, below 2e-15 relative).
+// sample, axis and feature) is cut into runs of kPhRun entries; a run's first entry is the sincos of
+// its phase, the next ones are products with the step e^{i w h} (over a run the products add a few
+// ulps, below 2e-15 relative). From n = 9 on the last entry, on the faces x, y, z = 1 that every node
+// of a face shares, is a run of its own: as the ninth of a run its error was ten times that of a sincos.
 // A thread fills `group` consecutive runs of a row with one sincos of the step between them. The
 // FP64 pipe bounds it (one sincos is worth about 40 operations, a product 4); the split runs on the
 // integer pipe. `all` = false leaves out the entries of tab that the tensor-core form does not read
@@ -80,7 +81,7 @@ __global__ void k_features(const uint64_t* __restrict__ ids, int B, int M, uint6
 // third of the bytes. 17^3 x 4096: 1.78 ms with a step sincos per run, FP64 splits and runs of 8, 8
 // and 1, 0.88 now; 33^3 x 103 72 -> 45 us.
 constexpr int kPhRun = 8;
-__device__ __forceinline__ int phasor_runs(int n) { return n > 2 * kPhRun ? (n - 1) / kPhRun : 1; }
+__host__ __device__ __forceinline__ int phasor_runs(int n) { return (n + kPhRun - 1) / kPhRun; }
 __global__ void k_phasors(const double* __restrict__ w, const double* __restrict__ bph, int B, int M, int n,
                           double h, double2* __restrict__ tab, float4* __restrict__ xs, int group = 1,
                           bool all = true) {
@@ -98,7 +99,7 @@ __global__ void k_phasors(const double* __restrict__ w, const double* __restrict
     double ds, dc;
     sincos(wa * h, &ds, &dc);
     for (int run = run0; run < run1; ++run) {
-      const int i0 = run * kPhRun, i1 = run == runs - 1 ? n : i0 + kPhRun;
+      const int i0 = run * kPhRun, i1 = i0 + kPhRun < n ? i0 + kPhRun : n;
       double ph = wa * ((double)i0 * h);
       if (axis == 0) ph += bph[f];
       double sn, cs;
@@ -1252,7 +1253,7 @@ int field_eval_dev(const mlmc_field_cfg& cfg, const uint64_t* ids_dev, int B, in
   const size_t nt = (size_t)B * 3 * cfg.M * n;
   // runs per thread: as many as leave two warps for each quarter of an SM, which fill its FP64 pipe
   const bool tc = (arith == kFieldTC || arith == kFieldTCWarp) && tc_applies(n);
-  const int runs = n > 2 * kPhRun ? (n - 1) / kPhRun : 1;
+  const int runs = phasor_runs(n);
   const size_t rows = (size_t)B * 3 * cfg.M;
   int group = (int)(rows * runs / (152u * 4 * 2 * 32));
   group = group < 1 ? 1 : (group > runs ? runs : group);
