@@ -47,6 +47,12 @@
  *   - Calls that say "blocking" synchronise `stream` before returning; the others only
  *     enqueue work, except where host-side outputs are requested.
  *   - Only one GPU is used: the device current on the calling thread.
+ *   - Calls take their workspaces from a memory pool of the library, one per device, and give
+ *     them back to it. Up to a sixteenth of the device's memory stays in the pool between calls
+ *     (it is reused by the next call instead of being mapped again); what is beyond that goes
+ *     back to the system when the stream next synchronises, all of it when one of the library's own
+ *     allocations fails. Another allocator of the process cannot take what the pool keeps:
+ *     mlmc_release_memory gives it back. The pool does not survive cudaDeviceReset.
  *   - There is no CPU fallback: without a usable CUDA device every compute call
  *     returns MLMC_ERR_CUDA.
  */
@@ -603,6 +609,15 @@ int mlmc_tune_set(int n, int precision, int smoother, int nu);
 int mlmc_set_wait_budget(int64_t clocks, int64_t* previous);
 int mlmc_inject_alloc_failure(int64_t after);
 int mlmc_inject_wait_failure(int launches);
+
+/*
+ * mlmc_release_memory -- gives the memory that the library keeps between calls on the current
+ * device (see the conventions above) back to the system; what running calls use stays with them.
+ * The next call maps its workspace again. For programs whose own allocator needs the memory.
+ * No counterpart in the paper. Blocking: waits for the work on the device (the caller's own
+ * streams must not be in capture). Thread-safe. Errors: MLMC_ERR_CUDA.
+ */
+int mlmc_release_memory(void);
 
 /* Text of the last error on the calling thread ("" if none). Never NULL. */
 const char* mlmc_last_error_string(void);

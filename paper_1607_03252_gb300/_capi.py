@@ -207,6 +207,7 @@ SIGNATURES = {
     "mlmc_set_wait_budget": (ctypes.c_int, [ctypes.c_int64, ctypes.POINTER(ctypes.c_int64)]),
     "mlmc_inject_alloc_failure": (ctypes.c_int, [ctypes.c_int64]),
     "mlmc_inject_wait_failure": (ctypes.c_int, [ctypes.c_int]),
+    "mlmc_release_memory": (ctypes.c_int, []),
     "mlmc_tune_set": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "mlmc_autotune": (ctypes.c_int, [ctypes.POINTER(MlmcCfg), ctypes.c_int, ctypes.c_uint64, ctypes.c_int,
                                      ctypes.POINTER(TuneEntry), ctypes.c_int, ctypes.POINTER(ctypes.c_int),
@@ -461,6 +462,11 @@ def inject_wait_failure(launches: int):
     """The next `launches` launches of the tcgen05 field kernel wait on an mbarrier that
     nothing arrives on, so the wait runs out after the wait budget (0: off)."""
     _check(lib().mlmc_inject_wait_failure(int(launches)), "mlmc_inject_wait_failure")
+
+
+def release_memory():
+    """Gives the memory the library keeps between calls on the current device back to the system."""
+    _check(lib().mlmc_release_memory(), "mlmc_release_memory")
 
 
 def make_mlmc_cfg(run_seed, sigma2, ell, M, n0=17, nu1=2, nu2=2, rtol=1e-10, max_cycles=100,

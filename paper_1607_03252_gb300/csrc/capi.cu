@@ -9,6 +9,7 @@
 #include <atomic>
 #include <chrono>
 #include <mutex>
+#include <shared_mutex>
 #include <utility>
 #include <vector>
 
@@ -38,6 +39,11 @@ const char* last_error() { return g_err; }
 static std::atomic<long long> g_wait_budget{2000000000LL};
 long long wait_budget_clocks() { return g_wait_budget.load(); }
 
+std::shared_mutex& capture_lock() {
+  static std::shared_mutex mu;
+  return mu;
+}
+
 // Host-side allocation-failure injection (mlmc_inject_alloc_failure): -1 = off, else the
 // number of further allocations that still succeed before every later one fails.
 static std::atomic<long long> g_alloc_budget{-1};
@@ -47,7 +53,8 @@ static std::atomic<long long> g_alloc_budget{-1};
 // of a blocking API mapped its workspace again (a 65^3 field alone 0.3 ms of 1.2, a level of 5 GB 6
 // ms of 29). This one keeps up to a sixteenth of the device's memory between calls; what is freed
 // beyond that goes back at the next synchronisation, all of it when an allocation fails
-// (DevBuf::alloc) or the device runs low (pool_give_back). Pools are safe with any number of
+// (DevBuf::alloc), the device runs low (pool_give_back) or the caller asks for it
+// (mlmc_release_memory). Pools are safe with any number of
 // threads and streams. NULL (the default pool is used) where the device offers none.
 static cudaMemPool_t device_pool(int dev) {
   static std::mutex mu;
@@ -608,6 +615,17 @@ static int field_eval_impl(const mlmc_field_cfg* cfg, const uint64_t* sample_ids
               "nodes of the blocks concerned hold NaN",
               wait_budget_clocks());
     return MLMC_ERR_TIMEOUT;
+  }
+  return MLMC_OK;
+}
+
+int mlmc_release_memory(void) {
+  MLMC_TRY(device_ready());
+  if (cudaMemPool_t p = current_pool()) {
+    // what earlier calls freed last counts as unused once the device has passed it
+    std::unique_lock<std::shared_mutex> lk(capture_lock());
+    MLMC_CUDA_TRY(cudaDeviceSynchronize());
+    MLMC_CUDA_TRY(cudaMemPoolTrimTo(p, 0));
   }
   return MLMC_OK;
 }

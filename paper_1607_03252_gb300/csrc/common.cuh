@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <shared_mutex>
 #include <string>
 
 #include "mlmc.h"
@@ -17,6 +18,10 @@ const char* last_error();
 // Budget, in SM clocks, of every bounded wait inside a kernel (mlmc_set_wait_budget;
 // about one second by default).
 long long wait_budget_clocks();
+
+// Held shared while a stream of the library is being captured: a device may not be synchronised then
+// (mlmc_release_memory takes it exclusively).
+std::shared_mutex& capture_lock();
 
 #define MLMC_CUDA_TRY(expr)                                                                 \
   do {                                                                                      \

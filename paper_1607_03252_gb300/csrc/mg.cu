@@ -26,6 +26,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 
+#include <shared_mutex>
 #include <type_traits>
 #include <vector>
 
@@ -2920,6 +2921,7 @@ struct GraphRunner {
       return MLMC_OK;
     }
     if (!exec) {
+      std::shared_lock<std::shared_mutex> lk(capture_lock());
       MLMC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       prof::tape_begin();
       vcycle<T>(H, j0, nu1, nu2, st, zero, red_done);

@@ -3,6 +3,7 @@
 // dynamic shared memory: every cycle has to report it, launched directly or captured.
 #include <cstddef>
 #include <cstdio>
+#include <shared_mutex>
 #include <type_traits>
 #include <vector>
 
@@ -33,6 +34,10 @@ static void set_error(const char*, ...) {}
     (void)(cls), (void)(bytes), (void)(flops), (void)(st); \
     launch_expr;                                        \
   } while (0)
+static std::shared_mutex& capture_lock() {
+  static std::shared_mutex mu;
+  return mu;
+}
 namespace prof {
 struct Tape {};
 static void tape_begin() {}
