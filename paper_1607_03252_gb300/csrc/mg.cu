@@ -4046,9 +4046,11 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     resolve_tuning(a.n, a.cfg.precision, &sm0, &nu1, &nu2);
     // FP32 correction cycles on finite volumes (mixed), or FP64 stationary and FMG cycles
     // on finite volumes or P1 elements (the split kernels are instantiated for n = 5 .. 1025)
-    // (not the 5^3 grid alone: it keeps the plain faces of its dense solve, nothing to sweep)
+    // (not the 5^3 grid alone: it keeps the plain faces of its dense solve, nothing to sweep; not an
+    // FP32 cycle without post-smoothing of more samples than half a launch's z extent, which its
+    // interpolation to both colours takes twice over: the plain storage gives the same iterates)
     H.split = !use_cta && sm0 == MLMC_SMOOTH_SPLIT && a.n <= 1025 && a.n > 5 &&
-              (mixed ? a.cfg.disc == MLMC_DISC_FV : !cg);
+              (mixed ? a.cfg.disc == MLMC_DISC_FV && (nu2 > 0 || a.B <= 32767) : !cg);
   }
   // operators of every level (k injected from k0); colour-split grids need no faces
   // except on the coarsest grid (its dense solve)
