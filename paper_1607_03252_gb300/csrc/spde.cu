@@ -114,7 +114,8 @@ __global__ void k_spde_noise(const uint64_t* __restrict__ ids, int B, int lc, in
 
 // One colour of red-black Gauss-Seidel (red: x + y + z even), one cell per thread: the plain form
 // of k_cc_rbgs4's pass, as are k_cc_restrict and k_cc_prolong of the restriction and interpolation
-// below (the cycle runs the row forms; these state the cycle in full and are what host runs use):
+// and k_cc_coarse of the exact solve below. The library launches the row forms and k_cc_tail; these
+// state the cycle in full, and the host tests compare the others with them:
 // Z_p = (g_p + sum of the neighbours inside the box) / (c h^2 + n_p), with the four
 // possible reciprocals of the diagonal precomputed.
 // Grid (colour cells / blockDim, samples), C = 2^lc >= 4.
