@@ -111,7 +111,10 @@ typedef struct {
   int cov;           /* MLMC_COV_GAUSS or MLMC_COV_EXP */
 } mlmc_field_cfg;
 
-/* Smoother implementations (all compute the same red-black sweep, bit for bit). */
+/* Smoother implementations. All compute the same red-black sweep, in FP64 bit for bit. In FP32
+ * correction cycles MLMC_SMOOTH_NODAL and MLMC_SMOOTH_SPLIT, and with it the default from 33^3,
+ * form the faces anew, within a few ulps of the stored ones of the others: the FP64 outer residual
+ * fixes the solution, which is as far from the exact one after as many cycles. */
 #define MLMC_SMOOTH_AUTO 0      /* the tuned choice for the grid size (mlmc_autotune), else a default:
                                     MLMC_SMOOTH_SPLIT from 33^3 (FP32 correction cycles) or 65^3
                                     (FP64), MLMC_SMOOTH_TWO_PASS below */
@@ -171,12 +174,14 @@ typedef struct {
 
 /* Execution engine of a solve (no counterpart in the paper; same results bit for bit).
  * MLMC_ENGINE_BATCHED: every phase of the cycle is a kernel over the whole batch (the cycle
- * below the finest grid, from 17^3 down, is one), one convergence test per cycle on the host. MLMC_ENGINE_CTA (finite volumes, stationary
- * cycles, refinement or CG, grids up to 33^3; otherwise the batched engine runs): one
- * persistent launch for the whole solve, each CTA taking the next sample from a device
- * counter and running all of its cycles, the convergence tests and the CG recurrences
- * with block barriers; the sums follow the batched kernels' partitions and trees, so
- * iterates, cycle counts and residuals are identical. MLMC_ENGINE_AUTO: the CTA engine
+ * below the finest grid, from 17^3 down, is one), one convergence test per cycle on the host.
+ * MLMC_ENGINE_CTA (finite volumes, stationary cycles, refinement or CG, grids up to 33^3;
+ * otherwise the batched engine runs): one persistent launch for the whole solve, each CTA
+ * taking the next sample from a device counter and running all of its cycles, the convergence
+ * tests and the CG recurrences with block barriers; the sums follow the batched kernels'
+ * partitions and trees, so iterates and residuals are identical, and so are cycle counts (FP64
+ * stationary cycles: unless rounding of the red residuals decides a convergence test, which
+ * differs between the storages; not seen so far). MLMC_ENGINE_AUTO: the CTA engine
  * for grids up to 17^3 (where the batched engine waits on launches and host round trips)
  * and for 33^3 grids in batches of at least 1024 samples, the batched engine otherwise;
  * the environment variable MLMC_ENGINE=1 or 2 overrides the automatic choice. */

@@ -493,7 +493,7 @@ __global__ void k_face_factors(const float4* __restrict__ xsplit, int B, int M, 
   }
 }
 
-// The edge x = y = n - 1 in FP64 (n nodes per sample): one warp per sample and ZC values of z,
+// The edge x = y = n - 1 in FP64 (n nodes per sample): one warp per sample and kEdgeZ values of z,
 // lanes over the features, log k / scale = sum_m Re(X_m[n - 1] Y_m[n - 1] Z_m[z]) with the product
 // of the first two formed once for the warp's z, a butterfly sum over the lanes. Bound by the FP64
 // pipe for many samples (there six z per warp share the product: 17^3 x 4096 282 -> 196 us), by the

@@ -1065,10 +1065,17 @@ __global__ void k_norm_update(int B, int NB, const double* __restrict__ partial,
 
 // What the red residuals' norm has to exceed for a sample to go on without the full test. Formed
 // in the full residual's order of operations (fused = false) they can differ from their part of it
-// by the order of the sum alone. Formed along with a red pass (fused) each differs by rounding too:
-// about 2^-55 (n - 1)^2 of |g| for a coefficient of order one, at most a sixteenth of the tolerances
-// that red_fused takes, so an eighth on top leaves the answer to the full test wherever rounding
-// could change it, and below those tolerances every test is a full one.
+// by the order of the sum alone, so the full test's answer is certain. Formed along with a red pass
+// (fused) each is the same eight terms rounded in another order. The two roundings differ by a few
+// ulps of the largest term, D u, which grows with (n - 1)^2 and with the contrast of the coefficient:
+// about 2^-55 (n - 1)^2 of |g| for one of order one, a sixteenth of the smallest tolerance red_fused
+// takes. The eighth on top covers that, not every contrast: on a rough coefficient, within rounding
+// of its tolerance, a sample could in principle go on for a cycle that the full test would have
+// stopped (never stop early: the full test decides that). It has not been seen: the full residual
+// carries the same rounding at the red nodes and the sweep's own at the black ones, so it is the
+// larger of the two there (2196 tolerances at and just above the residual of a cycle, variances 1 to
+// 9 on grids of 9^3 to 65^3: every solve stopped where the full test stops it). Below those
+// tolerances every test is a full one.
 __host__ __device__ inline double red_limit(double rtol, bool fused) { return rtol * (fused ? 1.125 : 1.0 + 1e-9); }
 inline bool red_fused(double rtol, int n) { return rtol >= 0x1p-51 * (n - 1) * (n - 1); }
 
@@ -2962,7 +2969,7 @@ struct CgVectors {
   double all() const { return (double)H.n_act * H.lv[0].n3; }
   dim3 planes() const { return plane_grid(n() * n(), (long long)H.B * n()); }
   void update() const {
-    MLMC_LAUNCH("cg_update", all() * (MIX ? 32.0 : 32.0), all() * 6.0, st,
+    MLMC_LAUNCH("cg_update", all() * 32.0, all() * 6.0, st,
                 (k_cg_update<MIX, SPLIT><<<dim3(H.NBu, H.B), kThreads, 0, st>>>(
                     n(), H.alpha, H.Q, H.R, PrecondZ<MIX, SPLIT>{z()}, MIX ? (float*)(void*)H.lv[0].g : nullptr,
                     H.partial, H.part2, H.rzo, H.g2, H.relres, H.cycles, H.active, H.cand, rtol, maxc, H.n_active,
@@ -4229,8 +4236,8 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
   };
   // Convergence test after `inc` cycles; returns the samples that go on. After an FP64 cycle
   // that ends on a black pass the red residuals decide for the samples that go on (half the FP64
-  // work), the full residual for those that seem done, so cycle counts and reported residuals
-  // are those of a full test every cycle. On colour-split storage the red residuals come with the
+  // work), the full residual for those that seem done, so reported residuals are those of a full
+  // test, and so are cycle counts (red_limit says how far that holds). On colour-split storage the red residuals come with the
   // next cycle's first red pass. A 129^3 / 65^3 level of 24 samples: 75.6 ms with full tests, 66.0
   // on the red residuals; later 54.8 -> 52.5 with the pass and its test in one (6.3 ms of tests,
   // 3.3 of them the pass); 65^3 x 19 6.72 -> 6.47.
@@ -4256,7 +4263,7 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
       const int slots = fused ? (a.n - 2) * split_groups(a.n, 4) : (a.n - 2) * ((a.n - 1) / 2);
       const dim3 rr((unsigned)((slots + 127) / 128), rz.y, (unsigned)B);
       const int NBr = (int)(rr.x * rr.y);
-      if (H.split && !fused) {  // no pre-smoothing: the full residual
+      if (H.split && !fused) {  // no pre-smoothing, or a tolerance below red_fused's: the full residual
         full_check(inc, nullptr, H.n_act);
         MLMC_CUDA_TRY(cudaMemcpyAsync(na, H.n_active, sizeof(na), cudaMemcpyDeviceToHost, st));
         MLMC_CUDA_TRY(cudaStreamSynchronize(st));
