@@ -9,7 +9,8 @@ Default workload (--config c2): 4-level FP64 MLMC, levels 17^3, 33^3, 65^3, 129^
 (fine grids), N_l = 4096, 1024, 256, 64, sigma^2 = 1, ell = 0.3, M = 256, V(2,2) to
 relative residual 1e-10, f = 1, QoI = mean of u over [0.25, 0.75]^3.
 
-Reported (one JSON line on rank 0):
+Reported (one JSON line on rank 0, below 1500 characters; the record with every table, plan and
+sub-record goes to standard error and, with --detail, to a file):
   value          MLMC samples/s over all levels (sum_l N_l per step x ranks / time),
                  ids already in HBM, outputs left in HBM (device-resident C-ABI call);
   per_level      samples/s per level;
@@ -109,9 +110,10 @@ def parse():
     p.add_argument("--no-extras", action="store_true",
                    help="c2: skip the c3 / c5 / c4 sub-records of the default line")
     p.add_argument("--lanes", type=int, default=4, help="concurrent level streams (1: levels in sequence)")
+    p.add_argument("--detail", default=None, help="file for the whole record (tables, plans, sub-records)")
     p.add_argument("--plan-from", default=None,
-                   help="reuse the autotuned choices (and pilot-sized N_l) of an earlier JSON line of the same "
-                        "config instead of measuring them again (for runs under a profiler)")
+                   help="reuse the autotuned choices (and pilot-sized N_l) of an earlier record of the same "
+                        "config (--detail) instead of measuring them again (for runs under a profiler)")
     return p.parse_args()
 
 
@@ -165,7 +167,7 @@ def plan_levels(mg, cfg, levels, stream, rank):
 
 
 def restore_plan(mg, cfg, levels, N, path):
-    """The plan of an earlier run of the same config (its JSON line): each level's tuned
+    """The plan of an earlier run of the same config (its --detail record): each level's tuned
     smoother and nu go back into the library's tuning table (mlmc_tune_set, for the
     level's fine grid and precision), and pilot-sized workloads take its N_l."""
     with open(path) as fh:
@@ -335,6 +337,39 @@ def reference_arm(args):
 # --------------------------------------------------------------------------------------
 # Own arm
 # --------------------------------------------------------------------------------------
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "gpu_launches")
+LINE_PARTS = {"config": ("workload", "levels", "N_per_gpu", "fine_n", "sigma2", "ell", "M", "rtol", "cycle", "parallelism",
+                         "l2"),
+              "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+              "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+              "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac"),
+              "cpu_baseline": ("value", "unit", "cores")}
+
+
+def headline(record):
+    """The result line of a record: the contract's keys, short parts of the others and the
+    sub-records' values."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    for part, keys in LINE_PARTS.items():
+        if record.get(part):
+            line[part] = {k: record[part][k] for k in keys if k in record[part]}
+    subs = {k: record[k]["value"] for k in ("c3", "c4", "c5", "c6") if record.get(k)}
+    if subs:
+        line["sub_values"] = subs
+    return line
+
+
+def report(record, detail):
+    """The whole record to standard error and to the file `detail` (if any), its short form as the
+    one line on standard output."""
+    print(json.dumps(record), file=sys.stderr, flush=True)
+    if detail:
+        with open(detail, "w") as fh:
+            fh.write(json.dumps(record) + "\n")
+    print(json.dumps(headline(record)), flush=True)
+
+
 def own_arm(args):
     import torch
 
@@ -355,7 +390,7 @@ def own_arm(args):
         line["c6"] = measure(args, "c6", full=False)
         line["extras_wall_s"] = time.perf_counter() - t0
     if line is not None:
-        print(json.dumps(line), flush=True)
+        report(line, args.detail)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
@@ -912,8 +947,7 @@ def serving_arm(args):
     N, plan = plan_levels(mg, CONFIGS["c3"], levels, stream, 0)  # autotunes every level, pilot, Eq. 11
     probs = np.array([n * c for n, c in zip(N, plan["pilot_cost_s"])])
     probs = probs / probs.sum()
-    line = serving_line(mg, probs, levels, cfg, plan, 1200, (0.1, 0.25, 0.5, 0.75, 0.9, 1.0, 1.2), 3000, 3.0)
-    print(json.dumps(line), flush=True)
+    report(serving_line(mg, probs, levels, cfg, plan, 1200, (0.1, 0.25, 0.5, 0.75, 0.9, 1.0, 1.2), 3000, 3.0), args.detail)
     return 0
 
 
@@ -1010,7 +1044,7 @@ def c5_arm(args):
     if rank != 0:
         return 0
     torch.cuda.set_device(local)
-    print(json.dumps(c5_results(args, mg, torch)), flush=True)
+    report(c5_results(args, mg, torch), args.detail)
     return 0
 
 
