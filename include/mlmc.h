@@ -591,8 +591,8 @@ int mlmc_tune_set(int n, int precision, int smoother, int nu);
  *
  * mlmc_set_wait_budget -- every bounded wait inside a kernel (the mbarrier waits of the
  * TMA bulk-copy smoothers and of the tcgen05 field kernel) gives up after `clocks` SM clocks: the kernel then records an
- * error word, waits (bounded by about one second, whatever `clocks` is) for the copies it
- * still has in flight, and returns; the solve reports MLMC_ERR_TIMEOUT and the context
+ * error word, waits (about one second for each at most, whatever `clocks` is) for the copies
+ * and products it still has in flight, and returns; the solve reports MLMC_ERR_TIMEOUT and the context
  * stays usable. Default 2e9 clocks (about one second). clocks = 0 gives up at the first
  * wait that finds its data not yet arrived. Read at each launch (a V-cycle captured as a
  * CUDA graph keeps the budget of its capture). *previous (may be NULL) receives the old

@@ -78,8 +78,8 @@ __global__ void k_features(const uint64_t* __restrict__ ids, int B, int M, uint6
 // FP64 pipe bounds it (one sincos is worth about 40 operations, a product 4); the split runs on the
 // integer pipe. `all` = false leaves out the entries of tab that the tensor-core form does not read
 // (it takes tab only for the edge x = y = n - 1: axis 2 and the last entries of the others), a
-// third of the bytes. 17^3 x 4096: 1.78 ms with a step sincos per run, FP64 splits and runs of 8, 8
-// and 1, 0.88 now; 33^3 x 103 72 -> 45 us.
+// third of the bytes. 17^3 x 4096: 1.78 ms with a step sincos per run and FP64 splits, 1.04 now (0.88
+// with the last entry in the run before it); 33^3 x 103 72 -> 49 us.
 constexpr int kPhRun = 8;
 __host__ __device__ __forceinline__ int phasor_runs(int n) { return (n + kPhRun - 1) / kPhRun; }
 __global__ void k_phasors(const double* __restrict__ w, const double* __restrict__ bph, int B, int M, int n,
@@ -768,7 +768,7 @@ int field_tc_dispatch(const float4* xsplit, const float4* pt, const uint4* Xf, c
 // copy per k-step. The face is further line tiles of the same launch: rows z, factors X_m[n - 1]
 // Z_m[z], the y-phasors' slices for B.
 //
-// The staging (about 190 FP32 and integer instructions per line and feature) is what bounds the
+// The staging (about 200 FP32 and integer instructions per line and feature) is what bounds the
 // kernel, so it must not stop: NS k-steps are in flight, each a stage with two mbarriers. A
 // staging warp waits for the products of the stage's last use (empty), writes its share, and
 // arrives (full); one thread of the last warp waits for full and for the bulk copy, issues the
@@ -776,9 +776,9 @@ int field_tc_dispatch(const float4* xsplit, const float4* pt, const uint4* Xf, c
 // all slices of B that it meets is one product of up to 256 columns (10 per k-step instead of 28
 // of 64 columns, which read A from shared memory 28 times and took 3300 clocks a k-step, more than
 // the staging). Volume and face, 129^3 x 8 (M = 256): 1042 us with a block barrier per two k-steps
-// and 28 products, 818 without the barrier, 631 now; 65^3 x 5 (M = 1024) 747 -> 340. Below 65^3 a
+// and 28 products, 818 without the barrier, 661 now; 65^3 x 5 (M = 1024) 747 -> 354. Below 65^3 a
 // block is small enough for three (N = 16) or two (N = 32) per SM; the warp-level mma.sync form
-// ran there with 8 warps per SM: 17^3 x 4096 6.7 -> 2.5 ms, 33^3 x 103 494 -> 193 us.
+// ran there with 8 warps per SM: 17^3 x 4096 6.7 -> 2.5 ms, 33^3 x 103 494 -> 188 us.
 //
 // Every 256 features (and at the end) the group sums are read from tensor memory and folded into
 // a double-float; the next product overwrites them. Every wait is bounded: a block whose wait

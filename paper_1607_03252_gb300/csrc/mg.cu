@@ -3654,12 +3654,14 @@ __global__ void __launch_bounds__(kCtaThreads) k_solve_cta(CtaArgs<T> A) {
 // ---------------------------------------------------------------------------------
 // The small-grid engine on 17^3 grids: one block of 512 threads per SM with the whole cycle in
 // registers and shared memory. A thread owns up to four nodes of either colour for the whole
-// solve and keeps their six faces in registers; 1/D,
-// iterate, right-hand side and red residuals of 17^3, 9^3 and 5^3 and the 9^3 coefficients are in
-// shared memory (222 KB in FP64). Operations, partitions and trees are k_solve_cta's (which keeps everything in
-// global memory, read through L2 in every pass, and serves 9^3 and 33^3), so results are bit for
-// bit the same. Bound by the chain of passes, one sample per SM. A served request (one mixed CG
-// sample) 1.12 -> 0.57 ms in this kernel, 1.38 -> 0.87 in all.
+// solve and keeps their six faces in registers; 1/D, iterate, right-hand side and red residuals of
+// 17^3, 9^3 and 5^3 and the 9^3 coefficients are in shared memory (183 KB in FP64, 92 KB in FP32).
+// Operations, partitions and trees are k_solve_cta's (which keeps everything in global memory,
+// read through L2 in every pass, and serves 9^3 and 33^3), so results are bit for bit the same.
+// Bound by the chain of passes, one sample per SM. A served request (one mixed CG sample) takes
+// 0.55 ms in this kernel (k_solve_cta 1.12), 0.86 in all. Stored faces only: a form that also took
+// 1/k for the nodal sweep through TailGrid's passes gave wrong iterates as ptxas compiles it by
+// default, right ones with -Xptxas -O1 or with those passes out of line.
 // ---------------------------------------------------------------------------------
 template <typename T>
 struct Solve17 {
@@ -4353,8 +4355,9 @@ int solve_impl(const MGSolveArgs& a, void* ws, cudaStream_t st, int* cycles_host
     MLMC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     MLMC_CUDA_TRY(cudaMemsetAsync(H.n_active, 0, sizeof(int), st));
     // k_solve17 fills an SM with one sample: always the faster form for FP32 cycles (17^3 x 400
-    // mixed: 1.06 against 1.5 ms), for FP64 ones while every SM has at most one sample (one sample
-    // 0.51 ms, 4096 15.1 against k_solve_cta's 14.3, whose four samples per SM fill the FP64 pipe)
+    // mixed refinement: 1.02 ms against 1.57), for FP64 ones while every SM has at most one sample
+    // (one sample 0.51 ms against 0.84; 4096 of them 15.1 against 14.2 when both were measured,
+    // k_solve_cta 11.8 since: its four samples per SM fill the FP64 pipe)
     if (a.n == 17 && nu1 > 0 && nu2 > 0 && !H.nodal[0] && !H.nodal[1] && A.NB == 2 && A.slabs == 1 && (mixed || B <= sms)) {
       const size_t smem = Solve17<T>::elems * sizeof(T);
       MLMC_CUDA_TRY(allow_dynamic_smem<k_solve17<T>>(smem));
