@@ -54,8 +54,8 @@ static std::atomic<long long> g_alloc_budget{-1};
 // ms of 29). This one keeps up to a sixteenth of the device's memory between calls; what is freed
 // beyond that goes back at the next synchronisation, all of it when an allocation fails
 // (DevBuf::alloc), the device runs low (pool_give_back) or the caller asks for it
-// (mlmc_release_memory). Pools are safe with any number of
-// threads and streams. NULL (the default pool is used) where the device offers none.
+// (mlmc_release_memory). Pools are safe with any number of threads and streams. NULL (the default
+// pool is used) where the device offers none.
 static cudaMemPool_t device_pool(int dev) {
   static std::mutex mu;
   static bool made[kMaxDevices] = {};
@@ -239,8 +239,8 @@ struct LevelRecord {
 // Welford's products (one lane each) and adds them to M2: with N samples before and
 // t = N v - (sum + comp), N v as a product and its rounding error, the product of a sample's
 // deviations from the means before and after it is t^2 / (N (N + 1)), never negative, and zero
-// for identical samples. Nothing depends on where a batch or a chunk ends. 4096 samples: 2.55 ms with Kahan's sum,
-// the mean's recurrence and its division in one thread, 0.28 ms now.
+// for identical samples. Nothing depends on where a batch or a chunk ends. 4096 samples: 2.55 ms with
+// Kahan's sum, the mean's recurrence and its division in one thread, 0.28 ms now.
 constexpr int kStatsThreads = 96;
 __global__ void __launch_bounds__(kStatsThreads)
     k_level_stats(const double* __restrict__ Qf, const double* __restrict__ Qc, const int* __restrict__ cf,
@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(kStatsThreads)
         const double N = r.N + (double)i, v = y[q][lane];
         double prod = 0.0;
         if (lane < cnt && N > 0.0) {
-          const double p = N * v, t = (p - s[q][lane]) + (fma(N, v, -p) - c[q][lane]);
+          const double p = __dmul_rn(N, v);  // (rounded: not to be contracted into the difference)
+          const double t = __dadd_rn(__dsub_rn(p, s[q][lane]), __dsub_rn(fma(N, v, -p), c[q][lane]));
           prod = t * (t / (N * (N + 1.0)));
         }
         part[1][lane] = prod;
